@@ -314,6 +314,8 @@ extern "C" int load_code(const tsx_code_desc *desc, void *stream, tsx_code **out
         const int dc = h.kind == TSX_CODE_QC ? h.rdeg[c] : h.c_ptr[c + 1] - h.c_ptr[c];
         if (dc < d.dc_min) d.dc_min = dc;
     }
+    if (h.kind == TSX_CODE_QC)
+        for (int i = 0; i < h.m_b; i++) d.E_odd += h.Z * (h.rdeg[i] | 1);
     d.wstart = std::max(1, girth / 2);
     d.n_rep = n_rep;
     d.rdeg = (const int16_t *)(dev + o_rdeg); d.reoff = (const int32_t *)(dev + o_reoff);
@@ -748,7 +750,7 @@ static int enqueue_decode(tsx_ts_list *L, cudaStream_t s) {
     const tsx_enum_params &p = L->p;
     if (!L->n_dchunks) {
         if (launch_decode(L->code->d, L->dp, L->b, p.warps_per_cta, 0, p.ctas_per_sm, L->grid_sms,
-                          p.kernel == 1 ? 1 : 0, s) != cudaSuccess)
+                          p.kernel == 1 ? 1 : 0, L->n_rec, s) != cudaSuccess)
             return TSX_ECUDA;
         return TSX_OK;
     }
@@ -759,7 +761,7 @@ static int enqueue_decode(tsx_ts_list *L, cudaStream_t s) {
         bk.cand_end = std::min<long long>(bk.cand_begin + L->dchunk, L->range_end);
         bk.queue = L->d_queues + k;
         if (launch_decode(L->code->d, L->dp, bk, p.warps_per_cta, 0, p.ctas_per_sm, L->grid_sms,
-                          p.kernel == 1 ? 1 : 0, s) != cudaSuccess)
+                          p.kernel == 1 ? 1 : 0, bk.cand_end - bk.cand_begin, s) != cudaSuccess)
             return TSX_ECUDA;
     }
     return TSX_OK;

@@ -1,7 +1,7 @@
 // decode.cu -- host side of the decoding and sieve kernels: shared-memory
 // layouts, launch shapes, dispatch, and the compaction of the trapping-set
 // hash table.
-#include "decode_impl.cuh"
+#include "decode_pair.cuh"
 
 namespace tsx {
 
@@ -27,12 +27,14 @@ enum { kLayScalar = 0, kLayPair = 1, kLaySieve = 2, kLayIs = 3, kLayPairVn = 4 }
 int msg_bytes(int decoder) { return decoder == TSX_DEC_NMS_I8 ? 1 : (decoder == TSX_DEC_SPA_F32 ? 4 : 2); }
 int post_bytes(int decoder) { return decoder == TSX_DEC_SPA_F32 ? 4 : 2; }
 
-SlotLayout make_layout(const DevCode &g, int decoder, int kind) {
+// odd_rows: the two-codeword kernels' variant for check degrees above 8 (QC: each row an odd number of words)
+SlotLayout make_layout(const DevCode &g, int decoder, int kind, bool odd_rows) {
     SlotLayout L{};
     L.tables_bytes = al16(tab_offsets(g, kind == kLayPair || kind == kLayIs || kind == kLayPairVn).total);
     const int nw = (g.n + 31) / 32;
     // message slots: QC edges, or the position-major m x dc_max grid of a CSR code
     const int nmsg = g.kind == TSX_CODE_QC ? g.E : g.m * g.dc_max;
+    const int nmsg2 = g.kind == TSX_CODE_QC && odd_rows ? g.E_odd : nmsg;
     int x = 0;
     if (kind == kLayScalar) {
         L.r_off = x; x += al16(nmsg * msg_bytes(decoder));
@@ -42,18 +44,18 @@ SlotLayout make_layout(const DevCode &g, int decoder, int kind) {
     } else if (kind == kLayPair) {
         const int rsz = decoder == TSX_DEC_NMS_I8 ? 2 : 4;
         const int xstride = (nw + 3) & ~3;
-        L.r_off = x; x += al16(nmsg * rsz);
+        L.r_off = x; x += al16(nmsg2 * rsz);
         L.p_off = x; x += al16(2 * g.n * 4);  // current and accumulating posteriors
         L.xa_off = x; x += al16(4 * xstride * 4);
         L.xb_off = L.xa_off;
     } else if (kind == kLayPairVn) {
         const int xstride = (nw + 3) & ~3;
-        L.r_off = x; x += al16(nmsg * 4);
+        L.r_off = x; x += al16(nmsg2 * 4);
         L.p_off = x; x += al16(g.n * 4);  // one posterior buffer, rebuilt by the variable-node pass
         L.xa_off = x; x += al16(4 * xstride * 4);
         L.xb_off = L.xa_off;
     } else if (kind == kLayIs) {
-        L.r_off = x; x += al16(nmsg * 4);
+        L.r_off = x; x += al16(nmsg2 * 4);
         L.p_off = x; x += al16(3 * g.n * 4);  // two posterior buffers and the channel values
         L.xa_off = x; x += al16(nw * 4);      // bitmask of the trapping set
         L.xb_off = L.xa_off;
@@ -65,7 +67,8 @@ SlotLayout make_layout(const DevCode &g, int decoder, int kind) {
         L.xa_off = x; x += al16(nw * 4);
         L.xb_off = L.xa_off;
     }
-    L.misc_off = x; x += al16((int)sizeof(Misc));
+    const bool pair = kind == kLayPair || kind == kLayPairVn;
+    L.misc_off = x; x += al16((int)(pair ? sizeof(PairMisc) : sizeof(Misc)));
     L.slot_bytes = x;
     return L;
 }
@@ -74,41 +77,36 @@ SlotLayout make_layout(const DevCode &g, int decoder, int kind) {
 // batch kernel's staged item)
 constexpr int kSmemCta = 226 * 1024;
 
+// units > 0: how many codeword groups the launch has work for (pairs of
+// candidates), where the host knows it.
 bool plan(const DevCode &g, int decoder, int kind, int G, int groups, int ctas_per_sm, int num_sms,
-          LaunchShape *out, int max_warps = 16) {
+          LaunchShape *out, int max_warps = 16, long long units = 0, bool odd_rows = false) {
     LaunchShape sh{};
-    sh.lay = make_layout(g, decoder, kind);
+    sh.lay = make_layout(g, decoder, kind, odd_rows || g.dc_max > 8);
     const int room = kSmemCta - sh.lay.tables_bytes;
     const int fit = room / sh.lay.slot_bytes;
     if (fit < 1) return false;
     if (kind == kLaySieve) G = 1;
     if (G <= 0) {
-        // as many codeword groups as fit (up to one per warp), the warps shared among them
-        G = max_warps / (fit < max_warps ? fit : max_warps);
-        int work = g.m < g.n ? g.m : g.n;
-        // QC passes run block by block (the variable-node-pass form, and the sampling kernel for
-        // check degree > 8, run all blocks at once)
-        const bool flat = kind == kLayPairVn || (kind == kLayIs && g.dc_max > 8);
-        if (g.kind == TSX_CODE_QC && !flat && g.Z < work) work = g.Z;
-        int gmax = work / 32;
-        if (gmax < 1) gmax = 1;
-        if (G > gmax) G = gmax;
-        if (G > 16) G = 16;
-        if (G < 1) G = 1;
-        if (flat && kind == kLayIs && fit == 1) {
-            // one sample pair per CTA: the width (up to max_warps) with the fewest checks per
-            // thread, the narrowest of those (the pass ends at the group barrier)
-            int best = G, best_rows = (g.m + 32 * G - 1) / (32 * G);
-            for (int w = 8; w <= max_warps && w <= gmax; w++) {
-                const int rows = (g.m + 32 * w - 1) / (32 * w);
-                if (rows < best_rows) {
-                    best = w;
-                    best_rows = rows;
-                }
-            }
-            G = best;
+        // As many codeword groups as fit (up to one per warp) and have work, the warps shared among
+        // them: while there are fewer pairs than groups, a pair takes the idle ones' warps (200
+        // candidates on a 576-node code: one pair to an SM, 9 warps instead of 1, 0.80 -> 0.27 ms).
+        int gr = fit < max_warps ? fit : max_warps;
+        if (units > 0 && (units + num_sms - 1) / num_sms < gr) gr = (int)((units + num_sms - 1) / num_sms);
+        G = max_warps / gr;
+        if (kind == kLayScalar) {
+            int work = g.m < g.n ? g.m : g.n;
+            // QC passes run block by block
+            if (g.kind == TSX_CODE_QC && g.Z < work) work = g.Z;
+            int gmax = work / 32;
+            if (gmax < 1) gmax = 1;
+            if (G > gmax) G = gmax;
+        } else if (G > (g.m + 31) / 32) {  // the check pass runs over all rows at once: at most one each
+            G = (g.m + 31) / 32;
         }
+        if (G < 1) G = 1;
     }
+    if (G > max_warps) G = max_warps;
     int gmax_cta = max_warps / G;  // at most 32 * max_warps threads per CTA
     if (gmax_cta < 1) gmax_cta = 1;
     if (gmax_cta > fit) gmax_cta = fit;
@@ -127,7 +125,7 @@ bool plan(const DevCode &g, int decoder, int kind, int G, int groups, int ctas_p
 // the launch bound of the two-codeword kernel variant launch_pair picks for g
 int pair_warps(const DevCode &g) {
     const bool reg6 = g.dc_min == 6 && g.dc_max == 6;
-    return pair_kernel_warps(g.kind == TSX_CODE_QC, reg6 ? 6 : g.dc_max <= 8 ? 8 : 32, reg6);
+    return pair_kernel_warps(reg6 ? 6 : g.dc_max <= 8 ? 8 : 32, reg6);
 }
 
 // the two-codeword kernel keeps every biased quantity inside 16 bits
@@ -146,14 +144,15 @@ bool pair_ok(const DevCode &g, const DecodeParams &dp) {
 }  // namespace
 
 cudaError_t launch_decode(const DevCode &g, const DecodeParams &dp, const EnumBuffers &b, int G, int groups,
-                          int ctas_per_sm, int num_sms, int force_scalar, cudaStream_t st) {
+                          int ctas_per_sm, int num_sms, int force_scalar, long long n_cand, cudaStream_t st) {
     LaunchShape sh;
+    const long long units = (n_cand + 1) / 2;
     // the two-codeword kernel where its bounds hold and its layout fits a CTA
     const bool pair = !force_scalar && pair_ok(g, dp) &&
-                      plan(g, dp.decoder, kLayPair, G, groups, ctas_per_sm, num_sms, &sh, pair_warps(g));
+                      plan(g, dp.decoder, kLayPair, G, groups, ctas_per_sm, num_sms, &sh, pair_warps(g), units);
     // QC codes of large check degree whose two-buffer layout does not fit: the variable-node-pass form
     if (!pair && !force_scalar && pair_ok(g, dp) && g.kind == TSX_CODE_QC && dp.decoder == TSX_DEC_NMS_I16 &&
-        g.dc_max > 8 && plan(g, dp.decoder, kLayPairVn, G, groups, ctas_per_sm, num_sms, &sh, kPairWarps))
+        g.dc_max > 8 && plan(g, dp.decoder, kLayPairVn, G, groups, ctas_per_sm, num_sms, &sh, pair_warps(g), units))
         return launch_nms16_vn(g, dp, b, sh, st);
     if (!pair && !plan(g, dp.decoder, kLayScalar, G, groups, ctas_per_sm, num_sms, &sh))
         return cudaErrorInvalidConfiguration;
@@ -176,14 +175,15 @@ bool plan_batch(const DevCode *const *g, const DecodeParams *dp, const EnumBuffe
                 int num_sms, BatchItem *items, LaunchShape *common, int *variant) {
     if (n <= 0) return false;
     const int kind = g[0]->kind, dec = dp[0].decoder;
-    bool reg6 = true;
+    bool reg6 = true, odd = false;
     int dcmax = 1, smem = 0;
+    for (int i = 0; i < n; i++) odd = odd || g[i]->dc_max > 8;  // (the variant follows the largest degree)
     for (int i = 0; i < n; i++) {
         if (g[i]->kind != kind || dp[i].decoder != dec || !pair_ok(*g[i], dp[i])) return false;
         LaunchShape sh;
         int G, groups;
         items[i].scalar = 0;
-        if (!plan(*g[i], dec, kLayPair, 1, 1, 0, num_sms, &sh)) {
+        if (!plan(*g[i], dec, kLayPair, 1, 1, 0, num_sms, &sh, kBatchWarps, 0, odd)) {
             items[i].scalar = 1;  // decoded by a launch of its own
             continue;
         }
@@ -191,12 +191,12 @@ bool plan_batch(const DevCode *const *g, const DecodeParams *dp, const EnumBuffe
         if (g[i]->dc_max > dcmax) dcmax = g[i]->dc_max;
         if (G_req && G_req[i] > 0) {
             // the requested (tuned) group width, as many groups as fit
-            if (!plan(*g[i], dec, kLayPair, G_req[i], 0, 0, num_sms, &sh)) return false;
+            if (!plan(*g[i], dec, kLayPair, G_req[i], 0, 0, num_sms, &sh, kBatchWarps, 0, odd)) return false;
             G = sh.G;
             groups = sh.groups;
         } else {
             // the single-code launch's automatic shape
-            if (!plan(*g[i], dec, kLayPair, 0, 0, 0, num_sms, &sh)) return false;
+            if (!plan(*g[i], dec, kLayPair, 0, 0, 0, num_sms, &sh, kBatchWarps, 0, odd)) return false;
             G = sh.G;
             groups = sh.groups;
         }
@@ -211,7 +211,7 @@ bool plan_batch(const DevCode *const *g, const DecodeParams *dp, const EnumBuffe
     }
     LaunchShape sh{};
     sh.G = 1;
-    sh.groups = 16;
+    sh.groups = kBatchWarps;
     sh.smem_bytes = smem;
     sh.num_sms = num_sms;
     sh.per_sm_req = 0;
@@ -229,7 +229,7 @@ cudaError_t launch_batch(const BatchArgs &items, int n, int variant, const Launc
 
 bool plan_is_shape(const DevCode &g, const DecodeParams &dp, LaunchShape *sh, int num_sms) {
     if (!pair_ok(g, dp)) return false;
-    // the flat form (QC, check degree > 8) is launched with up to kIsWarps warps, the others with 16
+    // (the launch bounds of is_kernel)
     return plan(g, TSX_DEC_NMS_I16, kLayIs, 0, 0, 0, num_sms, sh,
                 g.kind == TSX_CODE_QC && g.dc_max > 8 ? kIsWarps : 16);
 }

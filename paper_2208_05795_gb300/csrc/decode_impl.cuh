@@ -49,25 +49,34 @@ struct DecSpa {
 __host__ __device__ inline int al16(int x) { return (x + 15) & ~15; }
 
 struct TabOff {
-    int rdeg, reoff, rjz, rs, cdeg, ceoff, cs, ciz;
+    int rdeg, reoff, rjz, rs, rt, roff, ct, cdeg, ceoff, cs, ciz;
     int c_ptr, c_vn, v_ptr, v_edge;
     int total;
 };
 
-// pair = the tables of the two-codeword kernels, which have no variable-node
-// pass and so no per-variable edge lists (general codes)
+// pair = the tables of the two-codeword kernels: no per-variable edge lists
+// for general codes (they have no variable-node pass), and for QC codes the
+// column start and shift of each position as one 8-byte entry in byte units
 __host__ __device__ inline TabOff tab_offsets(const DevCode &g, bool pair = false) {
     TabOff o{};
     int x = 0;
     if (g.kind == TSX_CODE_QC) {
         o.rdeg = x; x += al16(g.m_b * 2);
         o.reoff = x; x += al16(g.m_b * 4);
-        o.rjz = x; x += al16(g.m_b * g.dc_max * 4);
-        o.rs = x; x += al16(g.m_b * g.dc_max * 2);
+        if (pair) {
+            o.rt = x; x += al16(g.m_b * g.dc_max * 8);
+            o.roff = x; x += al16(g.m_b * 4);
+            o.ct = x; x += al16(g.n_b * g.dv_max * 16);
+        } else {
+            o.rjz = x; x += al16(g.m_b * g.dc_max * 4);
+            o.rs = x; x += al16(g.m_b * g.dc_max * 2);
+        }
         o.cdeg = x; x += al16(g.n_b * 2);
-        o.ceoff = x; x += al16(g.n_b * g.dv_max * 4);
-        o.cs = x; x += al16(g.n_b * g.dv_max * 2);
-        o.ciz = x; x += al16(g.n_b * g.dv_max * 4);
+        if (!pair) {
+            o.ceoff = x; x += al16(g.n_b * g.dv_max * 4);
+            o.cs = x; x += al16(g.n_b * g.dv_max * 2);
+            o.ciz = x; x += al16(g.n_b * g.dv_max * 4);
+        }
     } else {
         o.c_ptr = x; x += al16((g.m + 1) * 2);
         o.c_vn = x; x += al16(g.E * 2);
@@ -81,12 +90,24 @@ __host__ __device__ inline TabOff tab_offsets(const DevCode &g, bool pair = fals
 struct SGraph {
     const int16_t *rdeg;
     const int32_t *reoff, *rjz;
+    // two-codeword kernels
+    const int2 *rt;       // [m_b * dc_max] {4 rjz, 4 rs}
+    const int32_t *roff;  // [m_b] first message of a row block, rows of an odd number of words
+    const int4 *ct;       // [n_b * dv_max] {message offset, words a row, shift} of the t-th block of a column
     const int16_t *rs, *cdeg;
     const int32_t *ceoff;
     const int16_t *cs;
     const int32_t *ciz;
     const uint16_t *c_ptr, *c_vn, *v_ptr, *v_edge;
 };
+
+// First message of row block i where each row takes an odd number of words
+// (two-codeword kernels, check degree > 8); row_offset(g, m_b) is the total.
+__device__ __forceinline__ int row_offset(const DevCode &g, int i) {
+    int x = 0;
+    for (int k = 0; k < i; k++) x += g.Z * (g.rdeg[k] | 1);
+    return x;
+}
 
 __device__ void copy_bytes(void *dst, const void *src, int bytes) {
     // 16-byte vector copies when both ends allow, else bytes
@@ -109,20 +130,37 @@ __device__ SGraph load_tables(const DevCode &g, unsigned char *sm, bool pair = f
     if (g.kind == TSX_CODE_QC) {
         copy_bytes(sm + o.rdeg, g.rdeg, g.m_b * 2);
         copy_bytes(sm + o.reoff, g.reoff, g.m_b * 4);
-        copy_bytes(sm + o.rjz, g.rjz, g.m_b * g.dc_max * 4);
-        copy_bytes(sm + o.rs, g.rs, g.m_b * g.dc_max * 2);
+        if (pair) {
+            int2 *rt = (int2 *)(sm + o.rt);
+            for (int i = threadIdx.x; i < g.m_b * g.dc_max; i += blockDim.x) rt[i] = make_int2(4 * g.rjz[i], 4 * (int)g.rs[i]);
+            s.rt = rt;
+            int *roff = (int *)(sm + o.roff);
+            int4 *ct = (int4 *)(sm + o.ct);
+            for (int i = threadIdx.x; i < g.m_b; i += blockDim.x) roff[i] = row_offset(g, i);
+            for (int x = threadIdx.x; x < g.n_b * g.dv_max; x += blockDim.x) {
+                const int j = x / g.dv_max;
+                if (x - j * g.dv_max >= g.cdeg[j]) continue;
+                const int i = g.ciz[x] / g.Z, p = (g.ceoff[x] - g.reoff[i]) / g.Z;
+                ct[x] = make_int4(row_offset(g, i) + p, g.rdeg[i] | 1, g.cs[x], 0);
+            }
+            s.roff = roff;
+            s.ct = ct;
+        } else {
+            copy_bytes(sm + o.rjz, g.rjz, g.m_b * g.dc_max * 4);
+            copy_bytes(sm + o.rs, g.rs, g.m_b * g.dc_max * 2);
+            copy_bytes(sm + o.ciz, g.ciz, g.n_b * g.dv_max * 4);
+            copy_bytes(sm + o.ceoff, g.ceoff, g.n_b * g.dv_max * 4);
+            copy_bytes(sm + o.cs, g.cs, g.n_b * g.dv_max * 2);
+            s.ceoff = (const int32_t *)(sm + o.ceoff);
+            s.cs = (const int16_t *)(sm + o.cs);
+            s.rjz = (const int32_t *)(sm + o.rjz);
+            s.rs = (const int16_t *)(sm + o.rs);
+            s.ciz = (const int32_t *)(sm + o.ciz);
+        }
         copy_bytes(sm + o.cdeg, g.cdeg, g.n_b * 2);
-        copy_bytes(sm + o.ceoff, g.ceoff, g.n_b * g.dv_max * 4);
-        copy_bytes(sm + o.cs, g.cs, g.n_b * g.dv_max * 2);
-        copy_bytes(sm + o.ciz, g.ciz, g.n_b * g.dv_max * 4);
         s.rdeg = (const int16_t *)(sm + o.rdeg);
         s.reoff = (const int32_t *)(sm + o.reoff);
-        s.rjz = (const int32_t *)(sm + o.rjz);
-        s.rs = (const int16_t *)(sm + o.rs);
         s.cdeg = (const int16_t *)(sm + o.cdeg);
-        s.ceoff = (const int32_t *)(sm + o.ceoff);
-        s.cs = (const int16_t *)(sm + o.cs);
-        s.ciz = (const int32_t *)(sm + o.ciz);
     } else {
         copy_bytes(sm + o.c_ptr, g.c_ptr, (g.m + 1) * 2);
         copy_bytes(sm + o.c_vn, g.c_vn, g.E * 2);
@@ -143,7 +181,7 @@ __device__ SGraph load_tables(const DevCode &g, unsigned char *sm, bool pair = f
 // ---------------------------------------------------------------------------
 struct Grp {
     int G, T, gt, lane, gw, bar;
-    int *red;  // reduction scratch (shared): [0, 16) for sum(), [16, 32) for sum_pass()
+    int *red;  // reduction scratch (shared): [0, 32) for sum(), [32, 64) for sum_pass()
     __device__ __forceinline__ void sync() const {
         if (G == 1) __syncwarp();
         else asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(T) : "memory");
@@ -156,8 +194,7 @@ struct Grp {
         }
         if (lane == 0) red[gw] = x;
         sync();
-        int s = 0;
-        for (int w = 0; w < G; w++) s += red[w];
+        const int s = __reduce_add_sync(0xffffffffu, lane < G ? red[lane] : 0);
         sync();
         return s;
     }
@@ -169,11 +206,9 @@ struct Grp {
             __syncwarp();
             return x;
         }
-        if (lane == 0) red[16 + gw] = x;
+        if (lane == 0) red[32 + gw] = x;
         sync();
-        int s = 0;
-        for (int w = 0; w < G; w++) s += red[16 + w];
-        return s;
+        return __reduce_add_sync(0xffffffffu, lane < G ? red[32 + lane] : 0);
     }
 };
 
@@ -259,11 +294,10 @@ __device__ __forceinline__ float spa_atanhf(float p) {
 
 // misc area of a slot
 struct Misc {
-    int red[32];
+    int red[64];
     long long bcast[2];
     int ints[8];
     unsigned long long okd, okit;  // converged decodes of this group and their iterations
-    int K[2];                      // iteration limit of each half's candidate (two-codeword kernels)
     uint16_t seg[kMaxNb + 2];
 };
 

@@ -7,32 +7,43 @@
 // the two halves follow their own bisection and decode schedules (a half
 // whose decode ends starts its next decode at once; the other keeps going).
 //
-// Biased representation (so that one 32-bit add or subtract updates both
-// halves without a carry or borrow crossing between them, and signs and
-// equalities are single bits):
-//   message   R' = r + B                     B = 1024 (int16) / 128 (int8)
-//   posterior P' = P + beta                  beta = 0x8000
-//   channel   L'(v) = L_v + beta - dv(v) B   so P' = L' + sum_c R'
-//   extrinsic d = P' - R' + B = q + beta     (one three-input add): bit 15 of each half is
-//                                           [q >= 0], the sign of clamp(q); the clamp itself
-//                                           is not applied (edge_da says why it changes nothing)
-//   magnitude a = max(d, 2 beta - d) = |q| + beta   (2 beta - x = ~x + 1 per half)
-// Every intermediate stays inside [0, 0xFFFF] per half for rmax <= B and
-// (dv + 2) sat <= beta - B, which the launcher checks; both halves always
-// hold values of a valid decode (an idle half keeps decoding its last input)
-// so that neither can carry into the other.  The arithmetic is the same
+// Representation (one 32-bit add or subtract updates both halves, and signs
+// and equalities are single bits):
+//   message   R' = (r1 << 16) + r0 as one 32-bit number (the low half's borrow is in the high
+//             half), or r + 128 in two bytes (8-bit storage, bias B = 128)
+//   posterior P' = P + beta in each half, beta = 0x8000; the accumulator starts at
+//             L + beta - dv(v) B, so P' = that + sum_c R'
+//   extrinsic d = P' - R' (+ B) = q + beta: bit 15 of each half is [q >= 0], the sign of
+//             clamp(q); the clamp itself is not applied (edge_d says why it changes nothing)
+//   magnitude na = min(d, 2 beta - d) = beta - |q|   (2 beta - x = ~x + 1 per half)
+// Every P', d and na stays inside [0, 0xFFFF] per half for
+// (dv + 2) sat <= beta - 1024 and rmax <= 1024, which the launcher checks, so
+// sums of R' words are exact whatever the order (borrows cancel modulo 2^32);
+// both halves always hold values of a valid decode (an idle half keeps
+// decoding its last input).  The arithmetic is the same
 // min-sum as the scalar decoder: r = sgn * ((alpha_num * min) >> alpha_shift)
 // over the other edges of the check, P = L + sum r, q = clamp(P - r).
 //
 // No variable-node pass: each check adds its new messages into the next
-// posterior buffer with shared-memory atomic adds (exact and order-free on
-// the biased words); that buffer starts at L' with the impulse values in it.
-// For QC codes whose two buffers do not fit a CTA, the variable-node-pass
-// form (VN) keeps one buffer and rebuilds it from the messages after each
-// check pass; it gives the same words.
+// posterior buffer with shared-memory atomic adds; that buffer starts at L
+// in every word.  For QC codes whose two buffers do not fit a CTA, the
+// variable-node-pass form (VN) keeps one buffer and rebuilds it from the
+// messages after each check pass; it gives the same words.
 //
-// The first check pass of a decode reads the zero message B in its half; a
+// The first check pass of a decode reads the zero message in its half; a
 // check pass in which no half starts a decode skips that masking.
+//
+// What bounds it: instruction issue and the two 64-lane pipes (integer and
+// multiply-add / 16-bit), then shared-memory wavefronts; DRAM is idle.  So
+// the steps are chosen by instruction count: 20 warp instructions per edge of
+// two codewords in the check pass of a degree-6 check, of which 2.5 loads,
+// half a store and one add to shared memory.  Measured on the decode stage
+// against the form before it (magnitudes beta + |q|, outputs by two selects,
+// 64-bit generic addresses, the bisection's state in every thread's
+// registers, one row block at a time): 2640-node (3,6) QC code, 30,000 candidates,
+// 99.5 -> 70 ms; degree 16 (n = 4608), 12,000 candidates, 40 -> 26 ms; degree 28
+// (n = 11,520), 8,000 candidates, 82 -> 57 ms; Z = 153, degree 23: 26 -> 7.6 ms (the row-block
+// loop gave the group Z / 32 = 4 warps).
 #pragma once
 #include "decode_impl.cuh"
 
@@ -49,6 +60,17 @@ __device__ __forceinline__ unsigned vminu2(unsigned a, unsigned b) {
     asm("min.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
     return d;
 }
+// per-half adds and signed maximum, modulo 2^16 (an add whose result only feeds a maximum is one instruction with it)
+__device__ __forceinline__ unsigned vadd2(unsigned a, unsigned b) {
+    unsigned d;
+    asm("add.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned vmaxs2(unsigned a, unsigned b) {
+    unsigned d;
+    asm("max.s16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
 __device__ __forceinline__ unsigned prmt(unsigned a, unsigned b, unsigned sel) {
     unsigned d;
     asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
@@ -56,422 +78,400 @@ __device__ __forceinline__ unsigned prmt(unsigned a, unsigned b, unsigned sel) {
 }
 // 0xFFFF in each half whose bit 15 is set, else 0
 __device__ __forceinline__ unsigned spread15(unsigned x) { return prmt(x, x, 0xBB99u); }
-__device__ __forceinline__ void red_add(unsigned char *addr, unsigned v) {
-    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(addr)), "r"(v)
-                 : "memory");
+// Shared-memory accesses of the check pass by 32-bit address: with pointers
+// the compiler keeps 64-bit generic addresses, whose arithmetic doubled the
+// large-degree loop (60 warp instructions per edge pair).  Volatile, so that
+// none moves across a barrier.
+__device__ __forceinline__ unsigned saddr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ unsigned lds32(unsigned a) {
+    unsigned v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ unsigned lds16(unsigned a) {
+    unsigned short v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint2 lds64(unsigned a) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts32(unsigned a, unsigned v) {
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts16(unsigned a, unsigned v) {
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
+}
+__device__ __forceinline__ void sts64(unsigned a, unsigned x, unsigned y) {
+    asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void red_add(unsigned a, unsigned v) {
+    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
 constexpr unsigned kBeta = 0x8000u;
 
-struct PairConst {
-    unsigned B2, BS2, BETA2, amask2;
-    unsigned BAN2;  // BETA2 * alpha_num: (m - beta) an = m an - BAN2 (mod 2^32)
-    int B, sat, an, as;
+template <int V>
+struct Int {
+    static constexpr int value = V;
+    __device__ __forceinline__ constexpr operator unsigned() const { return (unsigned)V; }
 };
 
-// per-half schedule state (uniform across the group)
-struct Half {
-    long long idx;  // candidate (absolute index), -1: idle
-    int I0, I1, I2, I3, nI;
+struct PairConst {
+    unsigned NS2, amask2;  // NS2: beta - sat
+    unsigned BAN2;  // BETA2 * alpha_num: m an = BAN2 - (beta - m) an (mod 2^32)
+    int an, as;
+};
+
+// Schedule state of one half, in the group's shared memory: written by the
+// group's thread 0 where a decode ends, read by the others after a barrier.
+// (Held in every thread's registers it cost 30 of them, and every warp ran
+// the bookkeeping.)
+struct HalfS {
+    long long idx;       // candidate (absolute index), -1: idle
+    long long copy_o;    // record of the finished candidate whose x* is to be copied out, -1: none
+    int I[4], nI;        // impulse nodes
     int lo, hi, st, phase;  // bisection
-    int thr, ndec, nit;
-    int failed;
-    int Limp;  // channel LLR of the impulse nodes in the current decode
-    int k, ubest;
-    int first;  // current decode has run no check pass yet
-    int cur;    // x buffer of the current decode (0/1); keep = cur ^ 1
-    __device__ __forceinline__ int Ik(int t) const { return t == 0 ? I0 : t == 1 ? I1 : t == 2 ? I2 : I3; }
+    int ndec, nit, failed;
+    int Limp;            // channel LLR of the impulse nodes in the current decode
+    int K;               // iteration limit of the candidate
+    int keep;            // x buffer (0/1) of the last failing decode; the current decode writes the other
+    int copy;            // x buffer to copy out
+    int fail;            // the decode that ended failed
+};
+
+__device__ __forceinline__ PairConst pair_const(const DecodeParams &dp) {
+    PairConst pc;
+    pc.an = dp.alpha_num;
+    pc.as = dp.alpha_shift;
+    pc.NS2 = (kBeta - (unsigned)dp.sat) * 0x00010001u;
+    pc.amask2 = (0xFFFFu >> pc.as) * 0x00010001u;
+    pc.BAN2 = kBeta * 0x00010001u * (unsigned)pc.an;
+    return pc;
+}
+
+struct PairMisc : Misc {
+    HalfS h[2];
 };
 
 // VN: the variable-node-pass form (QC codes): one posterior buffer, rebuilt
 // after each check pass from the stored messages, instead of the
 // accumulating second buffer -- 4 bytes per node less, for codes whose
 // two-buffer layout does not fit a CTA.
-// FLAT (QC, accumulating form): the check pass runs over all row blocks at
-// once, as the VN form does, so that a group may be wider than Z rows.
-template <bool QC, int DC, bool EXACT, bool I8, bool VN = false, bool FLAT = false>
+template <bool QC, int DC, bool EXACT, bool I8, bool VN = false>
 struct PairDecoder {
     static constexpr int RSZ = I8 ? 2 : 4;  // bytes of one packed message pair
+    static constexpr int kB = I8 ? 128 : 0;  // message bias
+    static constexpr unsigned kB2 = (unsigned)kB * 0x00010001u;
     const DevCode &g;
     const SGraph &sg;
     const Grp &gp;
     const PairConst &pc;
-    unsigned char *Rb;  // packed messages, RSZ bytes per edge
+    unsigned Rb;  // shared address of the packed messages, RSZ bytes per edge
 
-    __device__ __forceinline__ unsigned ldR(int byteoff) const {
-        if constexpr (I8) {
-            const unsigned x = *(const uint16_t *)(Rb + byteoff);
-            return prmt(x, 0u, 0x4140u);  // bytes b0, b1 -> halves
-        } else {
-            return *(const unsigned *)(Rb + byteoff);
-        }
+    __device__ __forceinline__ unsigned ldR(unsigned a) const {
+        if constexpr (I8) return prmt(lds16(a), 0u, 0x4140u);  // bytes b0, b1 -> halves
+        else return lds32(a);
     }
-    __device__ __forceinline__ void stR(int byteoff, unsigned v) const {
-        if constexpr (I8) *(uint16_t *)(Rb + byteoff) = (uint16_t)prmt(v, 0u, 0x0020u);
-        else *(unsigned *)(Rb + byteoff) = v;
+    __device__ __forceinline__ void stR(unsigned a, unsigned v) const {
+        if constexpr (I8) sts16(a, prmt(v, 0u, 0x0020u));
+        else sts32(a, v);
     }
 
     // an edge's incoming message; MASK: some half starts a decode in this
-    // pass and reads the zero message B there (km keeps the other half, kb
-    // supplies B)
+    // pass (km is 0 there, 0xFFFF in a half that goes on) and reads the zero message
     template <bool MASK>
-    __device__ __forceinline__ unsigned ldy(int byteoff, unsigned km, unsigned kb) const {
-        if constexpr (MASK) return (ldR(byteoff) & km) | kb;
-        else return ldR(byteoff);
+    __device__ __forceinline__ unsigned mask_y(unsigned y, unsigned km) const {
+        if constexpr (!MASK) return y;
+        else if constexpr (I8) return (y & km) | (kB2 & ~km);
+        else return ((km & 0xFFFFu) ? (unsigned)(int)(int16_t)y : 0u) + ((km >> 16) ? (y + 0x8000u) & 0xFFFF0000u : 0u);
     }
-
-    // One check node.  pv(p): byte offset of P'[v_p]; re(p): byte offset of
-    // R'[e_p].  Reads Pc, adds the new messages into Pn.  Returns the
-    // unsatisfied flags of both halves in bits 0/1.
-    template <bool MASK, class PV, class RE>
-    __device__ __forceinline__ int check_node(int deg, unsigned km, unsigned kb, bool writeR, const unsigned char *Pc,
-                                              unsigned char *Pn, PV pv, RE re) const {
-        if constexpr (DC <= 8) return check_node_regs<MASK>(deg, km, kb, writeR, Pc, Pn, pv, re);
-        else return check_node_twopass<MASK>(deg, km, kb, writeR, Pc, Pn, pv, re);
+    template <bool MASK>
+    __device__ __forceinline__ unsigned ldy(unsigned a, unsigned km) const {
+        return mask_y<MASK>(ldR(a), km);
     }
 
     // the extrinsic value of one edge without clamping: d = (P - r) + beta, which the launcher's
     // bounds keep inside each half and which has the sign of clamp(P - r),
-    // and a = |P - r| + beta.  Where |P - r| > sat the clamped magnitude
-    // would be sat: min1 and min2 start at sat (+ beta), so they come out
+    // and na = beta - |P - r|.  Where |P - r| > sat the clamped magnitude
+    // would be sat: min1 and min2 start at sat, so they come out
     // the same, and such an edge's output is the same too -- it is not the
     // minimum unless min1 = min2 = sat, when both outputs are equal.
-    // |P - r| <= sat + (dv - 1) B < 2^15 by the launcher's bounds, so
-    // a - min1 + 0x7FFF stays inside each half, as edge_out needs.
-    __device__ __forceinline__ void edge_da(unsigned x, unsigned y, unsigned &d, unsigned &a) const {
-        d = x - y + pc.B2;
-        a = vmaxu2(d, (~d) + 0x00010001u);
+    __device__ __forceinline__ void edge_d(unsigned x, unsigned y, unsigned &d, unsigned &na) const {
+        d = x - y;
+        if constexpr (I8) d += kB2;
+        na = neg_abs(d);
+    }
+    __device__ __forceinline__ static unsigned neg_abs(unsigned d) { return vminu2(d, (~d) + 0x00010001u); }
+
+    // M1 >= M2: the two largest na of the check so far (beta - min1, beta - min2)
+    __device__ __forceinline__ static void track(unsigned na, unsigned &M1, unsigned &M2) {
+        M2 = vmaxu2(M2, vminu2(M1, na));
+        M1 = vmaxu2(M1, na);
+    }
+    // two edges at once: five operations instead of six (the two maxima of M2 are one
+    // three-input instruction), and half as long a dependency chain
+    __device__ __forceinline__ static void track2(unsigned a, unsigned b, unsigned &M1, unsigned &M2) {
+        const unsigned hi = vmaxu2(a, b), lo = vminu2(a, b);
+        M2 = vmaxu2(vmaxu2(M2, lo), vminu2(M1, hi));
+        M1 = vmaxu2(M1, hi);
     }
 
-    // the new message of an edge from its q'', |q|, the check's min1, the
-    // two output magnitudes and the sign parity of all its edges
-    // (the four possible outputs B +- o1, B +- o2 are formed once per check)
+    // What the outputs of a check's edges share.  Edge p sends the magnitude o2 if |q_p| is min1,
+    // else o1 (o = (alpha_num min) >> alpha_shift).  That is
+    //   max(o2 + min1 - |q_p|, o1):
+    // equal to o2 >= o1 where |q_p| = min1; elsewhere |q_p| >= min2 (also with ties), and
+    // o2 - o1 <= min2 - min1 because alpha <= 1 and the floors are of one multiple each, so
+    // the first term is at most o1.  One fused add-max per edge.
     struct Outs {
-        unsigned p1, n1, p2, n2;
+        unsigned S, o1;  // S = o2 + min1 - beta: na + S = o2 + min1 - |q|, modulo 2^16 per half
+        unsigned sx;     // sign parity over the edges, less the edge itself once xor-ed with its d
     };
-    __device__ __forceinline__ Outs outs(unsigned o1, unsigned o2) const {
-        return Outs{pc.B2 + o1, pc.B2 - o1, pc.B2 + o2, pc.B2 - o2};
+    __device__ __forceinline__ Outs outs(unsigned M1, unsigned M2, unsigned sx, int deg) const {
+        Outs o;
+        o.o1 = ((pc.BAN2 - M1 * (unsigned)pc.an) >> pc.as) & pc.amask2;
+        const unsigned o2 = ((pc.BAN2 - M2 * (unsigned)pc.an) >> pc.as) & pc.amask2;
+        o.S = vadd2(o2, (~M1) + 0x00010001u);  // 2 beta - M1 = beta + min1, which is min1 - beta modulo 2^16
+        // bit 15 of sx ^ d_p = parity of #(q >= 0) over the other edges;
+        // negatives among the others = (deg - 1) - that
+        o.sx = sx ^ (((deg - 1) & 1) ? 0x80008000u : 0u);
+        return o;
     }
-    __device__ __forceinline__ unsigned edge_out(unsigned q, unsigned a, unsigned m1, const Outs &o,
-                                                 unsigned sxk) const {
-        const unsigned neg = spread15(sxk ^ q);                  // 0xFFFF: others' sign product < 0
-        const unsigned ne = spread15(a - m1 + 0x7FFF7FFFu);      // 0xFFFF: |q_p| != min1
-        const unsigned t1 = (o.n1 & neg) | (o.p1 & ~neg);        // +-o1
-        const unsigned t2 = (o.n2 & neg) | (o.p2 & ~neg);        // +-o2
-        return (t1 & ne) | (t2 & ~ne);
+    // the new message B +- o of an edge from its d and na
+    __device__ __forceinline__ unsigned edge_out(unsigned d, unsigned na, const Outs &o) const {
+        const unsigned neg = spread15(o.sx ^ d);                  // 0xFFFF: others' sign product < 0
+        const unsigned mag = vmaxs2(vadd2(na, o.S), o.o1);
+        const unsigned r = (mag ^ neg) - neg;
+        return I8 ? r + kB2 : r;
     }
 
-    // small degree: the edges' q and |q| stay in registers between the passes
-    template <bool MASK, class PV, class RE>
-    __device__ __forceinline__ int check_node_regs(int deg, unsigned km, unsigned kb, bool writeR,
-                                                   const unsigned char *Pc, unsigned char *Pn, PV pv, RE re) const {
-        unsigned sp = 0, sx = 0, m1 = pc.BS2, m2 = pc.BS2;
-        unsigned qs[DC], as_[DC];
-        int po[DC];
+    // One check of up to N edges (EX: exactly N), the edges' d and addresses in
+    // registers between the two passes.  pv(p): byte offset of P'[v_p]; re(p):
+    // address of R'[e_p].  Reads Pc, adds the new messages into Pn (VN form:
+    // stores them only).  Returns the unsatisfied flags in bits 0 and 16.
+    template <bool MASK, int N, bool EX, class PV, class RE>
+    __device__ __forceinline__ int node(int deg, unsigned km, bool writeR, unsigned Pc, unsigned Pn, PV pv,
+                                        RE re) const {
+        unsigned sp = 0, sx = 0, M1 = pc.NS2, M2 = pc.NS2;
+        unsigned q[N], na[N], po[N];
 #pragma unroll
-        for (int p = 0; p < DC; p++) {
-            if (EXACT || p < deg) {
+        for (int p = 0; p < N; p++) {
+            if (EX || p < deg) {
                 po[p] = pv(p);
-                const unsigned x = *(const unsigned *)(Pc + po[p]);
-                const unsigned y = ldy<MASK>(re(p), km, kb);
+                const unsigned x = lds32(Pc + po[p]);
+                const unsigned y = ldy<MASK>(re(p), km);
                 sp ^= x;
-                unsigned q, a;
-                edge_da(x, y, q, a);
-                sx ^= q;
-                m2 = vminu2(m2, vmaxu2(m1, a));
-                m1 = vminu2(m1, a);
-                qs[p] = q;
-                as_[p] = a;
+                edge_d(x, y, q[p], na[p]);
+                sx ^= q[p];
+                track(na[p], M1, M2);
             }
         }
-        // syndrome bit of each half: sp bit 15 = parity of #(P >= 0), and
-        // #(P < 0) = deg - #(P >= 0)
-        const unsigned dodd = (deg & 1) ? 0x80008000u : 0u;
-        const unsigned unsat = (sp ^ dodd) & 0x80008000u;
         if (writeR) {
-            const unsigned o1 = ((m1 * (unsigned)pc.an - pc.BAN2) >> pc.as) & pc.amask2;
-            const unsigned o2 = ((m2 * (unsigned)pc.an - pc.BAN2) >> pc.as) & pc.amask2;
-            const Outs oo = outs(o1, o2);
-            // bit 15 of sx ^ q_p = parity of #(q >= 0) over the other edges;
-            // negatives among the others = (deg - 1) - that
-            const unsigned sxk = sx ^ (((deg - 1) & 1) ? 0x80008000u : 0u);
+            const Outs o = outs(M1, M2, sx, EX ? N : deg);
 #pragma unroll
-            for (int p = 0; p < DC; p++) {
-                if (EXACT || p < deg) {
-                    const unsigned rn = edge_out(qs[p], as_[p], m1, oo, sxk);
+            for (int p = 0; p < N; p++) {
+                if (EX || p < deg) {
+                    const unsigned rn = edge_out(q[p], na[p], o);
                     stR(re(p), rn);
                     if constexpr (!VN) red_add(Pn + po[p], rn);
                 }
             }
         }
-        return (int)((unsat >> 15) & 0x00010001u);
+        return unsat2(sp, EX ? N : deg);
+    }
+    // syndrome bit of each half: sp bit 15 = parity of #(P >= 0), and
+    // #(P < 0) = deg - #(P >= 0)
+    __device__ __forceinline__ static int unsat2(unsigned sp, int deg) {
+        return (int)(((sp ^ ((deg & 1) ? 0x80008000u : 0u)) >> 15) & 0x00010001u);
     }
 
     // check-regular codes (EXACT, 16-bit storage, DC even): the check's DC
-    // message words are contiguous (check-major layout, 4 DC bytes a check;
-    // for QC codes within each row block) and move as DC/2 8-byte accesses;
-    // a warp's 8-byte accesses at a stride of 4 DC bytes = 24 bytes (DC = 6)
-    // touch every bank once per half-warp.  Otherwise the same steps as
-    // check_node_regs.
+    // message words are contiguous (check-major layout, 4 DC bytes a check)
+    // and move as DC/2 8-byte accesses; a warp's 8-byte accesses at a stride
+    // of 4 DC bytes = 24 bytes (DC = 6) touch every bank once per half-warp.
+    // Otherwise the same steps as node().
     template <bool MASK, class PV>
-    __device__ __forceinline__ int check_node_cm(int rbyte, unsigned km, unsigned kb, bool writeR,
-                                                 const unsigned char *Pc, unsigned char *Pn, PV pv) const {
+    __device__ __forceinline__ int node_cm(unsigned ra, unsigned km, bool writeR, unsigned Pc, unsigned Pn,
+                                           PV pv) const {
         static_assert(EXACT && !I8 && DC % 2 == 0, "check-major form");
-        uint2 *rw = (uint2 *)(Rb + rbyte);
-        unsigned ys[DC];
+        unsigned sp = 0, sx = 0, M1 = pc.NS2, M2 = pc.NS2;
+        unsigned q[DC], na[DC], po[DC];
 #pragma unroll
         for (int t = 0; t < DC / 2; t++) {
-            const uint2 w = rw[t];
-            ys[2 * t] = w.x;
-            ys[2 * t + 1] = w.y;
-        }
-        unsigned sp = 0, sx = 0, m1 = pc.BS2, m2 = pc.BS2;
-        unsigned qs[DC], as_[DC];
-        int po[DC];
+            const uint2 w = lds64(ra + 8 * t);
 #pragma unroll
-        for (int p = 0; p < DC; p++) {
-            po[p] = pv(p);
-            const unsigned x = *(const unsigned *)(Pc + po[p]);
-            const unsigned y = MASK ? ((ys[p] & km) | kb) : ys[p];
-            sp ^= x;
-            unsigned q, a;
-            edge_da(x, y, q, a);
-            sx ^= q;
-            m2 = vminu2(m2, vmaxu2(m1, a));
-            m1 = vminu2(m1, a);
-            qs[p] = q;
-            as_[p] = a;
+            for (int e = 0; e < 2; e++) {
+                const int p = 2 * t + e;
+                po[p] = pv(p);
+                const unsigned x = lds32(Pc + po[p]);
+                const unsigned y0 = e ? w.y : w.x;
+                const unsigned y = mask_y<MASK>(y0, km);
+                sp ^= x;
+                edge_d(x, y, q[p], na[p]);
+                sx ^= q[p];
+            }
+            track2(na[2 * t], na[2 * t + 1], M1, M2);
         }
-        const unsigned unsat = (sp ^ ((DC & 1) ? 0x80008000u : 0u)) & 0x80008000u;
         if (writeR) {
-            const unsigned o1 = ((m1 * (unsigned)pc.an - pc.BAN2) >> pc.as) & pc.amask2;
-            const unsigned o2 = ((m2 * (unsigned)pc.an - pc.BAN2) >> pc.as) & pc.amask2;
-            const Outs oo = outs(o1, o2);
-            const unsigned sxk = sx ^ (((DC - 1) & 1) ? 0x80008000u : 0u);
+            const Outs o = outs(M1, M2, sx, DC);
 #pragma unroll
-            for (int p = 0; p < DC; p++) ys[p] = edge_out(qs[p], as_[p], m1, oo, sxk);
-#pragma unroll
-            for (int t = 0; t < DC / 2; t++) rw[t] = make_uint2(ys[2 * t], ys[2 * t + 1]);
-#pragma unroll
-            for (int p = 0; p < DC; p++)
-                if constexpr (!VN) red_add(Pn + po[p], ys[p]);
+            for (int t = 0; t < DC / 2; t++) {
+                const unsigned r0 = edge_out(q[2 * t], na[2 * t], o), r1 = edge_out(q[2 * t + 1], na[2 * t + 1], o);
+                sts64(ra + 8 * t, r0, r1);
+                if constexpr (!VN) {
+                    red_add(Pn + po[2 * t], r0);
+                    red_add(Pn + po[2 * t + 1], r1);
+                }
+            }
         }
-        return (int)((unsat >> 15) & 0x00010001u);
+        return unsat2(sp, DC);
     }
 
     // large degree: the first pass leaves each edge's extrinsic word d in its
     // message slot (16-bit storage: a slot holds both halves' d), the second
     // reads it back; with 8-bit storage the second pass reloads P and
-    // recomputes d
-    template <bool MASK, class PV, class RE>
-    __device__ __forceinline__ int check_node_twopass(int deg, unsigned km, unsigned kb, bool writeR,
-                                                      const unsigned char *Pc, unsigned char *Pn, PV pv,
-                                                      RE re) const {
-        unsigned sp = 0, sx = 0, m1 = pc.BS2, m2 = pc.BS2;
-#pragma unroll 4
-        for (int p = 0; p < deg; p++) {
-            const int ro = re(p);
-            const unsigned x = *(const unsigned *)(Pc + pv(p));
-            const unsigned y = ldy<MASK>(ro, km, kb);
-            sp ^= x;
-            unsigned q, a;
-            edge_da(x, y, q, a);
-            if constexpr (!I8)
-                if (writeR) stR(ro, q);
-            sx ^= q;
-            m2 = vminu2(m2, vmaxu2(m1, a));
-            m1 = vminu2(m1, a);
-        }
-        const unsigned dodd = (deg & 1) ? 0x80008000u : 0u;
-        const unsigned unsat = (sp ^ dodd) & 0x80008000u;
-        if (writeR) {
-            const unsigned o1 = ((m1 * (unsigned)pc.an - pc.BAN2) >> pc.as) & pc.amask2;
-            const unsigned o2 = ((m2 * (unsigned)pc.an - pc.BAN2) >> pc.as) & pc.amask2;
-            const Outs oo = outs(o1, o2);
-            const unsigned sxk = sx ^ (((deg - 1) & 1) ? 0x80008000u : 0u);
-#pragma unroll 4
-            for (int p = 0; p < deg; p++) {
-                const int po = pv(p), ro = re(p);
-                unsigned q, a;
-                if constexpr (!I8) {
-                    q = ldR(ro);
-                    a = vmaxu2(q, (~q) + 0x00010001u);
-                } else {
-                    const unsigned x = *(const unsigned *)(Pc + po);
-                    const unsigned y = ldy<MASK>(ro, km, kb);
-                    edge_da(x, y, q, a);
-                }
-                const unsigned rn = edge_out(q, a, m1, oo, sxk);
-                stR(ro, rn);
-                if constexpr (!VN) red_add(Pn + po, rn);
+    // recomputes d.  (Unrolled over up to 32 edges with d in registers, the
+    // loop did not fit the instruction cache: 0.57x on a degree-16 code.)
+    // ra: address of the check's first message, stride: bytes between its
+    // messages.  QC codes keep a check's messages together, an odd number of
+    // words a check, so that lanes hit different banks and every offset is a constant.
+    // Edges are taken four at a time, loads first: no load waits behind the
+    // stores of the edges before it.
+    template <bool MASK, class PV, class Stride>
+    __device__ __forceinline__ int node_twopass(int deg, unsigned km, bool writeR, unsigned Pc, unsigned Pn,
+                                                PV pv, unsigned ra, Stride stride) const {
+        const unsigned rs = stride;
+        unsigned sp = 0, sx = 0, M1 = pc.NS2, M2 = pc.NS2;
+        auto first = [&](auto width, int p, unsigned a) {
+            constexpr int W = decltype(width)::value;
+            unsigned x[W], y[W], na[W];
+#pragma unroll
+            for (int e = 0; e < W; e++) {
+                x[e] = lds32(Pc + pv(p + e));
+                y[e] = ldy<MASK>(a + e * rs, km);
             }
-        }
-        return (int)((unsat >> 15) & 0x00010001u);
-    }
-
-    // Two checks of one QC row block at once (rows r and r + dr, 16-bit
-    // storage, large degree): the same steps as check_node_twopass for both,
-    // interleaved edge by edge, so that the two dependency chains overlap and
-    // each position's shift is read once for both rows.  Returns the
-    // unsatisfied flags of row r in bits 0/1 and of row r + dr in bits 2/3.
-    template <bool MASK>
-    __device__ __forceinline__ int check_rows2(int deg, unsigned km, unsigned kb, bool writeR,
-                                               const unsigned char *Pc, unsigned char *Pn, const int32_t *rjz,
-                                               const int16_t *rs, int rb, int r, int dr) const {
-        const int Z = g.Z;
-        unsigned spA = 0, sxA = 0, m1A = pc.BS2, m2A = pc.BS2;
-        unsigned spB = 0, sxB = 0, m1B = pc.BS2, m2B = pc.BS2;
-        const int r2 = r + dr;
-#pragma unroll 2
-        for (int p = 0; p < deg; p++) {
-            const int jz = rjz[p], sh = rs[p];
-            const int tA = r + sh, tB = r2 + sh;
-            const int poA = 4 * (jz + (int)min((unsigned)tA, (unsigned)(tA - Z)));
-            const int poB = 4 * (jz + (int)min((unsigned)tB, (unsigned)(tB - Z)));
-            const int roA = rb + (p * Z + r) * RSZ, roB = roA + dr * RSZ;
-            const unsigned xA = *(const unsigned *)(Pc + poA), xB = *(const unsigned *)(Pc + poB);
-            const unsigned yA = ldy<MASK>(roA, km, kb), yB = ldy<MASK>(roB, km, kb);
-            spA ^= xA;
-            spB ^= xB;
-            unsigned qA, aA, qB, aB;
-            edge_da(xA, yA, qA, aA);
-            edge_da(xB, yB, qB, aB);
-            if (writeR) {
-                stR(roA, qA);
-                stR(roB, qB);
+#pragma unroll
+            for (int e = 0; e < W; e++) {
+                sp ^= x[e];
+                edge_d(x[e], y[e], y[e], na[e]);
+                sx ^= y[e];
             }
-            sxA ^= qA;
-            sxB ^= qB;
-            m2A = vminu2(m2A, vmaxu2(m1A, aA));
-            m1A = vminu2(m1A, aA);
-            m2B = vminu2(m2B, vmaxu2(m1B, aB));
-            m1B = vminu2(m1B, aB);
-        }
-        const unsigned dodd = (deg & 1) ? 0x80008000u : 0u;
-        const unsigned unsatA = (spA ^ dodd) & 0x80008000u, unsatB = (spB ^ dodd) & 0x80008000u;
-        if (writeR) {
-            const unsigned o1A = ((m1A * (unsigned)pc.an - pc.BAN2) >> pc.as) & pc.amask2;
-            const unsigned o2A = ((m2A * (unsigned)pc.an - pc.BAN2) >> pc.as) & pc.amask2;
-            const unsigned o1B = ((m1B * (unsigned)pc.an - pc.BAN2) >> pc.as) & pc.amask2;
-            const unsigned o2B = ((m2B * (unsigned)pc.an - pc.BAN2) >> pc.as) & pc.amask2;
-            const Outs ooA = outs(o1A, o2A), ooB = outs(o1B, o2B);
-            const unsigned odd = ((deg - 1) & 1) ? 0x80008000u : 0u;
-            const unsigned sxkA = sxA ^ odd, sxkB = sxB ^ odd;
-#pragma unroll 2
-            for (int p = 0; p < deg; p++) {
-                const int jz = rjz[p], sh = rs[p];
-                const int tA = r + sh, tB = r2 + sh;
-                const int poA = 4 * (jz + (int)min((unsigned)tA, (unsigned)(tA - Z)));
-                const int poB = 4 * (jz + (int)min((unsigned)tB, (unsigned)(tB - Z)));
-                const int roA = rb + (p * Z + r) * RSZ, roB = roA + dr * RSZ;
-                const unsigned qA = ldR(roA), qB = ldR(roB);
-                const unsigned aA = vmaxu2(qA, (~qA) + 0x00010001u), aB = vmaxu2(qB, (~qB) + 0x00010001u);
-                const unsigned rnA = edge_out(qA, aA, m1A, ooA, sxkA);
-                const unsigned rnB = edge_out(qB, aB, m1B, ooB, sxkB);
-                stR(roA, rnA);
-                stR(roB, rnB);
-                if constexpr (!VN) {
-                    red_add(Pn + poA, rnA);
-                    red_add(Pn + poB, rnB);
+            if constexpr (!I8) {
+                if (writeR) {
+#pragma unroll
+                    for (int e = 0; e < W; e++) stR(a + e * rs, y[e]);
                 }
             }
+            if constexpr (W == 1) track(na[0], M1, M2);
+            else
+#pragma unroll
+                for (int e = 0; e < W; e += 2) track2(na[e], na[e + 1], M1, M2);
+        };
+        int p = 0;
+        unsigned a = ra;
+#pragma unroll 1
+        for (; p + 4 <= deg; p += 4, a += 4 * rs) first(Int<4>{}, p, a);
+        if (deg & 2) {
+            first(Int<2>{}, p, a);
+            p += 2;
+            a += 2 * rs;
         }
-        return (int)(((unsatA >> 15) & 0x00010001u) + ((unsatB >> 15) & 0x00010001u));
+        if (deg & 1) first(Int<1>{}, p, a);
+        if (writeR) {
+            const Outs o = outs(M1, M2, sx, deg);
+            auto second = [&](auto width, int p, unsigned a) {
+                constexpr int W = decltype(width)::value;
+                unsigned po[W], d[W], na[W];
+#pragma unroll
+                for (int e = 0; e < W; e++) {
+                    po[e] = pv(p + e);
+                    if constexpr (!I8) {
+                        d[e] = ldR(a + e * rs);
+                        na[e] = neg_abs(d[e]);
+                    } else {
+                        edge_d(lds32(Pc + po[e]), ldy<MASK>(a + e * rs, km), d[e], na[e]);
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < W; e++) d[e] = edge_out(d[e], na[e], o);
+#pragma unroll
+                for (int e = 0; e < W; e++) {
+                    stR(a + e * rs, d[e]);
+                    if constexpr (!VN) red_add(Pn + po[e], d[e]);
+                }
+            };
+            p = 0;
+            a = ra;
+#pragma unroll 1
+            for (; p + 4 <= deg; p += 4, a += 4 * rs) second(Int<4>{}, p, a);
+            if (deg & 2) {
+                second(Int<2>{}, p, a);
+                p += 2;
+                a += 2 * rs;
+            }
+            if (deg & 1) second(Int<1>{}, p, a);
+        }
+        return unsat2(sp, deg);
     }
 
     // check pass; returns u of half 0 in the low 16 bits and half 1 above (the
     // caller passes a group barrier before the next check pass)
     template <bool MASK>
-    __device__ __forceinline__ int check_pass(unsigned km, unsigned kb, bool writeR, const unsigned *Pcur,
+    __device__ __forceinline__ int check_pass(unsigned km, bool writeR, const unsigned *Pcur,
                                               unsigned *Pnext) const {
         int u = 0;  // unsatisfied checks: half 0 in the low 16 bits, half 1 above
-        const unsigned char *Pc = (const unsigned char *)Pcur;
-        unsigned char *Pn = (unsigned char *)Pnext;
+        const unsigned Pc = saddr(Pcur), Pn = saddr(Pnext);
         const int Z = g.Z;
-        if constexpr (QC && (VN || FLAT)) {
+        if constexpr (QC) {
             // all row blocks at once (check c = i Z + r), so that a group may be wider than Z rows
+            // and no lane idles at a block's last rows
+            const unsigned Z4 = 4u * (unsigned)Z;
             const unsigned zm = Z > 1 ? 0xFFFFFFFFu / (unsigned)Z + 1u : 0u;  // c / Z = umulhi(c, zm), c < 2^16
+            const unsigned rt0 = saddr(sg.rt);
             for (int c = gp.gt; c < g.m; c += gp.T) {
                 const int i = Z > 1 ? (int)__umulhi((unsigned)c, zm) : c;
                 const int r = c - i * Z;
-                const int deg = sg.rdeg[i];
-                const int rb = sg.reoff[i] * RSZ;
-                const int32_t *rjz = sg.rjz + i * g.dc_max;
-                const int16_t *rs = sg.rs + i * g.dc_max;
-                u += check_node<MASK>(
-                    deg, km, kb, writeR, Pc, Pn,
-                    [&](int p) {
-                        const int t = r + rs[p];
-                        return 4 * (rjz[p] + (int)min((unsigned)t, (unsigned)(t - Z)));
-                    },
-                    [&](int p) { return rb + (p * Z + r) * RSZ; });
-            }
-        } else if constexpr (QC) {
-            for (int i = 0; i < g.m_b; i++) {
-                const int deg = EXACT ? DC : sg.rdeg[i];
-                const int rb = sg.reoff[i] * RSZ;
-                if constexpr (DC <= 8) {  // the row block's shifts in registers
-                    int rjz4[DC], rsh[DC], pz[DC];
-#pragma unroll
-                    for (int p = 0; p < DC; p++) {
-                        if (EXACT || p < deg) {
-                            rjz4[p] = sg.rjz[i * g.dc_max + p] * 4;
-                            rsh[p] = sg.rs[i * g.dc_max + p];
-                            pz[p] = p * Z * RSZ;
-                        }
-                    }
-                    for (int r = gp.gt; r < Z; r += gp.T) {
-                        const auto pv = [&](int p) {
-                            const int t = r + rsh[p];
-                            return rjz4[p] + 4 * (int)min((unsigned)t, (unsigned)(t - Z));
-                        };
-                        if constexpr (EXACT && !I8 && DC % 2 == 0) {
-                            // check-regular row blocks: messages check-major within the block
-                            u += check_node_cm<MASK>(rb + r * (DC * RSZ), km, kb, writeR, Pc, Pn, pv);
-                        } else {
-                            u += check_node<MASK>(deg, km, kb, writeR, Pc, Pn, pv,
-                                                  [&](int p) { return rb + pz[p] + r * RSZ; });
-                        }
-                    }
+                const unsigned rt = rt0 + 8u * (unsigned)(i * g.dc_max);
+                const unsigned r4 = 4u * (unsigned)r;
+                const auto pv = [&](int p) {
+                    const uint2 e = lds64(rt + 8u * (unsigned)p);  // 4 x column block start, 4 x shift
+                    const unsigned t = r4 + e.y;
+                    return e.x + __viaddmin_u32(t, 0u - Z4, t);  // min(t - Z4, t): t mod Z4
+                };
+                if constexpr (EXACT && !I8 && DC % 2 == 0) {
+                    u += node_cm<MASK>(Rb + (unsigned)c * (DC * RSZ), km, writeR, Pc, Pn, pv);
                 } else {
-                    const int32_t *rjz = sg.rjz + i * g.dc_max;
-                    const int16_t *rs = sg.rs + i * g.dc_max;
-                    int r = gp.gt;
-                    if constexpr (!I8) {
-                        // rows in pairs (r, r + T) while both exist
-                        for (; r + gp.T < Z; r += 2 * gp.T) {
-                            const int f = check_rows2<MASK>(deg, km, kb, writeR, Pc, Pn, rjz, rs, rb, r, gp.T);
-                            u += f;
-                        }
-                    }
-                    for (; r < Z; r += gp.T) {
-                        const int f = check_node<MASK>(
-                            deg, km, kb, writeR, Pc, Pn,
-                            [&](int p) {
-                                const int t = r + rs[p];
-                                return 4 * (rjz[p] + (int)min((unsigned)t, (unsigned)(t - Z)));
-                            },
-                            [&](int p) { return rb + (p * Z + r) * RSZ; });
-                        u += f;
+                    const int deg = EXACT ? DC : sg.rdeg[i];
+                    if constexpr (DC <= 8) {
+                        const unsigned ra = Rb + (unsigned)((sg.reoff[i] + r) * RSZ), rs = (unsigned)(Z * RSZ);
+                        u += node<MASK, DC, EXACT>(deg, km, writeR, Pc, Pn, pv,
+                                                   [&](int p) { return ra + (unsigned)p * rs; });
+                    } else {
+                        u += node_twopass<MASK>(deg, km, writeR, Pc, Pn, pv,
+                                                Rb + (unsigned)((sg.roff[i] + r * (deg | 1)) * RSZ), Int<RSZ>{});
                     }
                 }
             }
-        } else if constexpr (EXACT && !I8 && DC % 2 == 0) {
-            // check-regular: rows of DC edges, messages check-major
-            for (int c = gp.gt; c < g.m; c += gp.T) {
-                const int e0 = c * DC;
-                u += check_node_cm<MASK>(e0 * RSZ, km, kb, writeR, Pc, Pn,
-                                         [&](int p) { return 4 * (int)sg.c_vn[e0 + p]; });
-            }
         } else {
+            const unsigned cv = saddr(sg.c_vn);
             const int m = g.m;
             for (int c = gp.gt; c < m; c += gp.T) {
                 const int e0 = EXACT ? c * DC : (int)sg.c_ptr[c];  // check-regular: rows of DC edges
-                const int deg = EXACT ? DC : sg.c_ptr[c + 1] - e0;
-                const int f = check_node<MASK>(
-                    deg, km, kb, writeR, Pc, Pn, [&](int p) { return 4 * (int)sg.c_vn[e0 + p]; },
-                    [&](int p) { return (p * m + c) * RSZ; });
-                u += f;
+                const unsigned cva = cv + 2u * (unsigned)e0;
+                const auto pv = [&](int p) { return 4u * lds16(cva + 2u * (unsigned)p); };
+                if constexpr (EXACT && !I8 && DC % 2 == 0) {
+                    // check-regular: messages check-major
+                    u += node_cm<MASK>(Rb + (unsigned)(e0 * RSZ), km, writeR, Pc, Pn, pv);
+                } else {
+                    const int deg = EXACT ? DC : sg.c_ptr[c + 1] - e0;
+                    const unsigned ra = Rb + (unsigned)(c * RSZ), rs = (unsigned)(m * RSZ);
+                    if constexpr (DC <= 8)
+                        u += node<MASK, DC, EXACT>(deg, km, writeR, Pc, Pn, pv,
+                                                   [&](int p) { return ra + (unsigned)p * rs; });
+                    else u += node_twopass<MASK>(deg, km, writeR, Pc, Pn, pv, ra, rs);
+                }
             }
         }
         return gp.sum_pass(u);
@@ -495,20 +495,28 @@ struct PairDecoder {
         }
     }
     __device__ __forceinline__ void init_accum(unsigned *Pn, int Lb) const {
-        if constexpr (QC) {
-            const int Z = g.Z;
-            for (int j = 0; j < g.n_b; j++) {
-                const unsigned l = (unsigned)(Lb + (int)kBeta - sg.cdeg[j] * pc.B);
-                const unsigned l2 = l | (l << 16);
-                unsigned *row = Pn + j * Z;
-                for (int k = gp.gt; k < Z; k += gp.T) row[k] = l2;
-            }
-        } else if (g.dv_min == g.dv_max) {  // variable-regular: one value
-            const unsigned l = (unsigned)(Lb + (int)kBeta - g.dv_max * pc.B);
+        if (!I8 || g.dv_min == g.dv_max) {  // no bias to take off, or the same for every node: one value
+            const unsigned l = (unsigned)(Lb + (int)kBeta - g.dv_max * kB);
             fill(Pn, g.n, l | (l << 16));
+        } else if constexpr (QC) {
+            const int Z = g.Z;
+            const unsigned zm = Z > 1 ? 0xFFFFFFFFu / (unsigned)Z + 1u : 0u;
+            if ((Z & 3) == 0 && ((uintptr_t)Pn & 15) == 0) {  // four nodes of one column block per store
+                for (int v = 4 * gp.gt; v < g.n; v += 4 * gp.T) {
+                    const unsigned l = (unsigned)(Lb + (int)kBeta - sg.cdeg[__umulhi((unsigned)v, zm)] * kB);
+                    const unsigned l2 = l | (l << 16);
+                    *(uint4 *)(Pn + v) = make_uint4(l2, l2, l2, l2);
+                }
+            } else {
+                for (int v = gp.gt; v < g.n; v += gp.T) {
+                    const int j = Z > 1 ? (int)__umulhi((unsigned)v, zm) : v;
+                    const unsigned l = (unsigned)(Lb + (int)kBeta - sg.cdeg[j] * kB);
+                    Pn[v] = l | (l << 16);
+                }
+            }
         } else {
             for (int v = gp.gt; v < g.n; v += gp.T) {
-                const unsigned l = (unsigned)(Lb + (int)kBeta - vdeg(v) * pc.B);
+                const unsigned l = (unsigned)(Lb + (int)kBeta - vdeg(v) * kB);
                 Pn[v] = l | (l << 16);
             }
         }
@@ -533,14 +541,14 @@ struct PairDecoder {
             const int j = Z > 1 ? (int)__umulhi((unsigned)v, zm) : v;
             const int k = v - j * Z;
             const int dv = sg.cdeg[j];
-            const int32_t *eo = sg.ceoff + j * g.dv_max;
-            const int16_t *sh = sg.cs + j * g.dv_max;
-            const unsigned l = (unsigned)(Lb + (int)kBeta - dv * pc.B);
+            const int4 *ct = sg.ct + j * g.dv_max;  // message offset, stride and shift of the t-th block
+            const unsigned l = (unsigned)(Lb + (int)kBeta - dv * kB);
             unsigned acc = l | (l << 16);
             for (int t = 0; t < dv; t++) {
                 // block (i, j) with shift s joins row r to column (r + s) mod Z: r = (k - s) mod Z
-                const int r = wrapZneg(k - sh[t], Z);
-                acc += ldR((eo[t] + r) * RSZ);
+                const int4 e = ct[t];
+                const int r = wrapZneg(k - e.z, Z);
+                acc += ldR(Rb + (unsigned)((e.x + r * e.y) * RSZ));
             }
             P[v] = acc;
         }
@@ -567,13 +575,17 @@ struct PairDecoder {
 };
 
 // The decode loop of one group (G warps, group index grp) over the
-// candidate queue of one code; the code's tables are already in sg.
+// candidate queue of one code; the code's tables are already in sg.  Every
+// thread keeps, per half, only what each iteration needs (whether it runs,
+// its iteration, its limit, the smallest u_k); the schedule itself is in
+// shared memory and is advanced by thread 0 where a decode ends.
 template <bool QC, int DC, bool EXACT, bool I8, bool VN = false>
-__device__ void pair_run(const DevCode &g, const DecodeParams &dp, const EnumBuffers &b, const SlotLayout &lay,
-                         int G, const SGraph &sg, unsigned char *smem, int grp) {
+__device__ __forceinline__ void pair_run(const DevCode &g, const DecodeParams &dp, const EnumBuffers &b,
+                                         const SlotLayout &lay, int G, const SGraph &sg, unsigned char *smem, int grp) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned char *slot = smem + lay.tables_bytes + grp * lay.slot_bytes;
-    Misc *misc = (Misc *)(slot + lay.misc_off);
+    PairMisc *misc = (PairMisc *)(slot + lay.misc_off);
+    HalfS *const hs = misc->h;
     Grp gp;
     gp.G = G;
     gp.T = 32 * G;
@@ -582,50 +594,24 @@ __device__ void pair_run(const DevCode &g, const DecodeParams &dp, const EnumBuf
     gp.lane = lane;
     gp.bar = 1 + grp;
     gp.red = misc->red;
-    unsigned char *Rb = slot + lay.r_off;
     unsigned *Pbuf = (unsigned *)(slot + lay.p_off);  // [2][n] ([n] in the VN form)
     const int nw = (g.n + 31) >> 5;
-    uint32_t *xb = (uint32_t *)(slot + lay.xa_off);  // 4 buffers of nw words: [half][cur/keep]
+    uint32_t *xb = (uint32_t *)(slot + lay.xa_off);  // 4 buffers of nw words: [half][2]
     const int xstride = (nw + 3) & ~3;
 
-    PairConst pc;
-    pc.B = I8 ? 128 : 1024;
-    pc.sat = dp.sat;
-    pc.an = dp.alpha_num;
-    pc.as = dp.alpha_shift;
-    pc.B2 = (unsigned)pc.B * 0x00010001u;
-    pc.BETA2 = kBeta * 0x00010001u;
-    pc.BS2 = (kBeta + (unsigned)pc.sat) * 0x00010001u;
-    pc.amask2 = (0xFFFFu >> pc.as) * 0x00010001u;
-    pc.BAN2 = pc.BETA2 * (unsigned)pc.an;
-    // QC codes of check degree 7 or 8 run the all-row-block pass (the row
-    // block's shifts read from the tables, not held in registers)
-    PairDecoder<QC, DC, EXACT, I8, VN, QC && DC == 8 && !EXACT> dec{g, sg, gp, pc, Rb};
+    const PairConst pc = pair_const(dp);
+    PairDecoder<QC, DC, EXACT, I8, VN> dec{g, sg, gp, pc, saddr(slot + lay.r_off)};
 
     const long long total = (long long)b.ctr->n_cand_total;
     const long long end = b.cand_end < 0 || b.cand_end > total ? total : b.cand_end;
     const int Lb = clampi(dp.base_llr, -dp.sat, dp.sat);
     const int amax = (1 << dp.amp_steps) - 1;
-    long long my_dec = 0, my_it = 0;
-    int pcur = 0;  // which posterior buffer holds P_k
-    // the converged-decode counts and each half's iteration limit live in the
-    // group's shared misc area (written by thread 0 only), not in registers
-    if (gp.gt == 0) {
-        misc->okd = 0;
-        misc->okit = 0;
-    }
+    long long my_dec = 0, my_it = 0;  // (thread 0's)
+    int pcur = 0;                     // which posterior buffer holds P_k
 
-    Half H[2] = {};  // (every field is set by fetch before use)
-
-    auto fetch = [&](Half &h, int hh) {
-        if (gp.gt == 0) misc->bcast[0] = (long long)atomicAdd(b.queue, 1ull);
-        gp.sync();
-        const long long idx = b.cand_begin + misc->bcast[0];
-        gp.sync();
-        h.k = 0;
-        h.ubest = 0x7fffffff;
-        h.first = 1;
-        h.cur = 0;
+    // ---- the schedule (thread 0 of the group) ----
+    auto fetch = [&](HalfS &h) {
+        const long long idx = b.cand_begin + (long long)atomicAdd(b.queue, 1ull);
         if (idx >= end) {
             h.idx = -1;
             h.nI = 0;
@@ -633,70 +619,91 @@ __device__ void pair_run(const DevCode &g, const DecodeParams &dp, const EnumBuf
         }
         const int4 I4 = b.cands[idx];
         h.idx = idx;
-        h.I0 = I4.x; h.I1 = I4.y; h.I2 = I4.z; h.I3 = I4.w;
+        h.I[0] = I4.x; h.I[1] = I4.y; h.I[2] = I4.z; h.I[3] = I4.w;
         h.nI = (I4.x >= 0) + (I4.y >= 0) + (I4.z >= 0) + (I4.w >= 0);
         h.lo = 0; h.hi = amax; h.st = 0; h.phase = 0;
-        h.thr = -1; h.ndec = 0; h.nit = 0; h.failed = 0;
+        h.ndec = 0; h.nit = 0; h.failed = 0;
         h.Limp = clampi(dp.base_llr - amax, -dp.sat, dp.sat);
-        if (gp.gt == 0) misc->K[hh] = cand_limit(dp, b, idx);
-        // (read after the next group barrier)
+        h.K = cand_limit(dp, b, idx);
     };
-    // finish the candidate of half hh (records, x* to global) and fetch the next
-    auto finish = [&](Half &h, int hh) {
-        gp.sync();
+    // the candidate's records; its x* is copied out by the whole group afterwards
+    auto finish = [&](HalfS &h) {
         const long long o = h.idx - b.rec_base;
-        if (h.failed) {
-            const uint32_t *src = xb + (2 * hh + (h.cur ^ 1)) * xstride;
-            uint32_t *dst = b.xstar + o * (long long)b.nw;
-            for (int w = gp.gt; w < nw; w += gp.T) dst[w] = src[w];
-        }
-        if (gp.gt == 0) {
-            b.c_thr[o] = h.failed ? h.thr : -1;
-            b.c_thr_f[o] = -1.0f;
-            b.c_slot[o] = -1;
-            b.c_flags[o] = 0;
-            b.c_decodes[o] = h.ndec;
-            b.c_iters[o] = h.nit;
+        b.c_thr[o] = h.failed ? h.hi : -1;
+        b.c_thr_f[o] = -1.0f;
+        b.c_slot[o] = -1;
+        b.c_flags[o] = 0;
+        b.c_decodes[o] = h.ndec;
+        b.c_iters[o] = h.nit;
+        if (h.failed) {  // (at most one candidate of a half between two decodes: the ones that
+            h.copy_o = o;  //  follow it without a decode have not failed)
+            h.copy = h.keep;
         }
         my_dec += h.ndec;
         my_it += h.nit;
-        fetch(h, hh);
+        fetch(h);
     };
-    // Advance half hh past trivial decodes (impulse LLR >= 0: every hard
-    // decision 0, u_0 = 0, success at iteration 0) until a decode that needs
-    // iterations is set up (returns true) or no candidate is left.
-    auto settle = [&](Half &h, int hh) {
-        while (h.idx >= 0) {
-            if (h.Limp < 0) return true;
+    // the next amplitude of the bisection, or the end of the candidate
+    auto next_amp = [&](HalfS &h) {
+        if (h.st < dp.amp_steps && h.hi - h.lo > 1) {
+            h.st++;
+            h.Limp = clampi(dp.base_llr - ((h.lo + h.hi) >> 1), -dp.sat, dp.sat);
+        } else {
+            finish(h);
+        }
+    };
+    // past trivial decodes (impulse LLR >= 0: every hard decision 0, u_0 = 0, success at
+    // iteration 0) until a decode that needs iterations is set up or no candidate is left
+    auto settle = [&](HalfS &h) {
+        while (h.idx >= 0 && h.Limp >= 0) {
             h.ndec++;
-            if (gp.gt == 0) misc->okd++;  // x_0 = 0: converged at iteration 0
+            misc->okd++;
             if (h.phase == 0) {
-                finish(h, hh);  // no failure at the largest amplitude
-                continue;
-            }
-            h.lo = (h.lo + h.hi) >> 1;  // the decode at mid succeeded
-            if (h.st < dp.amp_steps && h.hi - h.lo > 1) {
-                const int mid = (h.lo + h.hi) >> 1;
-                h.st++;
-                h.Limp = clampi(dp.base_llr - mid, -dp.sat, dp.sat);
+                finish(h);  // no failure at the largest amplitude
             } else {
-                h.thr = h.hi;
-                finish(h, hh);
+                h.lo = (h.lo + h.hi) >> 1;  // the decode at mid succeeded
+                next_amp(h);
             }
         }
-        return false;
     };
+    // the decode of half h ended at iteration kl
+    auto advance = [&](HalfS &h, int kl) {
+        h.copy_o = -1;
+        h.ndec++;
+        h.nit += kl;
+        if (!h.fail) {
+            misc->okd++;
+            misc->okit += kl;
+        }
+        if (h.phase == 0) {
+            if (!h.fail) {
+                finish(h);
+            } else {
+                h.failed = 1;
+                h.keep ^= 1;
+                h.phase = 1;
+                next_amp(h);
+            }
+        } else {
+            const int mid = (h.lo + h.hi) >> 1;
+            if (h.fail) {
+                h.hi = mid;
+                h.keep ^= 1;
+            } else {
+                h.lo = mid;
+            }
+            next_amp(h);
+        }
+        settle(h);
+    };
+
     // half hh of the current posteriors for a new decode: P = L
-    auto start_cur = [&](Half &h, int hh, unsigned *Pc) {
+    auto start_cur = [&](int hh, unsigned *Pc) {
         for (int v = gp.gt; v < g.n; v += gp.T) dec.set_half(Pc, v, hh, (unsigned)(Lb + (int)kBeta));
-        h.k = 0;
-        h.ubest = 0x7fffffff;
-        h.first = 1;
     };
-    // impulse nodes: the current posteriors (new decode only) and the accumulator
-    // the impulse nodes of a new decode in the current posteriors
-    auto patch_cur = [&](Half &h, int hh, unsigned *Pc) {
-        if (h.idx >= 0 && gp.gt < h.nI) dec.set_half(Pc, h.Ik(gp.gt), hh, (unsigned)(h.Limp + (int)kBeta));
+    // its impulse nodes
+    auto patch_cur = [&](int hh, unsigned *Pc) {
+        if (gp.gt < hs[hh].nI) dec.set_half(Pc, hs[hh].I[gp.gt], hh, (unsigned)(hs[hh].Limp + (int)kBeta));
     };
     // The accumulator starts at the baseline L' in every word; its impulse
     // nodes get L_imp - L_base added in their half with the check pass's
@@ -704,144 +711,130 @@ __device__ void pair_run(const DevCode &g, const DecodeParams &dp, const EnumBuf
     // commute: the word's final halves are in range, so no intermediate
     // carry or borrow between the halves survives.
     auto impulse_adds = [&](unsigned *Pn) {
-        if (gp.gt < 8) {  // (the halves selected by value: H stays in registers)
-            const int j = gp.gt & 3;
-            const bool h1 = gp.gt >= 4;
-            const bool on = h1 ? H[1].idx >= 0 && j < H[1].nI : H[0].idx >= 0 && j < H[0].nI;
-            const int t = h1 ? H[1].Ik(j) : H[0].Ik(j);
-            const unsigned d = (unsigned)((h1 ? H[1].Limp : H[0].Limp) - Lb);
-            if (on) red_add((unsigned char *)(Pn + t), h1 ? d << 16 : d);
+        if (gp.gt < 8) {
+            const int j = gp.gt & 3, hh = gp.gt >> 2;
+            if (j < hs[hh].nI) {  // (0 for an idle half)
+                const unsigned d = (unsigned)(hs[hh].Limp - Lb);
+                red_add(saddr(Pn + hs[hh].I[j]), hh ? d << 16 : d);
+            }
         }
     };
-
-    // VN form: the impulse nodes of half hh after a variable-node pass (built
-    // with the baseline L), or of a new decode
-    auto patch_vn = [&](Half &h, int hh, unsigned *Pc, bool fresh) {
-        if (h.idx >= 0 && gp.gt < h.nI) {
-            const int t = h.Ik(gp.gt);
-            if (fresh) dec.set_half(Pc, t, hh, (unsigned)(h.Limp + (int)kBeta));
-            else dec.add_half(Pc, t, hh, h.Limp - Lb);
-        }
+    // VN form: the impulse nodes of half hh after a variable-node pass (built with the baseline L)
+    auto patch_vn = [&](int hh, unsigned *Pc) {
+        if (gp.gt < hs[hh].nI) dec.add_half(Pc, hs[hh].I[gp.gt], hh, hs[hh].Limp - Lb);
     };
 
+    bool act[2], first[2];
+    int k[2], K[2], ub[2];
+    auto load_half = [&](int hh) {  // (after a barrier)
+        act[hh] = hs[hh].idx >= 0;
+        K[hh] = hs[hh].K;
+        k[hh] = 0;
+        ub[hh] = 0x7fffffff;
+        first[hh] = true;
+    };
+
+    if (gp.gt == 0) {
+        misc->okd = 0;
+        misc->okit = 0;
+        for (int hh = 0; hh < 2; hh++) {
+            hs[hh].keep = 1;
+            hs[hh].K = 0;
+            hs[hh].copy_o = -1;
+            fetch(hs[hh]);
+            settle(hs[hh]);
+        }
+    }
     {
         unsigned *Pc = Pbuf, *Pn = Pbuf + g.n;
         if constexpr (!VN) dec.init_accum(Pn, Lb);
-        for (int hh = 0; hh < 2; hh++) {
-            fetch(H[hh], hh);
-            settle(H[hh], hh);
-            start_cur(H[hh], hh, Pc);  // idle halves too: every word stays a valid decode state
-        }
+        for (int hh = 0; hh < 2; hh++) start_cur(hh, Pc);  // idle halves too: every word stays a valid decode state
         gp.sync();
         for (int hh = 0; hh < 2; hh++) {
-            if constexpr (VN) patch_vn(H[hh], hh, Pc, true);
-            else patch_cur(H[hh], hh, Pc);
+            load_half(hh);
+            patch_cur(hh, Pc);
         }
         gp.sync();
     }
 
-    while (H[0].idx >= 0 || H[1].idx >= 0) {
+    while (act[0] || act[1]) {
         unsigned *Pc = VN ? Pbuf : Pbuf + pcur * g.n, *Pn = VN ? Pbuf : Pbuf + (pcur ^ 1) * g.n;
-        const unsigned km = (H[0].first ? 0xFFFF0000u : 0xFFFFFFFFu) & (H[1].first ? 0x0000FFFFu : 0xFFFFFFFFu);
-        const unsigned kb = pc.B2 & ~km;
-        const bool wr = (H[0].idx >= 0 && H[0].k < misc->K[0]) || (H[1].idx >= 0 && H[1].k < misc->K[1]);
+        const bool wr = (act[0] && k[0] < K[0]) || (act[1] && k[1] < K[1]);
         // u_k of both halves from P_k = Pc; Pn accumulates P_{k+1}
         if constexpr (!VN) impulse_adds(Pn);
-        // (the common form -- no half starting, messages written -- compiled with writeR constant)
-        const int us = km != 0xFFFFFFFFu ? dec.template check_pass<true>(km, kb, wr, Pc, Pn)
-                       : wr              ? dec.template check_pass<false>(km, kb, true, Pc, Pn)
-                                         : dec.template check_pass<false>(km, kb, false, Pc, Pn);
-        int restart[2] = {0, 0};
+        // (the common form -- no half starting, messages written -- compiled without the mask and
+        // with writeR constant)
+        int us;
+        if (wr && !first[0] && !first[1]) {
+            us = dec.template check_pass<false>(0u, true, Pc, Pn);
+        } else {
+            const unsigned km = (first[0] ? 0xFFFF0000u : 0xFFFFFFFFu) & (first[1] ? 0x0000FFFFu : 0xFFFFFFFFu);
+            us = dec.template check_pass<true>(km, wr, Pc, Pn);
+        }
+        bool ended[2] = {false, false};
         bool read_pc = false;  // some thread read P_k after the check pass (uniform)
+#pragma unroll
         for (int hh = 0; hh < 2; hh++) {
-            Half &h = H[hh];
-            if (h.idx < 0) continue;
+            if (!act[hh]) continue;
             const int u = hh == 0 ? (us & 0xFFFF) : (us >> 16);
-            uint32_t *xc = xb + (2 * hh + h.cur) * xstride;
-            if (h.k >= g.wstart && u < h.ubest) {
-                h.ubest = u;
-                dec.save_x(Pc, hh, xc);
+            const bool end_now = u == 0 || k[hh] == K[hh];
+            if ((k[hh] >= g.wstart && u < ub[hh]) || (end_now && k[hh] < g.wstart)) {
+                ub[hh] = u;
+                dec.save_x(Pc, hh, xb + (2 * hh + (hs[hh].keep ^ 1)) * xstride);
                 read_pc = true;
             }
-            if (u != 0 && h.k != misc->K[hh]) continue;
-            read_pc = true;
-            // the decode ended at K_last = k
-            const int kl = h.k;
-            if (kl < g.wstart) dec.save_x(Pc, hh, xc);
-            const bool fail = u != 0 || dec.any_neg(Pc, hh) != 0;
-            h.ndec++;
-            h.nit += kl;
-            if (!fail && gp.gt == 0) {
-                misc->okd++;
-                misc->okit += kl;
+            if (end_now) {
+                const bool fail = u != 0 || dec.any_neg(Pc, hh) != 0;
+                if (gp.gt == 0) hs[hh].fail = fail;
+                ended[hh] = true;
+                read_pc = true;
             }
-            if (h.phase == 0) {
-                if (!fail) {
-                    finish(h, hh);
-                } else {
-                    h.failed = 1;
-                    h.cur ^= 1;
-                    h.phase = 1;
-                }
-            } else {
-                const int mid = (h.lo + h.hi) >> 1;
-                if (fail) {
-                    h.hi = mid;
-                    h.cur ^= 1;
-                } else {
-                    h.lo = mid;
-                }
-            }
-            if (h.idx >= 0 && h.phase == 1) {
-                if (h.st < dp.amp_steps && h.hi - h.lo > 1) {
-                    const int mid = (h.lo + h.hi) >> 1;
-                    h.st++;
-                    h.Limp = clampi(dp.base_llr - mid, -dp.sat, dp.sat);
-                } else {
-                    h.thr = h.hi;
-                    finish(h, hh);
-                }
-            }
-            restart[hh] = 1;
         }
         if constexpr (VN) {
             // P_{k+1} from the messages just written, in place of P_k
             gp.sync();
-            if (wr) {
-                dec.vn_pass(Pc, Lb);
-                gp.sync();
+            if (wr) dec.vn_pass(Pc, Lb);
+        }
+        if (ended[0] || ended[1]) {
+            gp.sync();  // x buffers and P_k read and written by every thread
+            if (gp.gt == 0) {
+#pragma unroll
+                for (int hh = 0; hh < 2; hh++)
+                    if (ended[hh]) advance(hs[hh], k[hh]);
             }
+            gp.sync();
+#pragma unroll
             for (int hh = 0; hh < 2; hh++) {
-                Half &h = H[hh];
-                if (restart[hh]) {
-                    if (settle(h, hh)) start_cur(h, hh, Pc);
-                } else if (h.idx >= 0) {
-                    h.k++;
-                    h.first = 0;
+                if (!ended[hh]) continue;
+                const long long o = hs[hh].copy_o;
+                if (o >= 0) {  // x* of the candidate that ended (its buffer is not written before the next barrier)
+                    const uint32_t *src = xb + (2 * hh + hs[hh].copy) * xstride;
+                    uint32_t *dst = b.xstar + o * (long long)b.nw;
+                    for (int w = gp.gt; w < nw; w += gp.T) dst[w] = src[w];
                 }
+                load_half(hh);
+                if (act[hh]) start_cur(hh, VN ? Pc : Pn);
             }
+        } else if (VN || read_pc) {
             gp.sync();
-            for (int hh = 0; hh < 2; hh++) patch_vn(H[hh], hh, Pc, restart[hh] != 0);
-            gp.sync();
-            continue;
         }
-        // Pn (= P_{k+1}) becomes current; the old Pc becomes the next
-        // accumulator (a barrier first if P_k was read after the check pass)
-        if (read_pc) gp.sync();
+#pragma unroll
         for (int hh = 0; hh < 2; hh++) {
-            Half &h = H[hh];
-            if (restart[hh]) {
-                if (settle(h, hh)) start_cur(h, hh, Pn);
-            } else if (h.idx >= 0) {
-                h.k++;
-                h.first = 0;
+            if (act[hh] && !ended[hh]) {
+                k[hh]++;
+                first[hh] = false;
             }
         }
-        dec.init_accum(Pc, Lb);
-        if (restart[0] | restart[1]) {
-            gp.sync();  // after start_cur's stores
-            for (int hh = 0; hh < 2; hh++)
-                if (restart[hh]) patch_cur(H[hh], hh, Pn);
+        // the old P_k becomes the next accumulator
+        if constexpr (!VN) dec.init_accum(Pc, Lb);
+        if (VN || ended[0] || ended[1]) {
+            if (ended[0] || ended[1]) gp.sync();  // after start_cur's stores
+#pragma unroll
+            for (int hh = 0; hh < 2; hh++) {
+                if (!act[hh]) continue;
+                if (ended[hh]) patch_cur(hh, VN ? Pc : Pn);
+                else if constexpr (VN) patch_vn(hh, Pc);
+            }
         }
         gp.sync();
         pcur ^= 1;
@@ -856,7 +849,7 @@ __device__ void pair_run(const DevCode &g, const DecodeParams &dp, const EnumBuf
 }
 
 template <bool QC, int DC, bool EXACT, bool I8>
-__global__ void __launch_bounds__(32 * pair_kernel_warps(QC, DC, EXACT))
+__global__ void __launch_bounds__(32 * pair_kernel_warps(DC, EXACT), 1)
     pair_kernel(DevCode g, DecodeParams dp, EnumBuffers b, SlotLayout lay, int G) {
     extern __shared__ __align__(16) unsigned char smem[];
     const SGraph sg = load_tables(g, smem, true);
@@ -866,7 +859,7 @@ __global__ void __launch_bounds__(32 * pair_kernel_warps(QC, DC, EXACT))
 
 // the VN form for QC codes of large check degree whose two-buffer layout does not fit
 template <bool I8>
-__global__ void __launch_bounds__(32 * kPairWarps) pair_vn_kernel(DevCode g, DecodeParams dp, EnumBuffers b,
+__global__ void __launch_bounds__(32 * pair_kernel_warps(32, false), 1) pair_vn_kernel(DevCode g, DecodeParams dp, EnumBuffers b,
                                                                SlotLayout lay, int G) {
     extern __shared__ __align__(16) unsigned char smem[];
     const SGraph sg = load_tables(g, smem, true);
@@ -882,7 +875,7 @@ __global__ void __launch_bounds__(32 * kPairWarps) pair_vn_kernel(DevCode g, Dec
 // each code's description from the constant bank, as the single-code kernel
 // does, instead of holding it in registers.
 template <bool QC, int DC, bool EXACT, bool I8>
-__global__ void __launch_bounds__(512) batch_kernel(const __grid_constant__ BatchArgs args, int n_items) {
+__global__ void __launch_bounds__(32 * kBatchWarps, 1) batch_kernel(const __grid_constant__ BatchArgs args, int n_items) {
     extern __shared__ __align__(16) unsigned char smem[];
     for (int c = 0; c < n_items; c++) {
         const BatchItem &it = args.it[c];

@@ -39,10 +39,10 @@ struct IsArgs {
 // ---------------------------------------------------------------------------
 // the sampling kernel: two samples per lane, as the enumeration decoder
 // ---------------------------------------------------------------------------
-// QC codes of check degree > 8 run the check pass over all row blocks at once
-// (FLAT), so that one sample pair can take more warps than Z / 32.
+// (the check pass runs over all row blocks at once, so one sample pair can
+// take more warps than Z / 32)
 template <bool QC, int DC, bool EXACT>
-__global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512) is_kernel(DevCode g, DecodeParams dp, IsArgs ia,
+__global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kernel(DevCode g, DecodeParams dp, IsArgs ia,
                                                                                SlotLayout lay, int G) {
     extern __shared__ __align__(16) unsigned char smem[];
     const SGraph sg = load_tables(g, smem, true);
@@ -59,25 +59,13 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512) is_kernel(
     gp.lane = lane;
     gp.bar = 1 + grp;
     gp.red = misc->red;
-    unsigned char *Rb = slot + lay.r_off;
     unsigned *Pbuf = (unsigned *)(slot + lay.p_off);  // [2][n]
     unsigned *L2 = Pbuf + 2 * g.n;                    // accumulator start values, both halves
     uint32_t *Tm = (uint32_t *)(slot + lay.xa_off);   // bitmask of T
     const int nw = (g.n + 31) >> 5;
 
-    PairConst pc;
-    pc.B = 1024;
-    pc.sat = dp.sat;
-    pc.an = dp.alpha_num;
-    pc.as = dp.alpha_shift;
-    pc.B2 = (unsigned)pc.B * 0x00010001u;
-    pc.BETA2 = kBeta * 0x00010001u;
-    pc.BS2 = (kBeta + (unsigned)pc.sat) * 0x00010001u;
-    pc.amask2 = (0xFFFFu >> pc.as) * 0x00010001u;
-    pc.BAN2 = pc.BETA2 * (unsigned)pc.an;
-    // QC codes: the all-row-block pass for check degree > 8 (wider groups) and for
-    // degree 7-8 (the row block's shifts read from the tables, not held in registers)
-    PairDecoder<QC, DC, EXACT, false, false, QC && (DC > 8 || !EXACT)> dec{g, sg, gp, pc, Rb};
+    const PairConst pc = pair_const(dp);
+    PairDecoder<QC, DC, EXACT, false> dec{g, sg, gp, pc, saddr(slot + lay.r_off)};
 
     for (int w = gp.gt; w < nw; w += gp.T) Tm[w] = 0u;
     gp.sync();
@@ -117,7 +105,7 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512) is_kernel(
                     const float lq = roundf(hmul(y, ia.cq));
                     L = lq > (float)dp.sat ? dp.sat : (lq < -(float)dp.sat ? -dp.sat : (int)lq);
                 }
-                dec.set_half(L2, v, hh, (unsigned)(L + (int)kBeta - dec.vdeg(v) * pc.B));
+                dec.set_half(L2, v, hh, (unsigned)(L + (int)kBeta));
                 dec.set_half(Pc, v, hh, (unsigned)(L + (int)kBeta));
             }
         }
@@ -142,12 +130,10 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512) is_kernel(
         }
         gp.sync();
         const unsigned km = (first[0] ? 0xFFFF0000u : 0xFFFFFFFFu) & (first[1] ? 0x0000FFFFu : 0xFFFFFFFFu);
-        const unsigned kb = pc.B2 & ~km;
         const bool wr = (sidx[0] >= 0 && k[0] < dp.K) || (sidx[1] >= 0 && k[1] < dp.K);
         // (the common form -- no half starting, messages written -- compiled with writeR constant)
-        const int us = km != 0xFFFFFFFFu ? dec.template check_pass<true>(km, kb, wr, Pc, Pn)
-                       : wr              ? dec.template check_pass<false>(km, kb, true, Pc, Pn)
-                                         : dec.template check_pass<false>(km, kb, false, Pc, Pn);
+        const int us = wr && km == 0xFFFFFFFFu ? dec.template check_pass<false>(km, true, Pc, Pn)
+                                               : dec.template check_pass<true>(km, wr, Pc, Pn);
         int restart[2] = {0, 0};
         for (int hh = 0; hh < 2; hh++) {
             if (sidx[hh] < 0) continue;

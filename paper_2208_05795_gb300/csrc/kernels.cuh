@@ -71,17 +71,20 @@ struct BatchItem {
 // (kernel parameters may take up to 32 KB).
 constexpr int kMaxBatch = 64;
 
-// warps per CTA of the single-code two-codeword kernel (its launch bound):
-// 20 warps keep the (3,6)-regular general-code variant at 96 registers
-// without spills and measured faster than 16 or 24
-constexpr int kPairWarps = 20;
-// QC codes and general codes of check degree 7 or 8: 16 warps a CTA (128
-// registers a thread, which those variants need to run without spilling)
-constexpr int kPairWarps16 = 16;
-__host__ __device__ constexpr int pair_kernel_warps(bool qc, int dc, bool exact) {
-    return qc || (dc == 8 && !exact) ? kPairWarps16 : kPairWarps;
+// Warps per CTA of the two-codeword kernels (their launch bounds).  Measured
+// on the decode stage, fewer registers against more warps in flight:
+//   check-regular codes of degree 6: 20 warps (96 registers): 92 ms on a general
+//     (1008, 504) code against 95 with 24 warps and 108 with 16
+//   degree 7 or 8: 16 warps (20: 4 B spilled, 0.19 -> 0.23 ms on a small job)
+//   degree 9 to 32: 24 warps: the n = 11,520 code, one pair to a CTA, 57 ms
+//     against 64 with 20 (two checks a thread instead of three); the others within 3 %
+__host__ __device__ constexpr int pair_kernel_warps(int dc, bool exact) {
+    return dc == 6 && exact ? 20 : dc <= 8 ? 16 : 24;
 }
-// warps per CTA of the importance-sampling kernel's flat form (its launch bound)
+// the multi-code kernel (24: spills, no faster)
+constexpr int kBatchWarps = 20;
+// the importance-sampling kernel's large-degree form: 18 measured faster than 16, 20 or 24 on the
+// n = 8,832 code (1,152 checks, two a thread)
 constexpr int kIsWarps = 18;
 struct BatchArgs {
     BatchItem it[kMaxBatch];
@@ -102,9 +105,10 @@ cudaError_t launch_batch(const BatchArgs &items, int n, int variant, const Launc
 // writes the per-candidate records and x* of failing candidates.  NMS
 // decoders use the two-codeword kernel where its 16-bit bias bounds hold
 // (else, or with force_scalar, the one-codeword kernel).  G / groups /
-// ctas_per_sm: 0 = automatic.
+// ctas_per_sm: 0 = automatic.  n_cand: at most this many candidates are
+// decoded (0 = not known): few candidates get wide groups.
 cudaError_t launch_decode(const DevCode &g, const DecodeParams &dp, const EnumBuffers &b, int G, int groups,
-                          int ctas_per_sm, int num_sms, int force_scalar, cudaStream_t st);
+                          int ctas_per_sm, int num_sms, int force_scalar, long long n_cand, cudaStream_t st);
 
 // Sieve (Tree / TS), classification, canonical key and hash insert of every
 // failing candidate (reads the records and x* written by the decoder).

@@ -134,7 +134,7 @@ extern "C" int decode_thresholds_noalloc(const tsx_code *code, const tsx_enum_pa
     b.queue = &b.ctr->next_cand;
     b.rec_base = 0;
     if (launch_decode(g, dp, b, params->warps_per_cta, 0, params->ctas_per_sm, code_num_sms(code),
-                      params->kernel == 1 ? 1 : 0, s) != cudaSuccess)
+                      params->kernel == 1 ? 1 : 0, n_cand, s) != cudaSuccess)
         return TSX_ECUDA;
     return TSX_OK;
 }
