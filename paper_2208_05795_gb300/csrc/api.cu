@@ -11,6 +11,7 @@
 #include <numeric>
 #include <vector>
 
+#include "banks.h"
 #include "kernels.cuh"
 
 using namespace tsx;
@@ -100,7 +101,7 @@ struct HostTables {
     int kind, n, m, E, Z = 0, n_b = 0, m_b = 0, dv_max = 1, dc_max = 1;
     std::vector<int16_t> rdeg, rs, cdeg, cs;
     std::vector<int32_t> reoff, rjz, ceoff, ciz;
-    std::vector<uint16_t> c_ptr, c_vn, v_ptr, v_edge, v_chk;
+    std::vector<uint16_t> c_ptr, c_vn, c_vnb, v_ptr, v_edge, v_chk;
     // generic adjacency for the girth search
     std::vector<std::vector<int>> vadj, cadj;
 };
@@ -193,6 +194,9 @@ int build_csr(const tsx_code_desc &d, HostTables &h) {
     if ((long long)h.dc_max * d.m > 65535) return TSX_EUNSUPPORTED;
     h.v_edge.resize(E);
     h.v_chk.resize(E);
+    bool reg6 = true;
+    for (int c = 0; c < d.m; c++) reg6 = reg6 && h.c_ptr[c + 1] - h.c_ptr[c] == 6;
+    if (reg6) h.c_vnb = bank_order(d.m, 6, h.c_vn);
     std::vector<int> fill(d.n, 0);
     for (int c = 0; c < d.m; c++)  // checks ascending -> edges of v ascending by check
         for (int e = h.c_ptr[c]; e < h.c_ptr[c + 1]; e++) {
@@ -287,7 +291,7 @@ extern "C" int load_code(const tsx_code_desc *desc, void *stream, tsx_code **out
     size_t o_rdeg = put(blob, h.rdeg), o_reoff = put(blob, h.reoff), o_rjz = put(blob, h.rjz),
            o_rs = put(blob, h.rs), o_cdeg = put(blob, h.cdeg), o_ceoff = put(blob, h.ceoff),
            o_cs = put(blob, h.cs), o_ciz = put(blob, h.ciz), o_cptr = put(blob, h.c_ptr),
-           o_cvn = put(blob, h.c_vn), o_vptr = put(blob, h.v_ptr), o_vedge = put(blob, h.v_edge),
+           o_cvn = put(blob, h.c_vn), o_cvnb = put(blob, h.c_vnb), o_vptr = put(blob, h.v_ptr), o_vedge = put(blob, h.v_edge),
            o_vchk = put(blob, h.v_chk);
     blob.resize((blob.size() + 255) & ~size_t(255));
     const int n_rep = h.kind == TSX_CODE_QC ? h.n_b : h.n;
@@ -323,6 +327,7 @@ extern "C" int load_code(const tsx_code_desc *desc, void *stream, tsx_code **out
     d.cdeg = (const int16_t *)(dev + o_cdeg); d.ceoff = (const int32_t *)(dev + o_ceoff);
     d.cs = (const int16_t *)(dev + o_cs); d.ciz = (const int32_t *)(dev + o_ciz);
     d.c_ptr = (const uint16_t *)(dev + o_cptr); d.c_vn = (const uint16_t *)(dev + o_cvn);
+    d.c_vnb = h.c_vnb.empty() ? nullptr : (const uint16_t *)(dev + o_cvnb);
     d.v_ptr = (const uint16_t *)(dev + o_vptr); d.v_edge = (const uint16_t *)(dev + o_vedge);
     d.v_chk = (const uint16_t *)(dev + o_vchk);
     d.ball_ptr = (const int64_t *)(dev + o_bptr);

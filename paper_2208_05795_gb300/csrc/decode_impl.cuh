@@ -163,7 +163,8 @@ __device__ SGraph load_tables(const DevCode &g, unsigned char *sm, bool pair = f
         s.cdeg = (const int16_t *)(sm + o.cdeg);
     } else {
         copy_bytes(sm + o.c_ptr, g.c_ptr, (g.m + 1) * 2);
-        copy_bytes(sm + o.c_vn, g.c_vn, g.E * 2);
+        // (the two-codeword kernels do not depend on the order of checks and edges)
+        copy_bytes(sm + o.c_vn, pair && g.c_vnb ? g.c_vnb : g.c_vn, g.E * 2);
         copy_bytes(sm + o.v_ptr, g.v_ptr, (g.n + 1) * 2);
         s.c_ptr = (const uint16_t *)(sm + o.c_ptr);
         s.c_vn = (const uint16_t *)(sm + o.c_vn);

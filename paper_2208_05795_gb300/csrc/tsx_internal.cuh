@@ -45,6 +45,7 @@ struct DevCode {
     // CSR tables (uint16; E < 65536)
     const uint16_t *c_ptr;   // [m+1]
     const uint16_t *c_vn;    // [E]
+    const uint16_t *c_vnb;   // [E] the rows of a code of check degree 6 in bank order (banks.h), else null
     const uint16_t *v_ptr;   // [n+1]
     const uint16_t *v_edge;  // [E] edges of v, ascending check
     const uint16_t *v_chk;   // [E] check of that edge
