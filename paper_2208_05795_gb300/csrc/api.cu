@@ -359,7 +359,7 @@ extern "C" int load_code(const tsx_code_desc *desc, void *stream, tsx_code **out
             return fail(TSX_ENOMEM);
         }
         std::vector<unsigned long long> hw((size_t)n_rep * (kCycLmax + 1));
-        if (launch_cycles(d, 3, walks, nullptr, s) != cudaSuccess ||
+        if (launch_cycles(d, 3, walks, nullptr, c->num_sms, s) != cudaSuccess ||
             cudaMemcpyAsync(hw.data(), walks, sizeof(unsigned long long) * hw.size(), cudaMemcpyDeviceToHost, s) !=
                 cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess) {
@@ -430,18 +430,23 @@ extern "C" int emd_spectrum(tsx_code *c, int32_t lmax, void *stream, tsx_emd_spe
     cudaStream_t s = (cudaStream_t)stream;
     unsigned long long *buf = nullptr;
     const size_t nw = (size_t)d.n_rep * (kCycLmax + 1), nh = (size_t)(kCycLmax + 1) * kEmdBins;
-    if (cudaMalloc(&buf, sizeof(unsigned long long) * (nw + nh)) != cudaSuccess) return TSX_ENOMEM;
+    if (cudaMallocAsync(&buf, sizeof(unsigned long long) * (nw + nh), s) != cudaSuccess) {
+        cudaGetLastError();
+        return TSX_ENOMEM;
+    }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     std::vector<unsigned long long> hw(nw), hh(nh);
     int st = TSX_OK;
+    cudaError_t le = cudaErrorUnknown;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess ||
-        cudaEventRecord(e0, s) != cudaSuccess || launch_cycles(d, lmax, buf, buf + nw, s) != cudaSuccess ||
-        cudaEventRecord(e1, s) != cudaSuccess ||
+        cudaEventRecord(e0, s) != cudaSuccess ||
+        (le = launch_cycles(d, lmax, buf, buf + nw, c->num_sms, s)) != cudaSuccess || cudaEventRecord(e1, s) != cudaSuccess ||
         cudaMemcpyAsync(hw.data(), buf, sizeof(unsigned long long) * nw, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaMemcpyAsync(hh.data(), buf + nw, sizeof(unsigned long long) * nh, cudaMemcpyDeviceToHost, s) !=
             cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
-        st = TSX_ECUDA;
+        st = le == cudaErrorMemoryAllocation ? TSX_ENOMEM : TSX_ECUDA;
+    if (st == TSX_ENOMEM) cudaGetLastError();
     if (st == TSX_OK) {
         float ms = 0.0f;
         cudaEventElapsedTime(&ms, e0, e1);
@@ -454,7 +459,7 @@ extern "C" int emd_spectrum(tsx_code *c, int32_t lmax, void *stream, tsx_emd_spe
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    cudaFree(buf);
+    cudaFreeAsync(buf, s);
     return st;
 }
 

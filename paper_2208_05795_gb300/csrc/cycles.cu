@@ -17,8 +17,18 @@
 // are twice the cycles through v.
 //
 // The EMD is the number of checks meeting exactly one variable node of the
-// walk.  One thread walks every continuation of one two-step prefix
-// (v0, c1, v1, c2, v2) with an explicit stack; lengths up to 2 kLmax.
+// walk.
+//
+// lmax <= 3 (load_code()): one thread per two-step prefix.  Longer walks are
+// searched from both ends: the last two steps v_{L-2} - c_{L-1} - v_{L-1} -
+// c_L - v0 are fixed by where they start and end, so every two-step path into
+// a representative is listed once, by its start (pairs_kernel), and a walk of
+// L nodes is a prefix of L - 2 steps and a listed path.  The search visits
+// prefixes of lmax - 2 steps instead of lmax - 1 steps and a test of every
+// closing check: on Code 1 (4 x 20, Z = 128) 4.2e6 prefixes instead of 2.3e8
+// for cycles up to length 10.
+#include <algorithm>
+
 #include "graph.cuh"
 #include "kernels.cuh"
 
@@ -26,6 +36,11 @@ namespace tsx {
 namespace {
 
 constexpr int kLmax = kCycLmax;
+
+template <int D>
+struct Depth {
+    static constexpr int value = D;
+};
 
 __device__ __forceinline__ bool has_check(const DevCode &g, int v, int c) {
     const int d = vn_degree(g, v);
@@ -83,18 +98,17 @@ __device__ int walk_reps(const int *vs, const int *cs, int L) {
 
 // walks[rep * (kLmax + 1) + l]: closed walks of l variable nodes from the
 // representative; hist2[l * kEmdBins + e]: sum of 2l / (p r) over them by EMD.
-// Thread id = (rep, t_1, p_1, ..., t_pd, p_pd): the walk's first pd steps
-// (check t of the last node, then node p of that check); the walks that
-// close within the prefix are counted by the thread whose deeper indices are
-// all 0, and the rest of the search runs from the prefix's last node.
-__global__ void __launch_bounds__(256) cycle_kernel(DevCode g, int lmax, int pd, long long n_prefix,
-                                                    unsigned long long *walks, unsigned long long *hist2) {
+// Thread id = (rep, t_1, p_1, t_2, p_2): the walk's first two steps (check t of
+// the last node, then node p of that check); the walks that close at the first
+// are counted by the thread whose deeper indices are 0.
+__global__ void __launch_bounds__(256) short_kernel(DevCode g, int lmax, long long n_prefix, unsigned long long *walks,
+                                                    unsigned long long *hist2) {
     const int dvm = g.dv_max, dcm = g.dc_max;
     for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < n_prefix;
          id += (long long)gridDim.x * blockDim.x) {
         long long x = id;
-        int tt[4], pp[4];
-        for (int lvl = pd; lvl >= 1; lvl--) {
+        int tt[3], pp[3];
+        for (int lvl = 2; lvl >= 1; lvl--) {
             pp[lvl] = (int)(x % dcm);
             x /= dcm;
             tt[lvl] = (int)(x % dvm);
@@ -103,85 +117,30 @@ __global__ void __launch_bounds__(256) cycle_kernel(DevCode g, int lmax, int pd,
         const int rep = (int)x;
         int vs[kLmax], cs[kLmax + 1];
         vs[0] = rep_vn(g, rep);
-        unsigned long long cnt[kLmax + 1] = {0, 0, 0, 0, 0, 0, 0};
-        // the walks that close at v_d through a check of v_d holding v0
-        auto closure = [&](int d) {
-            if (vs[d] == vs[0]) return;
-            const int dv = vn_degree(g, vs[d]);
-            for (int t = 0; t < dv; t++) {
-                const int c = vn_check(g, vs[d], t);
-                if (c == cs[d] || c == cs[1] || !has_check(g, vs[0], c)) continue;
-                const int L = d + 1;
-                cs[L] = c;
-                cnt[L]++;
-                if (hist2) atomicAdd(&hist2[L * kEmdBins + emd_of(g, vs, L)], (unsigned long long)(2 * L / walk_reps(vs, cs, L)));
-            }
-        };
-        int d = 0;
-        bool ok = true;
-        for (int lvl = 1; lvl <= pd && ok; lvl++) {
+        unsigned long long cnt[4] = {0, 0, 0, 0};
+        for (int lvl = 1; lvl <= 2; lvl++) {
             const int v = vs[lvl - 1];
-            if (tt[lvl] >= vn_degree(g, v)) { ok = false; break; }
+            if (tt[lvl] >= vn_degree(g, v)) break;
             const int c = vn_check(g, v, tt[lvl]);
-            if (lvl > 1 && c == cs[lvl - 1]) { ok = false; break; }
-            if (pp[lvl] >= cn_degree(g, c)) { ok = false; break; }
+            if (lvl > 1 && c == cs[lvl - 1]) break;
+            if (pp[lvl] >= cn_degree(g, c)) break;
             const int u = cn_vn(g, c, pp[lvl]);
-            if (u == v) { ok = false; break; }
+            if (u == v) break;
             cs[lvl] = c;
             vs[lvl] = u;
-            d = lvl;
-            bool zero_below = true;
-            for (int l2 = lvl + 1; l2 <= pd; l2++) zero_below = zero_below && tt[l2] == 0 && pp[l2] == 0;
-            if (zero_below) closure(lvl);
-            if (lvl >= lmax - 1) {  // no longer walk needed; deeper prefix indices count nothing
-                ok = zero_below;
-                break;
-            }
-        }
-        if (ok && d == pd && d < lmax - 1) {
-            int ti[kLmax], pi[kLmax];
-            ti[d] = 0;
-            pi[d] = 0;
-            bool enter = false;  // the prefix's last node is counted already
-            while (d >= pd) {
-                if (enter) {
-                    closure(d);
-                    if (d >= lmax - 1) {
-                        d--;
-                        enter = false;
-                        continue;
-                    }
-                    ti[d] = 0;
-                    pi[d] = 0;
-                }
-                bool pushed = false;
-                const int dv = vn_degree(g, vs[d]);
-                while (ti[d] < dv && !pushed) {
-                    const int c = vn_check(g, vs[d], ti[d]);
-                    if (c != cs[d]) {
-                        const int dc = cn_degree(g, c);
-                        while (pi[d] < dc) {
-                            const int u = cn_vn(g, c, pi[d]);
-                            pi[d]++;
-                            if (u != vs[d]) {
-                                cs[d + 1] = c;
-                                vs[d + 1] = u;
-                                pushed = true;
-                                break;
-                            }
-                        }
-                    }
-                    if (!pushed) {
-                        ti[d]++;
-                        pi[d] = 0;
-                    }
-                }
-                if (pushed) {
-                    d++;
-                    enter = true;
-                } else {
-                    d--;
-                    enter = false;
+            if (lvl == 1 && (tt[2] || pp[2])) continue;
+            // the walks that close here, through a check of u holding v0
+            if (lvl < lmax && u != vs[0]) {
+                const int dv = vn_degree(g, u);
+                for (int t = 0; t < dv; t++) {
+                    const int cl = vn_check(g, u, t);
+                    if (cl == c || cl == cs[1] || !has_check(g, vs[0], cl)) continue;
+                    const int L = lvl + 1;
+                    cs[L] = cl;
+                    cnt[L]++;
+                    if (hist2)
+                        atomicAdd(&hist2[L * kEmdBins + emd_of(g, vs, L)],
+                                  (unsigned long long)(2 * L / walk_reps(vs, cs, L)));
                 }
             }
         }
@@ -190,27 +149,331 @@ __global__ void __launch_bounds__(256) cycle_kernel(DevCode g, int lmax, int pd,
     }
 }
 
+// ---------------------------------------------------------------------------
+// lmax >= 4: prefixes and listed two-step paths
+// ---------------------------------------------------------------------------
+constexpr unsigned short kNone = 0xFFFFu;
+
+// Adjacency of the code as rows of 16-bit ids (kNone: no such edge): vadj
+// [n][dvp], dvp = dv_max filled up to a multiple of 4, and cadj [m][dc_max].
+__global__ void adj_kernel(DevCode g, int dvp, unsigned short *vadj, unsigned short *cadj) {
+    const long long nv = (long long)g.n * dvp, nc = (long long)g.m * g.dc_max;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nv + nc;
+         i += (long long)gridDim.x * blockDim.x) {
+        if (i < nv) {
+            const int v = (int)(i / dvp), t = (int)(i - (long long)v * dvp);
+            vadj[i] = t < vn_degree(g, v) ? (unsigned short)vn_check(g, v, t) : kNone;
+        } else {
+            const int c = (int)((i - nv) / g.dc_max), p = (int)((i - nv) - (long long)c * g.dc_max);
+            cadj[i - nv] = p < cn_degree(g, c) ? (unsigned short)cn_vn(g, c, p) : kNone;
+        }
+    }
+}
+
+struct Paths {
+    DevCode g;
+    int dvp;                      // row length of vadj
+    int rep0, nrep;               // representatives of this launch
+    const unsigned short *vadj, *cadj;
+    unsigned *off;                // [nrep][n + 1]: paths of rep0 + r that start at node w: ent[off[w] .. off[w + 1])
+    uint2 *ent;                   // [nrep][per]: {u | c' << 16, c} of a path w - c - u - c' - v0
+    long long per;                // room per representative
+};
+
+// One block per representative: the two-step paths w - c - u - c' - v0 with
+// u != v0, c != c', w != u (w may be v0), sorted by w: counted, scanned and
+// placed by counters in off.
+__global__ void __launch_bounds__(512) pairs_kernel(Paths a) {
+    const int r = blockIdx.x, n = a.g.n, dvp = a.dvp, dc = a.g.dc_max;
+    const int v0 = rep_vn(a.g, a.rep0 + r);
+    unsigned *off = a.off + (long long)r * (n + 1);
+    uint2 *ent = a.ent + (long long)r * a.per;
+    for (int w = threadIdx.x; w <= n; w += blockDim.x) off[w] = 0;
+    __syncthreads();
+    const int total = dvp * dc * dvp * dc;
+    auto each = [&](auto f) {
+        for (int i = threadIdx.x; i < total; i += blockDim.x) {
+            int x = i;
+            const int p2 = x % dc;
+            x /= dc;
+            const int t2 = x % dvp;
+            x /= dvp;
+            const int p1 = x % dc, t1 = x / dc;
+            const int c1 = a.vadj[(long long)v0 * dvp + t1];
+            if (c1 == kNone) continue;
+            const int u = a.cadj[(long long)c1 * dc + p1];
+            if (u == kNone || u == v0) continue;
+            const int c = a.vadj[(long long)u * dvp + t2];
+            if (c == kNone || c == c1) continue;
+            const int w = a.cadj[(long long)c * dc + p2];
+            if (w == kNone || w == u) continue;
+            f(w, u, c1, c);
+        }
+    };
+    each([&](int w, int, int, int) { atomicAdd(&off[w + 1], 1u); });
+    __syncthreads();
+    // inclusive scan of off[1 .. n] in blocks of blockDim
+    __shared__ unsigned wsum[16];
+    __shared__ unsigned carry;
+    if (threadIdx.x == 0) carry = 0;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int base = 1; base <= n; base += blockDim.x) {
+        __syncthreads();
+        const int i = base + threadIdx.x;
+        unsigned v = i <= n ? off[i] : 0u;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += y;
+        }
+        if (lane == 31) wsum[wid] = v;
+        __syncthreads();
+        unsigned add = carry;
+        for (int k = 0; k < wid; k++) add += wsum[k];
+        v += add;
+        if (i <= n) off[i] = v;
+        __syncthreads();
+        if (threadIdx.x == blockDim.x - 1) carry = v;
+    }
+    __syncthreads();
+    // off[w] is the start of w; placing advances it to the end, which is the start of w + 1: shift back
+    each([&](int w, int u, int c1, int c) {
+        ent[atomicAdd(&off[w], 1u)] = make_uint2((unsigned)u | ((unsigned)c1 << 16), (unsigned)c);
+    });
+    __syncthreads();
+    for (int base = ((n + blockDim.x) / blockDim.x) * blockDim.x; base >= 0; base -= blockDim.x) {
+        const int w = base + threadIdx.x;
+        const unsigned x = w >= 1 && w <= n ? off[w - 1] : 0u;
+        __syncthreads();
+        if (w <= n) off[w] = x;
+        __syncthreads();
+    }
+}
+
+// checks meeting exactly one of the L distinct nodes vs[0..L-1], whose rows of
+// vadj are compared pair by pair
+template <int L, int DVP>
+__device__ __forceinline__ int emd_distinct(const unsigned short *vadj, const int *vs) {
+    unsigned short ch[L][DVP];
+#pragma unroll
+    for (int x = 0; x < L; x++)
+#pragma unroll
+        for (int q = 0; q < DVP / 4; q++) *(uint2 *)&ch[x][4 * q] = __ldg((const uint2 *)(vadj + (long long)vs[x] * DVP) + q);
+    int emd = 0;
+#pragma unroll
+    for (int x = 0; x < L; x++)
+#pragma unroll
+        for (int t = 0; t < DVP; t++) {
+            bool other = ch[x][t] == kNone;
+#pragma unroll
+            for (int y = 0; y < L; y++)
+                if (y != x)
+#pragma unroll
+                    for (int q = 0; q < DVP; q++) other |= ch[y][q] == ch[x][t];
+            emd += !other;
+        }
+    return emd;
+}
+
+// One thread per prefix of PD steps (PD = LMAX - 2, or LMAX - 3 where that is
+// already enough threads); it counts the walks that close two steps after
+// its last node (and, PD = LMAX - 3, after each node one step further), and
+// those of the shorter prefixes whose deeper indices are 0.
+template <int LMAX, int PD, int DVP>
+__global__ void __launch_bounds__(256) walk_kernel(Paths a, long long n_prefix, unsigned long long *walks,
+                                                   unsigned long long *hist2) {
+    // the CTA's histogram and walk counts, low words and carries
+    __shared__ unsigned hs[(kLmax + 1) * kEmdBins], hc[(kLmax + 1) * kEmdBins], ws[kLmax + 1], wc[kLmax + 1];
+    for (int i = threadIdx.x; i < (kLmax + 1) * kEmdBins; i += blockDim.x) hs[i] = hc[i] = 0;
+    if (threadIdx.x <= kLmax) ws[threadIdx.x] = wc[threadIdx.x] = 0;
+    __syncthreads();
+    auto add = [](unsigned *lo, unsigned *hi, unsigned x) {
+        const unsigned old = atomicAdd(lo, x);
+        if (old + x < old) atomicAdd(hi, 1u);
+    };
+    const int dvp = a.dvp, dc = a.g.dc_max, n = a.g.n;
+    for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < n_prefix;
+         id += (long long)gridDim.x * blockDim.x) {
+        long long x = id;
+        int tt[PD + 1], pp[PD + 1];
+#pragma unroll
+        for (int l = PD; l >= 1; l--) {
+            pp[l] = (int)(x % dc);
+            x /= dc;
+            tt[l] = (int)(x % dvp);
+            x /= dvp;
+        }
+        const int r = (int)x;
+        const unsigned *off = a.off + (long long)r * (n + 1);
+        const uint2 *ent = a.ent + (long long)r * a.per;
+        int vs[kLmax], cs[kLmax + 1];
+        vs[0] = rep_vn(a.g, a.rep0 + r);
+        unsigned cnt[LMAX + 1] = {};
+        // the walks of D + 2 nodes that continue v_D with a listed path
+        auto close = [&](auto depth) {
+            constexpr int D = decltype(depth)::value, L = D + 2;
+            const unsigned e1 = __ldg(off + vs[D] + 1);
+            for (unsigned e = __ldg(off + vs[D]); e < e1; e++) {
+                const uint2 q = __ldg(ent + e);
+                const int u = (int)(q.x & 0xFFFFu), cl = (int)(q.x >> 16), c = (int)q.y;
+                if constexpr (D > 0)
+                    if (c == cs[D] || cl == cs[1]) continue;
+                vs[D + 1] = u;
+                cs[D + 1] = c;
+                cs[L] = cl;
+                cnt[L]++;
+                if (!hist2) continue;
+                bool distinct = true;
+#pragma unroll
+                for (int i = 0; i < L; i++)
+#pragma unroll
+                    for (int k = i + 1; k < L; k++) distinct = distinct && vs[i] != vs[k];
+                // all nodes distinct: no rotation and no reversal gives the same walk, weight 2L / (2L)
+                int emd, wt = 1;
+                bool fast = false;
+                if constexpr (DVP <= 4) fast = distinct;
+                if (fast) {
+                    if constexpr (DVP <= 4) emd = emd_distinct<L, DVP>(a.vadj, vs);
+                } else {
+                    emd = emd_of(a.g, vs, L);
+                    if (!distinct) wt = 2 * L / walk_reps(vs, cs, L);
+                }
+                add(&hs[L * kEmdBins + emd], &hc[L * kEmdBins + emd], (unsigned)wt);
+            }
+        };
+        bool ok = true;
+        // counted once: by the thread whose remaining indices are 0
+        auto zero_from = [&](int l0) {
+            bool z = true;
+#pragma unroll
+            for (int l = 1; l <= PD; l++)
+                if (l >= l0) z = z && tt[l] == 0 && pp[l] == 0;
+            return z;
+        };
+        if (zero_from(1)) close(Depth<0>{});
+#pragma unroll
+        for (int l = 1; l <= PD; l++) {
+            if (!ok) break;
+            const int c = a.vadj[(long long)vs[l - 1] * dvp + tt[l]];
+            ok = c != kNone && (l == 1 || c != cs[l > 1 ? l - 1 : 1]);
+            if (!ok) break;
+            const int u = a.cadj[(long long)c * dc + pp[l]];
+            ok = u != kNone && u != vs[l - 1];
+            if (!ok) break;
+            cs[l] = c;
+            vs[l] = u;
+            if (l == 1 && PD > 1 && zero_from(2)) close(Depth<1>{});
+            if constexpr (PD > 2)
+                if (l == 2 && zero_from(3)) close(Depth<2>{});
+            if constexpr (PD > 3)
+                if (l == 3 && zero_from(4)) close(Depth<3>{});
+        }
+        if (ok) {
+            close(Depth<PD>{});
+            if constexpr (PD < LMAX - 2) {
+                // one step further, node by node
+                for (int t = 0; t < dvp; t++) {
+                    const int c = a.vadj[(long long)vs[PD] * dvp + t];
+                    if (c == kNone || c == cs[PD]) continue;
+                    for (int p = 0; p < dc; p++) {
+                        const int u = a.cadj[(long long)c * dc + p];
+                        if (u == kNone || u == vs[PD]) continue;
+                        cs[PD + 1] = c;
+                        vs[PD + 1] = u;
+                        close(Depth<PD + 1>{});
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int L = 2; L <= LMAX; L++)
+            if (cnt[L]) add(&ws[L], &wc[L], cnt[L]);
+    }
+    __syncthreads();
+    // (walks: summed over the representatives, in the row of the launch's first)
+    if (threadIdx.x <= LMAX && (ws[threadIdx.x] || wc[threadIdx.x]))
+        atomicAdd(&walks[(long long)a.rep0 * (kLmax + 1) + threadIdx.x],
+                  ((unsigned long long)wc[threadIdx.x] << 32) + ws[threadIdx.x]);
+    if (hist2)
+        for (int i = threadIdx.x; i < (kLmax + 1) * kEmdBins; i += blockDim.x)
+            if (hs[i] || hc[i]) atomicAdd(&hist2[i], ((unsigned long long)hc[i] << 32) + hs[i]);
+}
+
+template <int LMAX, int DVP>
+cudaError_t launch_walk(const Paths &a, long long steps, unsigned long long *walks, unsigned long long *hist,
+                        int num_sms, cudaStream_t st) {
+    // prefixes of LMAX - 2 steps while they are few, else of one step less with the last step looped over
+    // (no id is decoded, and no prefix walked, for each of a check's nodes)
+    long long full = a.nrep, less = a.nrep;
+    for (int l = 0; l < LMAX - 2; l++) full *= steps;
+    for (int l = 0; l < LMAX - 3; l++) less *= steps;
+    const bool loop = less >= 32LL * 1024;
+    const long long np = loop ? less : full;
+    long long blocks = (np + 255) / 256;
+    if (blocks > (long long)num_sms * 64) blocks = (long long)num_sms * 64;
+    if (loop) walk_kernel<LMAX, LMAX - 3, DVP><<<(int)blocks, 256, 0, st>>>(a, np, walks, hist);
+    else walk_kernel<LMAX, LMAX - 2, DVP><<<(int)blocks, 256, 0, st>>>(a, np, walks, hist);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
-// Closed walks per representative and length (walks[n_rep][kLmax + 1]) and,
+// Closed walks per representative and length (walks[n_rep][kLmax + 1]; for
+// lmax > 3 only their sums over the representatives are there) and,
 // if hist is not null, the class-weighted counts per length and EMD
 // (hist[kLmax + 1][kEmdBins]); both zeroed here.
 cudaError_t launch_cycles(const DevCode &g, int lmax, unsigned long long *walks, unsigned long long *hist,
-                          cudaStream_t st) {
+                          int num_sms, cudaStream_t st) {
     if (lmax < 2 || lmax > kLmax) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(walks, 0, sizeof(unsigned long long) * g.n_rep * (kLmax + 1), st);
     if (e != cudaSuccess) return e;
     if (hist && (e = cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * (kLmax + 1) * kEmdBins, st)) !=
                     cudaSuccess)
         return e;
-    // three-step prefixes for the deep searches (more, shorter subtrees), two otherwise
-    const int pd = lmax >= 5 ? 3 : 2;
-    long long n_prefix = g.n_rep;
-    for (int l = 0; l < pd; l++) n_prefix *= (long long)g.dv_max * g.dc_max;
-    long long blocks = (n_prefix + 255) / 256;
-    if (blocks > 1 << 20) blocks = 1 << 20;
-    cycle_kernel<<<(int)blocks, 256, 0, st>>>(g, lmax, pd, n_prefix, walks, hist);
-    return cudaGetLastError();
+    if (lmax <= 3) {
+        long long n_prefix = g.n_rep;
+        for (int l = 0; l < 2; l++) n_prefix *= (long long)g.dv_max * g.dc_max;
+        long long blocks = (n_prefix + 255) / 256;
+        if (blocks > 1 << 20) blocks = 1 << 20;
+        short_kernel<<<(int)blocks, 256, 0, st>>>(g, lmax, n_prefix, walks, hist);
+        return cudaGetLastError();
+    }
+    // working memory: adjacency rows, and the listed paths of as many representatives at a time as
+    // fit about 64 MB
+    Paths a{};
+    a.g = g;
+    a.dvp = (g.dv_max + 3) / 4 * 4;
+    a.per = (long long)g.dv_max * (g.dc_max - 1) * std::max(1, g.dv_max - 1) * (g.dc_max - 1);
+    if (a.per < 1) a.per = 1;
+    const long long per_rep = 4LL * (g.n + 1) + 8 * a.per;
+    long long chunk = (64LL << 20) / per_rep;
+    if (chunk < 1) chunk = 1;
+    if (chunk > g.n_rep) chunk = g.n_rep;
+    auto r256 = [](long long x) { return (x + 255) / 256 * 256; };
+    const long long b_vadj = r256(2LL * g.n * a.dvp), b_cadj = r256(2LL * g.m * g.dc_max),
+                    b_off = r256(4LL * chunk * (g.n + 1)), b_ent = r256(8LL * chunk * a.per);
+    unsigned char *buf = nullptr;
+    if ((e = cudaMallocAsync(&buf, (size_t)(b_vadj + b_cadj + b_off + b_ent), st)) != cudaSuccess) return e;
+    a.vadj = (unsigned short *)buf;
+    a.cadj = (unsigned short *)(buf + b_vadj);
+    a.off = (unsigned *)(buf + b_vadj + b_cadj);
+    a.ent = (uint2 *)(buf + b_vadj + b_cadj + b_off);
+    const long long na = (long long)g.n * a.dvp + (long long)g.m * g.dc_max;
+    adj_kernel<<<(int)std::min<long long>((na + 255) / 256, 4096), 256, 0, st>>>(g, a.dvp, (unsigned short *)a.vadj,
+                                                                                (unsigned short *)a.cadj);
+    e = cudaGetLastError();
+    const long long steps = (long long)a.dvp * g.dc_max;
+    for (int r0 = 0; r0 < g.n_rep && e == cudaSuccess; r0 += (int)chunk) {
+        a.rep0 = r0;
+        a.nrep = (int)std::min<long long>(chunk, g.n_rep - r0);
+        pairs_kernel<<<a.nrep, 512, 0, st>>>(a);
+        if ((e = cudaGetLastError()) != cudaSuccess) break;
+        const bool d4 = a.dvp == 4;
+        if (lmax == 4) e = d4 ? launch_walk<4, 4>(a, steps, walks, hist, num_sms, st) : launch_walk<4, 16>(a, steps, walks, hist, num_sms, st);
+        else if (lmax == 5) e = d4 ? launch_walk<5, 4>(a, steps, walks, hist, num_sms, st) : launch_walk<5, 16>(a, steps, walks, hist, num_sms, st);
+        else e = d4 ? launch_walk<6, 4>(a, steps, walks, hist, num_sms, st) : launch_walk<6, 16>(a, steps, walks, hist, num_sms, st);
+    }
+    cudaFreeAsync(buf, st);
+    return e;
 }
 
 }  // namespace tsx

@@ -136,8 +136,10 @@ constexpr int kEmdBins = 128;   // EMD values per length
 // Closed walks from the representatives, per representative and number of
 // variable nodes (walks[n_rep][kCycLmax + 1]) and, with hist, per number of
 // variable nodes and EMD (hist[kCycLmax + 1][kEmdBins]); zeroed first.
+// lmax > 3: walks holds only the sums over the representatives, spread over the
+// rows; takes working memory (about 64 MB at most) from the stream's pool.
 cudaError_t launch_cycles(const DevCode &g, int lmax, unsigned long long *walks, unsigned long long *hist,
-                          cudaStream_t st);
+                          int num_sms, cudaStream_t st);
 
 // accessors of a loaded code (api.cu)
 const DevCode *code_dev(const tsx_code *c);
