@@ -94,16 +94,7 @@ bool plan(const DevCode &g, int decoder, int kind, int G, int groups, int ctas_p
         int gr = fit < max_warps ? fit : max_warps;
         if (units > 0 && (units + num_sms - 1) / num_sms < gr) gr = (int)((units + num_sms - 1) / num_sms);
         G = max_warps / gr;
-        if (kind == kLayScalar) {
-            int work = g.m < g.n ? g.m : g.n;
-            // QC passes run block by block
-            if (g.kind == TSX_CODE_QC && g.Z < work) work = g.Z;
-            int gmax = work / 32;
-            if (gmax < 1) gmax = 1;
-            if (G > gmax) G = gmax;
-        } else if (G > (g.m + 31) / 32) {  // the check pass runs over all rows at once: at most one each
-            G = (g.m + 31) / 32;
-        }
+        if (G > (g.m + 31) / 32) G = (g.m + 31) / 32;  // the check pass runs over all rows at once: at most one each
         if (G < 1) G = 1;
     }
     if (G > max_warps) G = max_warps;
@@ -154,8 +145,12 @@ cudaError_t launch_decode(const DevCode &g, const DecodeParams &dp, const EnumBu
     if (!pair && !force_scalar && pair_ok(g, dp) && g.kind == TSX_CODE_QC && dp.decoder == TSX_DEC_NMS_I16 &&
         g.dc_max > 8 && plan(g, dp.decoder, kLayPairVn, G, groups, ctas_per_sm, num_sms, &sh, pair_warps(g), units))
         return launch_nms16_vn(g, dp, b, sh, st);
-    if (!pair && !plan(g, dp.decoder, kLayScalar, G, groups, ctas_per_sm, num_sms, &sh))
+    const int sw = scalar_warps(dp.decoder == TSX_DEC_SPA_F32, g.dc_max);
+    if (!pair && !plan(g, dp.decoder, kLayScalar, G, groups, ctas_per_sm, num_sms, &sh, sw, n_cand))
         return cudaErrorInvalidConfiguration;
+    // more one-warp groups than 24 fit and have work: the 32-warp form of the sum-product kernel
+    if (!pair && sw == 24 && sh.G == 1 && sh.groups == 24)
+        plan(g, dp.decoder, kLayScalar, 1, groups, ctas_per_sm, num_sms, &sh, 32, n_cand);
     switch (dp.decoder) {
         case TSX_DEC_NMS_I16: return launch_nms16(g, dp, b, sh, pair, st);
         case TSX_DEC_NMS_I8: return launch_nms8(g, dp, b, sh, pair, st);

@@ -399,13 +399,15 @@ struct Decoder {
                 }
             }
             if (writeR) {
+                float pre = 1.0f;  // product of the edges before p, in ascending order
 #pragma unroll
                 for (int p = 0; p < DCMAX; p++) {
                     if (p < deg) {
-                        float prod = 1.0f;
+                        float prod = pre;
 #pragma unroll
-                        for (int p2 = 0; p2 < DCMAX; p2++)
-                            if (p2 < deg && p2 != p) prod = __fmul_rn(prod, t[p2]);
+                        for (int p2 = p + 1; p2 < DCMAX; p2++)
+                            if (p2 < deg) prod = __fmul_rn(prod, t[p2]);
+                        pre = __fmul_rn(pre, t[p]);
                         float rr;
                         if (fabsf(prod) >= 1.0f) rr = prod > 0.0f ? clip : -clip;
                         else rr = __fmul_rn(2.0f, spa_atanhf(prod));
@@ -994,8 +996,14 @@ __device__ __forceinline__ void scalar_run(const DevCode &g, const DecodeParams 
     }
 }
 
-template <class Dec, int DCMAX, bool QC>
-__global__ void __launch_bounds__(512, 1) enum_kernel(DevCode g, DecodeParams dp, EnumBuffers b,
+// WARPS: launch bound.  Min-sum codes here are the ones the two-codeword
+// kernels do not take; the sum-product decoder (check degree <= 8) is bound by
+// the latency of its series and divisions, one chain per check and warp, so
+// warps in flight count more than registers: on a general (1008, 504) code 13
+// groups of one warp took 113 ms for 5,000 candidates, 12 of two 67 (24 warps, 80 registers;
+// 28: 69, 32: 73); small codes, which fill 32 one-warp groups, 25.7 -> 20.4 (n = 306).
+template <class Dec, int DCMAX, bool QC, int WARPS = 16>
+__global__ void __launch_bounds__(32 * WARPS, 1) enum_kernel(DevCode g, DecodeParams dp, EnumBuffers b,
                                                     SlotLayout lay, int G) {
     extern __shared__ __align__(16) unsigned char smem[];
     const SGraph sg = load_tables(g, smem);
@@ -1094,9 +1102,14 @@ template <class Dec>
 cudaError_t launch_scalar(const DevCode &g, const DecodeParams &dp, const EnumBuffers &b, const LaunchShape &sh,
                           cudaStream_t st) {
     const bool qc = g.kind == TSX_CODE_QC;
+    if constexpr (Dec::kFloat) {
+        if (g.dc_max <= 8 && sh.G * sh.groups > 24)
+            return qc ? launch_persistent(enum_kernel<Dec, 8, true, 32>, sh, st, g, dp, b, sh.lay, sh.G)
+                      : launch_persistent(enum_kernel<Dec, 8, false, 32>, sh, st, g, dp, b, sh.lay, sh.G);
+    }
     if (g.dc_max <= 8)
-        return qc ? launch_persistent(enum_kernel<Dec, 8, true>, sh, st, g, dp, b, sh.lay, sh.G)
-                  : launch_persistent(enum_kernel<Dec, 8, false>, sh, st, g, dp, b, sh.lay, sh.G);
+        return qc ? launch_persistent(enum_kernel<Dec, 8, true, scalar_warps(Dec::kFloat, 8)>, sh, st, g, dp, b, sh.lay, sh.G)
+                  : launch_persistent(enum_kernel<Dec, 8, false, scalar_warps(Dec::kFloat, 8)>, sh, st, g, dp, b, sh.lay, sh.G);
     return qc ? launch_persistent(enum_kernel<Dec, 32, true>, sh, st, g, dp, b, sh.lay, sh.G)
               : launch_persistent(enum_kernel<Dec, 32, false>, sh, st, g, dp, b, sh.lay, sh.G);
 }

@@ -81,6 +81,8 @@ constexpr int kMaxBatch = 64;
 __host__ __device__ constexpr int pair_kernel_warps(int dc, bool exact) {
     return dc == 6 && exact ? 20 : dc <= 8 ? 16 : 24;
 }
+// the one-codeword kernel (the sum-product decoder's codes of small degree: see enum_kernel)
+__host__ __device__ constexpr int scalar_warps(bool is_float, int dc) { return is_float && dc <= 8 ? 24 : 16; }
 // the multi-code kernel (24: spills, no faster)
 constexpr int kBatchWarps = 20;
 // the importance-sampling kernel's large-degree form: 18 measured faster than 16, 20 or 24 on the
