@@ -111,6 +111,19 @@ __device__ __forceinline__ void red_add(unsigned a, unsigned v) {
     asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
+// M1 >= M2: the two largest of the values so far
+__device__ __forceinline__ void track_max(unsigned a, unsigned &M1, unsigned &M2) {
+    M2 = vmaxu2(M2, vminu2(M1, a));
+    M1 = vmaxu2(M1, a);
+}
+// two values at once: five operations instead of six (the two maxima of M2 are one
+// three-input instruction), and half as long a dependency chain
+__device__ __forceinline__ void track_max2(unsigned a, unsigned b, unsigned &M1, unsigned &M2) {
+    const unsigned hi = vmaxu2(a, b), lo = vminu2(a, b);
+    M2 = vmaxu2(vmaxu2(M2, lo), vminu2(M1, hi));
+    M1 = vmaxu2(M1, hi);
+}
+
 constexpr unsigned kBeta = 0x8000u;
 
 template <int V>
@@ -206,19 +219,6 @@ struct PairDecoder {
     }
     __device__ __forceinline__ static unsigned neg_abs(unsigned d) { return vminu2(d, (~d) + 0x00010001u); }
 
-    // M1 >= M2: the two largest na of the check so far (beta - min1, beta - min2)
-    __device__ __forceinline__ static void track(unsigned na, unsigned &M1, unsigned &M2) {
-        M2 = vmaxu2(M2, vminu2(M1, na));
-        M1 = vmaxu2(M1, na);
-    }
-    // two edges at once: five operations instead of six (the two maxima of M2 are one
-    // three-input instruction), and half as long a dependency chain
-    __device__ __forceinline__ static void track2(unsigned a, unsigned b, unsigned &M1, unsigned &M2) {
-        const unsigned hi = vmaxu2(a, b), lo = vminu2(a, b);
-        M2 = vmaxu2(vmaxu2(M2, lo), vminu2(M1, hi));
-        M1 = vmaxu2(M1, hi);
-    }
-
     // What the outputs of a check's edges share.  Edge p sends the magnitude o2 if |q_p| is min1,
     // else o1 (o = (alpha_num min) >> alpha_shift).  That is
     //   max(o2 + min1 - |q_p|, o1):
@@ -265,7 +265,7 @@ struct PairDecoder {
                 sp ^= x;
                 edge_d(x, y, q[p], na[p]);
                 sx ^= q[p];
-                track(na[p], M1, M2);
+                track_max(na[p], M1, M2);
             }
         }
         if (writeR) {
@@ -312,7 +312,7 @@ struct PairDecoder {
                 edge_d(x, y, q[p], na[p]);
                 sx ^= q[p];
             }
-            track2(na[2 * t], na[2 * t + 1], M1, M2);
+            track_max2(na[2 * t], na[2 * t + 1], M1, M2);
         }
         if (writeR) {
             const Outs o = outs(M1, M2, sx, DC);
@@ -364,10 +364,10 @@ struct PairDecoder {
                     for (int e = 0; e < W; e++) stR(a + e * rs, y[e]);
                 }
             }
-            if constexpr (W == 1) track(na[0], M1, M2);
+            if constexpr (W == 1) track_max(na[0], M1, M2);
             else
 #pragma unroll
-                for (int e = 0; e < W; e += 2) track2(na[e], na[e + 1], M1, M2);
+                for (int e = 0; e < W; e += 2) track_max2(na[e], na[e + 1], M1, M2);
         };
         int p = 0;
         unsigned a = ra;

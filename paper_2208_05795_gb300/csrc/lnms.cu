@@ -14,9 +14,13 @@
 // full iteration x = [P < 0] and the syndrome is checked (also before the
 // first).  Failure: x != 0 at the end.
 //
-// One group of G warps owns one frame: P (int8, n) and r (int8, E) in
-// shared memory; lanes take the rows of a layer, a barrier separates the
-// layers.  Frames come from a work queue: either the caller's LLRs or BPSK
+// Two frames per lane (lnms_pair_kernel): a group of G warps owns two frames,
+// every shared-memory word holds both frames' posterior or message in 16-bit
+// halves with the representation of decode_pair.cuh, lanes take the rows of a
+// layer and a barrier separates the layers; a frame that ends is replaced
+// while the other goes on.  Codes whose words do not fit a CTA's shared memory, and
+// normalizations whose products leave 16 bits, take one frame per group
+// (lnms_kernel): P (int8, n) and r (int8, E).  Frames come from a work queue: either the caller's LLRs or BPSK
 // over AWGN drawn on the device (the noise generator of the
 // importance-sampling kernel, mu = 0), the channel LLR 2 y / sigma^2 scaled,
 // rounded half away from zero and saturated to the LLR width.
@@ -25,7 +29,7 @@
 #include <cstring>
 #include <vector>
 
-#include "decode_impl.cuh"
+#include "decode_pair.cuh"
 #include "noise.cuh"
 
 namespace tsx {
@@ -45,6 +49,9 @@ struct LnmsArgs {
     unsigned long long *queue;   // work queue (frames)
     Counters *ctr;
 };
+
+// warps per CTA of the two-frame kernel (its launch bound); 16, 20 and 28 measured within 7 %
+constexpr int kLnmsWarps = 24;
 
 struct LnmsLayout {
     int tables_bytes, p_off, r_off, misc_off, slot_bytes;
@@ -196,12 +203,269 @@ __global__ void __launch_bounds__(512, 1) lnms_kernel(DevCode g, LnmsArgs a, Lnm
     }
 }
 
+// The same decoder, two frames per lane.  Per edge of two frames the passes
+// over a layer's rows take about 34 warp instructions (the one-frame form 75
+// per frame).
+__global__ void __launch_bounds__(32 * kLnmsWarps, 1) lnms_pair_kernel(DevCode g, LnmsArgs a, SlotLayout lay, int G) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const SGraph sg = load_tables(g, smem, true);
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int grp = warp / G;
+    unsigned char *slot = smem + lay.tables_bytes + grp * lay.slot_bytes;
+    Misc *misc = (Misc *)(slot + lay.misc_off);
+    Grp gp;
+    gp.G = G;
+    gp.T = 32 * G;
+    gp.gw = warp - grp * G;
+    gp.gt = gp.gw * 32 + lane;
+    gp.lane = lane;
+    gp.bar = 1 + grp;
+    gp.red = misc->red;
+    unsigned *P = (unsigned *)(slot + lay.p_off);
+    unsigned *R = (unsigned *)(slot + lay.r_off);
+    const unsigned Pa = saddr(P), Ra = saddr(R), rt0 = saddr(sg.rt);
+    const int n = g.n, Z = g.Z;
+    const unsigned Z4 = 4u * (unsigned)Z;
+    // clamps of the biased words
+    const unsigned hi = (kBeta + (unsigned)a.lim_v2c) * 0x00010001u, lo = (kBeta - (unsigned)a.lim_v2c) * 0x00010001u;
+    const unsigned limr = (unsigned)a.lim_c2v * 0x00010001u;
+    const unsigned amask = (0xFFFFu >> a.as) * 0x00010001u, BAN = kBeta * 0x00010001u * (unsigned)a.an;
+    long long my_frames = 0, my_it = 0, my_fail = 0;
+    long long f[2];
+    int k[2];
+
+    // the next frame of half hh: channel values into its half of P, zero into its half of R
+    auto load = [&](int hh) {
+        if (gp.gt == 0) misc->bcast[0] = (long long)atomicAdd(a.queue, 1ull);
+        gp.sync();
+        f[hh] = misc->bcast[0] < a.n_frames ? misc->bcast[0] : -1;
+        gp.sync();
+        k[hh] = 0;
+        uint16_t *Ph = (uint16_t *)P + hh;
+        if (f[hh] < 0) {  // an idle half decodes the all-zero word
+            for (int v = gp.gt; v < n; v += gp.T) Ph[2 * v] = (uint16_t)kBeta;
+        } else if (a.llr) {
+            const int8_t *src = a.llr + f[hh] * (long long)n;
+            if ((((uintptr_t)a.llr | (uintptr_t)n) & 3) == 0) {
+                for (int q = gp.gt; 4 * q < n; q += gp.T) {
+                    const char4 c = __ldg((const char4 *)src + q);
+                    Ph[8 * q] = (uint16_t)(kBeta + satw(c.x, a.lim_llr));
+                    Ph[8 * q + 2] = (uint16_t)(kBeta + satw(c.y, a.lim_llr));
+                    Ph[8 * q + 4] = (uint16_t)(kBeta + satw(c.z, a.lim_llr));
+                    Ph[8 * q + 6] = (uint16_t)(kBeta + satw(c.w, a.lim_llr));
+                }
+            } else {
+                for (int v = gp.gt; v < n; v += gp.T) Ph[2 * v] = (uint16_t)(kBeta + satw(src[v], a.lim_llr));
+            }
+        } else {
+            for (int q = gp.gt; 4 * q < n; q += gp.T) {
+                float gq[4];
+                normals4(a.job, (unsigned long long)(a.f0 + f[hh]), (uint32_t)q, gq);
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const int v = 4 * q + j;
+                    if (v < n) {
+                        const float y = hadd(1.0f, hmul(a.sigf, gq[j]));
+                        Ph[2 * v] = (uint16_t)(kBeta + round_half_away(hmul(y, a.cq), a.lim_llr));
+                    }
+                }
+            }
+        }
+        // (a word is (r1 << 16) + r0: the other half's message alone)
+        for (int e = gp.gt; e < g.E_odd; e += gp.T)
+            R[e] = hh == 0 ? (R[e] + 0x8000u) & 0xFFFF0000u : (unsigned)(int)(int16_t)R[e];
+    };
+    // x = [P < 0] of half hh out: weight, decision, iterations
+    auto finish = [&](int hh) {
+        int w = 0;
+        const unsigned bit = 15u + 16u * hh;
+        if (a.x_out && (((uintptr_t)a.x_out | (uintptr_t)n) & 3) == 0) {
+            unsigned *dst = (unsigned *)(a.x_out + f[hh] * (long long)n);
+            for (int q = gp.gt; 4 * q < n; q += gp.T) {
+                const uint4 p = *(const uint4 *)(P + 4 * q);
+                const unsigned x = ((~p.x >> bit) & 1u) | (((~p.y >> bit) & 1u) << 8) | (((~p.z >> bit) & 1u) << 16) |
+                                   (((~p.w >> bit) & 1u) << 24);
+                w += __popc(x);
+                dst[q] = x;
+            }
+        } else {
+            for (int v = gp.gt; v < n; v += gp.T) {
+                const unsigned x = (~P[v] >> bit) & 1u;
+                w += (int)x;
+                if (a.x_out) a.x_out[f[hh] * (long long)n + v] = (unsigned char)x;
+            }
+        }
+        w = gp.sum(w);
+        if (gp.gt == 0) {
+            a.fail[f[hh]] = w != 0;
+            if (a.iters) a.iters[f[hh]] = k[hh];
+            if (a.weight) a.weight[f[hh]] = w;
+        }
+        my_frames++;
+        my_it += k[hh];
+        my_fail += w != 0;
+    };
+    // byte offset of the p-th node of a row: column block start + (r + shift) mod Z
+    auto pos = [&](unsigned rt, int p, unsigned r4) {
+        const uint2 e = lds64(rt + 8u * (unsigned)p);
+        const unsigned t = r4 + e.y;
+        return Pa + e.x + __viaddmin_u32(t, 0u - Z4, t);
+    };
+
+    for (int e = gp.gt; e < g.E_odd; e += gp.T) R[e] = 0;
+    gp.sync();
+    load(0);
+    load(1);
+    gp.sync();
+    while (f[0] >= 0 || f[1] >= 0) {
+        // unsatisfied checks of x = [P < 0], half 0 in the low 16 bits
+        int u = 0;
+        for (int i = 0; i < g.m_b; i++) {
+            const int deg = sg.rdeg[i];
+            const unsigned rt = rt0 + 8u * (unsigned)(i * g.dc_max);
+            for (int r = gp.gt; r < Z; r += gp.T) {
+                unsigned sp = (deg & 1) ? 0x80008000u : 0u;
+                int p = 0;
+#pragma unroll 1
+                for (; p + 4 <= deg; p += 4)
+                    sp ^= lds32(pos(rt, p, 4u * r)) ^ lds32(pos(rt, p + 1, 4u * r)) ^ lds32(pos(rt, p + 2, 4u * r)) ^
+                          lds32(pos(rt, p + 3, 4u * r));
+#pragma unroll 1
+                for (; p < deg; p++) sp ^= lds32(pos(rt, p, 4u * r));
+                u += (int)((sp >> 15) & 0x00010001u);
+            }
+        }
+        u = gp.sum(u);
+        bool fresh = false;
+        for (int hh = 0; hh < 2; hh++) {
+            if (f[hh] < 0) continue;
+            const int uh = hh == 0 ? (u & 0xFFFF) : (u >> 16);
+            if (uh != 0 && k[hh] < a.K) continue;
+            finish(hh);
+            gp.sync();
+            load(hh);
+            fresh = true;
+        }
+        if (fresh) {  // u_0 of the new frame first
+            gp.sync();
+            continue;
+        }
+        for (int i = 0; i < g.m_b; i++) {
+            const int deg = sg.rdeg[i];
+            const unsigned rt = rt0 + 8u * (unsigned)(i * g.dc_max);
+            for (int r = gp.gt; r < Z; r += gp.T) {
+                const unsigned r4 = 4u * (unsigned)r;
+                const unsigned ra = Ra + 4u * (unsigned)(sg.roff[i] + r * (deg | 1));
+                unsigned sx = 0, M1 = 0, M2 = 0;  // the two largest beta - |q|
+                // q = sat(P - r), left in the message's word
+                auto first = [&](auto width, int p) {
+                    constexpr int W = decltype(width)::value;
+                    unsigned x[W], na[W];
+#pragma unroll
+                    for (int e = 0; e < W; e++) x[e] = lds32(pos(rt, p + e, r4)) - lds32(ra + 4u * (unsigned)(p + e));
+#pragma unroll
+                    for (int e = 0; e < W; e++) {
+                        x[e] = vmaxu2(vminu2(x[e], hi), lo);
+                        sx ^= x[e];
+                        na[e] = vminu2(x[e], (~x[e]) + 0x00010001u);
+                    }
+#pragma unroll
+                    for (int e = 0; e < W; e++) sts32(ra + 4u * (unsigned)(p + e), x[e]);
+                    if constexpr (W == 1) track_max(na[0], M1, M2);
+                    else
+#pragma unroll
+                        for (int e = 0; e < W; e += 2) track_max2(na[e], na[e + 1], M1, M2);
+                };
+                int p = 0;
+#pragma unroll 1
+                for (; p + 4 <= deg; p += 4) first(Int<4>{}, p);
+                if (deg & 2) {
+                    first(Int<2>{}, p);
+                    p += 2;
+                }
+                if (deg & 1) first(Int<1>{}, p);
+                // output magnitudes (edge_out of decode_pair.cuh: the saturation keeps o2 - o1 <= min2 - min1)
+                unsigned o1 = vminu2(((BAN - M1 * (unsigned)a.an) >> a.as) & amask, limr);
+                unsigned o2 = vminu2(((BAN - M2 * (unsigned)a.an) >> a.as) & amask, limr);
+                if (deg == 1) o1 = o2 = limr;
+                const unsigned S = vadd2(o2, (~M1) + 0x00010001u);
+                sx ^= ((deg - 1) & 1) ? 0x80008000u : 0u;
+                auto second = [&](auto width, int p) {
+                    constexpr int W = decltype(width)::value;
+                    unsigned po[W], x[W];
+#pragma unroll
+                    for (int e = 0; e < W; e++) {
+                        po[e] = pos(rt, p + e, r4);
+                        x[e] = lds32(ra + 4u * (unsigned)(p + e));
+                    }
+#pragma unroll
+                    for (int e = 0; e < W; e++) {
+                        const unsigned na = vminu2(x[e], (~x[e]) + 0x00010001u);
+                        const unsigned neg = spread15(sx ^ x[e]);
+                        const unsigned w = (vmaxs2(vadd2(na, S), o1) ^ neg) - neg;
+                        sts32(ra + 4u * (unsigned)(p + e), w);
+                        sts32(po[e], vmaxu2(vminu2(x[e] + w, hi), lo));
+                    }
+                };
+                p = 0;
+#pragma unroll 1
+                for (; p + 4 <= deg; p += 4) second(Int<4>{}, p);
+                if (deg & 2) {
+                    second(Int<2>{}, p);
+                    p += 2;
+                }
+                if (deg & 1) second(Int<1>{}, p);
+            }
+            gp.sync();
+        }
+        k[0]++;
+        k[1]++;
+    }
+    if (gp.gt == 0) {
+        atomicAdd(&a.ctr->decodes, (unsigned long long)my_frames);
+        atomicAdd(&a.ctr->iterations, (unsigned long long)my_it);
+        atomicAdd(&a.ctr->edge_updates, (unsigned long long)my_it * (unsigned long long)g.E);
+        atomicAdd(&a.ctr->n_fail, (unsigned long long)my_fail);
+    }
+}
+
 constexpr int kSmemCta = 226 * 1024;
 
 struct LnmsShape {
     LnmsLayout lay;
     int G, groups, smem;
 };
+
+// shape of the two-frame kernel; false: its words do not fit a CTA, or products alpha_num |q| leave 16 bits
+bool lnms_pair_shape(const DevCode &g, const LnmsArgs &a, int num_sms, LaunchShape *sh) {
+    if ((long long)a.an * a.lim_v2c > 0xFFFF) return false;
+    SlotLayout L{};
+    L.tables_bytes = al16(tab_offsets(g, true).total);
+    int x = 0;
+    L.r_off = x; x += al16(4 * g.E_odd);
+    L.p_off = x; x += al16(4 * g.n);
+    L.misc_off = x; x += al16((int)sizeof(Misc));
+    L.slot_bytes = x;
+    const int fit = (kSmemCta - L.tables_bytes) / L.slot_bytes;
+    if (fit < 1) return false;
+    // as many pairs as fit and have work, a layer's rows shared by the warps
+    const long long units = (a.n_frames + 1) / 2, per = (units + num_sms - 1) / num_sms;
+    int gr = fit < kLnmsWarps ? fit : kLnmsWarps;
+    if (per < gr) gr = (int)per;
+    int G = kLnmsWarps / gr;
+    if (G > (g.Z + 31) / 32) G = (g.Z + 31) / 32;
+    int groups = kLnmsWarps / G;
+    if (groups > fit) groups = fit;
+    if (G > 1 && groups > 15) groups = 15;  // named barriers 1..15
+    sh->lay = L;
+    sh->G = G;
+    sh->groups = groups;
+    sh->smem_bytes = L.tables_bytes + groups * L.slot_bytes;
+    sh->num_sms = num_sms;
+    sh->per_sm_req = 0;
+    return true;
+}
 
 bool lnms_shape(const DevCode &g, LnmsShape *sh) {
     sh->lay = lnms_layout(g);
@@ -234,6 +498,8 @@ cudaError_t launch_lnms_t(Kern k, const LnmsShape &sh, int num_sms, cudaStream_t
 }
 
 cudaError_t launch_lnms(const DevCode &g, const LnmsArgs &a, int num_sms, cudaStream_t st) {
+    LaunchShape ps{};
+    if (lnms_pair_shape(g, a, num_sms, &ps)) return launch_persistent(lnms_pair_kernel, ps, st, g, a, ps.lay, ps.G);
     LnmsShape sh;
     if (!lnms_shape(g, &sh)) return cudaErrorInvalidConfiguration;
     if (g.dc_max <= 8) return launch_lnms_t(lnms_kernel<8>, sh, num_sms, st, g, a);
