@@ -64,8 +64,8 @@ SlotLayout make_layout(const DevCode &g, int decoder, int kind, bool odd_rows) {
         if (rbytes < 2 * g.n) rbytes = 2 * g.n;
         L.r_off = x; x += al16(rbytes);
         L.p_off = x; x += al16(2 * g.n);
-        L.xa_off = x; x += al16(nw * 4);
-        L.xb_off = L.xa_off;
+        L.xa_off = x; x += al16(nw * 4);  // the set
+        L.xb_off = x; x += al16(nw * 4);  // what the closure adds
     }
     const bool pair = kind == kLayPair || kind == kLayPairVn;
     L.misc_off = x; x += al16((int)(pair ? sizeof(PairMisc) : sizeof(Misc)));

@@ -299,7 +299,7 @@ struct Misc {
     long long bcast[2];
     int ints[8];
     unsigned long long okd, okit;  // converged decodes of this group and their iterations
-    uint16_t seg[kMaxNb + 2];
+    uint16_t seg[kMaxNb + 2], segw[kMaxNb + 2];
 };
 
 // ---------------------------------------------------------------------------
@@ -518,43 +518,49 @@ __device__ __forceinline__ int cand_limit(const DecodeParams &dp, const EnumBuff
 // ---------------------------------------------------------------------------
 // sieving: Tree(), TS(), (a,b)
 // ---------------------------------------------------------------------------
+// Sets of variable nodes are bitmasks; a warp takes a word of 32 nodes at a
+// time and passes over empty words, so the work follows the set's size and not
+// the code's: the degrees |N(c) n S| are counted from the set's nodes (shared
+// atomics) and not from the checks' rows, and a node's column block comes from
+// a multiplication.  (Row by row, with a division by Z per neighbour, three
+// counts of every check made the ordered list's second stage
+// several times a decoding iteration per pattern.)
 template <bool QC>
 struct Sieve {
     const DevCode &g;
     const SGraph &sg;
     const Grp &gp;
 
-    __device__ __forceinline__ int vn_check_s(int v, int t) const {
+    // f(check) for every check of v
+    template <class F>
+    __device__ __forceinline__ void each_check(int v, F f) const {
         if (QC) {
-            const int j = v / g.Z, k = v - j * g.Z;
-            const int idx = j * g.dv_max + t;
-            return sg.ciz[idx] + wrapZneg(k - sg.cs[idx], g.Z);
+            const int Z = g.Z;
+            const int j = Z > 1 ? (int)__umulhi((unsigned)v, 0xFFFFFFFFu / (unsigned)Z + 1u) : v;  // v / Z, v < 2^15
+            const int k = v - j * Z, d = sg.cdeg[j], i0 = j * g.dv_max;
+            for (int t = 0; t < d; t++) f(sg.ciz[i0 + t] + wrapZneg(k - sg.cs[i0 + t], Z));
+        } else {
+            const int t1 = sg.v_ptr[v + 1];
+            for (int t = sg.v_ptr[v]; t < t1; t++) f((int)g.v_chk[t]);
         }
-        return g.v_chk[sg.v_ptr[v] + t];
     }
-    __device__ __forceinline__ int vn_deg_s(int v) const {
-        if (QC) return sg.cdeg[v / g.Z];
-        return sg.v_ptr[v + 1] - sg.v_ptr[v];
+    // f(v, word index, whether v is in S) for the group's words of S, every lane of a warp together;
+    // empty words only with ALL
+    template <bool ALL, class F>
+    __device__ __forceinline__ void each_word(const uint32_t *S, F f) const {
+        const int nw = (g.n + 31) >> 5;
+        for (int wi = gp.gw; wi < nw; wi += gp.G) {
+            const uint32_t x = S[wi];
+            if (!ALL && x == 0) continue;
+            f((wi << 5) + gp.lane, wi, (x >> gp.lane) & 1u);
+        }
     }
-    __device__ __forceinline__ static bool bit(const uint32_t *S, int v) { return (S[v >> 5] >> (v & 31)) & 1u; }
 
-    // deg[c] = |N(c) n S|
-    __device__ void count_deg(const uint32_t *S, int *deg) const {
-        for (int c = gp.gt; c < g.m; c += gp.T) {
-            int cnt = 0;
-            if (QC) {
-                const int i = c / g.Z, r = c - i * g.Z;
-                const int d = sg.rdeg[i];
-                for (int p = 0; p < d; p++) {
-                    const int idx = i * g.dc_max + p;
-                    cnt += bit(S, sg.rjz[idx] + wrapZ(r + sg.rs[idx], g.Z));
-                }
-            } else {
-                const int e0 = sg.c_ptr[c], e1 = sg.c_ptr[c + 1];
-                for (int e = e0; e < e1; e++) cnt += bit(S, sg.c_vn[e]);
-            }
-            deg[c] = cnt;
-        }
+    // deg[c] += 1 for the checks of S's nodes
+    __device__ void add_deg(const uint32_t *S, int *deg) const {
+        each_word<false>(S, [&](int v, int, bool in) {
+            if (in) each_check(v, [&](int c) { atomicAdd(&deg[c], 1); });
+        });
     }
 
     // Tree(S): delete variable nodes with fewer than two checks of degree >= 2
@@ -562,44 +568,43 @@ struct Sieve {
     __device__ void peel(uint32_t *S, int *deg) const {
         while (true) {
             int changed = 0;
-            for (int base = 0; base < g.n; base += gp.T) {
-                const int v = base + gp.gt;
+            each_word<false>(S, [&](int v, int wi, bool in) {
                 bool rm = false;
-                if (v < g.n && bit(S, v)) {
-                    const int d = vn_deg_s(v);
+                if (in) {
                     int live = 0;
-                    for (int t = 0; t < d; t++) live += deg[vn_check_s(v, t)] >= 2;
+                    each_check(v, [&](int c) { live += deg[c] >= 2; });
                     rm = live < 2;
                 }
                 const unsigned mask = __ballot_sync(0xffffffffu, rm);
-                const int wi = (base >> 5) + gp.gw;
-                if (gp.lane == 0 && mask) S[wi] &= ~mask;
-                if (rm) {
-                    const int d = vn_deg_s(v);
-                    for (int t = 0; t < d; t++) atomicSub(&deg[vn_check_s(v, t)], 1);
-                }
-                changed |= mask != 0;
-            }
-            gp.sync();
-            if (!gp.sum(changed)) break;
+                if (mask == 0) return;
+                if (gp.lane == 0) S[wi] &= ~mask;
+                if (rm) each_check(v, [&](int c) { atomicSub(&deg[c], 1); });
+                changed = 1;
+            });
+            __syncwarp();
+            if (!gp.sum(changed)) break;  // (a barrier after the warps' changes, and one after all have read)
         }
     }
 
-    // S <- S u {v not in S : at least two checks of v touch S} (deg = |N(c) n S|)
-    __device__ void closure(uint32_t *S, const int *deg) const {
-        for (int base = 0; base < g.n; base += gp.T) {
-            const int v = base + gp.gt;
+    // S <- S u {v not in S : at least two checks of v touch S} (deg = |N(c) n S|); afterwards deg
+    // counts the larger set
+    __device__ void closure(uint32_t *S, uint32_t *added, int *deg) const {
+        each_word<true>(S, [&](int v, int wi, bool in) {
             bool add = false;
-            if (v < g.n && !bit(S, v)) {
-                const int d = vn_deg_s(v);
+            if (v < g.n && !in) {
                 int k = 0;
-                for (int t = 0; t < d; t++) k += deg[vn_check_s(v, t)] >= 1;
+                each_check(v, [&](int c) { k += deg[c] >= 1; });
                 add = k >= 2;
             }
             const unsigned mask = __ballot_sync(0xffffffffu, add);
-            const int wi = (base >> 5) + gp.gw;
-            if (gp.lane == 0 && mask) S[wi] |= mask;
-        }
+            if (gp.lane == 0) added[wi] = mask;
+        });
+        gp.sync();  // every count read before any changes
+        add_deg(added, deg);
+        const int nw = (g.n + 31) >> 5;
+        for (int wi = gp.gw; wi < nw; wi += gp.G)
+            if (gp.lane == 0) S[wi] |= added[wi];
+        gp.sync();
     }
 
     __device__ int popcount(const uint32_t *S) const {
@@ -612,26 +617,29 @@ struct Sieve {
     // X = xk u I into S, and deg for it
     __device__ void load_x(uint32_t *S, const uint32_t *xk, const int *I, int nI, int *deg) const {
         const int nw = (g.n + 31) >> 5;
-        for (int w = gp.gt; w < nw; w += gp.T) S[w] = xk[w];
+        for (int w = gp.gt; w < nw; w += gp.T) {
+            uint32_t x = xk[w];
+#pragma unroll
+            for (int t = 0; t < 4; t++)
+                if (t < nI && (I[t] >> 5) == w) x |= 1u << (I[t] & 31);
+            S[w] = x;
+        }
+        for (int c = gp.gt; c < g.m; c += gp.T) deg[c] = 0;
         gp.sync();
-        if (gp.gt < nI) atomicOr(&S[I[gp.gt] >> 5], 1u << (I[gp.gt] & 31));
-        gp.sync();
-        count_deg(S, deg);
+        add_deg(S, deg);
         gp.sync();
     }
 
     // Returns the sieve used (1: S1 = Tree(X), 2: S2 = Tree(TS(X)), 0: both
     // empty); S holds T and deg[c] = |N(c) n T| on return.
-    __device__ int run(uint32_t *S, const uint32_t *xk, const int *I, int nI, int *deg, int &a) const {
+    __device__ int run(uint32_t *S, uint32_t *added, const uint32_t *xk, const int *I, int nI, int *deg,
+                       int &a) const {
         load_x(S, xk, I, nI, deg);
         peel(S, deg);
         a = popcount(S);
         if (a > 0) return 1;
         load_x(S, xk, I, nI, deg);
-        closure(S, deg);
-        gp.sync();
-        count_deg(S, deg);
-        gp.sync();
+        closure(S, added, deg);
         peel(S, deg);
         a = popcount(S);
         return a > 0 ? 2 : 0;
@@ -639,43 +647,22 @@ struct Sieve {
 
     // b = checks of odd degree in T, elementary = every check degree <= 2
     __device__ void classify(const int *deg, int &b, int &elem) const {
-        int odd = 0, big = 0;
+        int x = 0;  // odd degrees, and degrees above 2 from bit 16 up (m < 2^16; a group's sum stays below 2^31
+                    // because only their presence is counted there, once a thread)
         for (int c = gp.gt; c < g.m; c += gp.T) {
-            odd += deg[c] & 1;
-            big |= deg[c] > 2;
+            const int d = deg[c];
+            x += d & 1;
+            if (d > 2) x |= 1 << 20;
         }
-        b = gp.sum(odd);
-        elem = gp.sum(big) == 0;
+        x = gp.sum(x);
+        b = x & 0xFFFFF;
+        elem = (x >> 20) == 0;
     }
 };
 
 // ---------------------------------------------------------------------------
 // canonical key, orbit, hash and insert (warp 0 of the group)
 // ---------------------------------------------------------------------------
-struct Cursor {
-    int seg, t, w, st, c, jz;
-};
-
-__device__ __forceinline__ void cur_enter(Cursor &cu, int seg, const uint16_t *L, const uint16_t *segs,
-                                          int Z, int s) {
-    cu.seg = seg;
-    cu.st = segs[seg];
-    cu.c = segs[seg + 1] - cu.st;
-    cu.t = 0;
-    cu.jz = (L[cu.st] / Z) * Z;
-    int w = cu.c;
-    for (int x = 0; x < cu.c; x++)
-        if ((int)L[cu.st + x] - cu.jz >= Z - s) { w = x; break; }
-    cu.w = w;
-}
-__device__ __forceinline__ int cur_elem(const Cursor &cu, const uint16_t *L, int Z, int s) {
-    int idx = cu.w + cu.t;
-    if (idx >= cu.c) idx -= cu.c;
-    int k = (int)L[cu.st + idx] - cu.jz + s;
-    if (k >= Z) k -= Z;
-    return cu.jz + k;
-}
-
 // Ordered list of the set bits of S (warp 0), returns count.
 __device__ int list_bits(const uint32_t *S, int n, uint16_t *list, int lane) {
     const int nw = (n + 31) >> 5;
@@ -703,79 +690,118 @@ __device__ int list_bits(const uint32_t *S, int n, uint16_t *list, int lane) {
 
 // Canonical key (QC: smallest sorted tuple over the shifts moving a member
 // to k = 0; CSR: the sorted set) into key[], returns the orbit size.
+//
+// The tuple is smallest where its first element is: only a shift that moves a
+// member of the first column block to k = 0 makes that 0, so the candidates
+// are that block's members.  Under the shift of its member i the block's
+// members are i, i + 1, ... in order, and every further block starts at the
+// first member past the wrap, found by bisection.  (Every member a candidate,
+// and the wrap found by a scan for each member written, cost a set of a nodes
+// a^2 / 10 steps of one warp: the ordered list's sets reach a = 2,500.)
 __device__ int canon_key(const DevCode &g, const uint16_t *L, int a, const uint32_t *S, uint16_t *key,
-                         uint16_t *segs, int lane) {
+                         uint16_t *segs, uint16_t *segw, int lane) {
     if (g.kind != TSX_CODE_QC) {
         for (int i = lane; i < a; i += 32) key[i] = L[i];
         __syncwarp();
         return 1;
     }
     const int Z = g.Z;
+    const unsigned zm = Z > 1 ? 0xFFFFFFFFu / (unsigned)Z + 1u : 0u;
+    auto block = [&](int v) { return Z > 1 ? (int)__umulhi((unsigned)v, zm) : v; };  // v / Z, v < 2^15
     // segments of equal column block
     int nseg = 0;
     for (int base = 0; base < a; base += 32) {
         const int i = base + lane;
-        const bool mk = i < a && (i == 0 || L[i] / Z != L[i - 1] / Z);
+        const bool mk = i < a && (i == 0 || block(L[i]) != block(L[i - 1]));
         const unsigned mask = __ballot_sync(0xffffffffu, mk);
         if (mk) segs[nseg + __popc(mask & ((1u << lane) - 1))] = (uint16_t)i;
         nseg += __popc(mask);
     }
     if (lane == 0) segs[nseg] = (uint16_t)a;
     __syncwarp();
-    // stabilizer: shifts sigma = k(L[i]) - k(L[0]) of segment-0 members
-    // with T + sigma = T
     const int c0 = segs[1];
-    const int k0 = L[0] % Z;
+    const int k0 = (int)L[0] - block(L[0]) * Z;
+    // stabilizer: shifts sigma = k(L[i]) - k(L[0]) of segment-0 members with T + sigma = T
     int stab = 0;
     for (int base = 0; base < c0; base += 32) {
         const int i = base + lane;
         bool ok = i < c0;
         if (ok) {
-            const int sig = (int)L[i] % Z - k0;  // >= 0: same block, ascending
+            const int sig = (int)L[i] - (int)L[0];  // >= 0: same block, ascending
             for (int x = 0; x < a && ok; x++) {
                 const int v = L[x];
-                const int j = v / Z;
-                int k = v - j * Z + sig;
+                const int jz = block(v) * Z;
+                int k = v - jz + sig;
                 if (k >= Z) k -= Z;
-                const int u = j * Z + k;
+                const int u = jz + k;
                 ok = (S[u >> 5] >> (u & 31)) & 1u;
             }
         }
         stab += __popc(__ballot_sync(0xffffffffu, ok));
     }
-    // tournament over the candidate shifts s_i = -k(L[i]) mod Z
-    int best_s = (Z - k0) % Z;
-    for (int cs0 = 1; cs0 < a; cs0 += 31) {
-        int s;
-        bool active;
-        if (lane == 0) {
-            s = best_s;
-            active = true;
-        } else {
-            const int i = cs0 + lane - 1;
-            active = i < a;
-            s = active ? (Z - (int)L[i] % Z) % Z : 0;
+    // first member of segment sg at or past k = lim
+    auto past = [&](int sg, int lim) {
+        int lo = segs[sg], hi = segs[sg + 1];
+        const int v = block(L[lo]) * Z + lim;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if ((int)L[mid] >= v) hi = mid;
+            else lo = mid + 1;
         }
-        Cursor cu;
-        cur_enter(cu, 0, L, segs, Z, s);
-        for (int pos = 0; pos < a; pos++) {
-            const int e = cur_elem(cu, L, Z, s);
-            const int mn = __reduce_min_sync(0xffffffffu, active ? e : 0x7fffffff);
+        return lo;
+    };
+    // tournament over segment 0's members, 31 against the best so far
+    int best = 0;
+    for (int base = 1; base < c0; base += 31) {
+        const int i = lane == 0 ? best : base + lane - 1;
+        bool active = lane == 0 || i < c0;
+        const int ki = active ? (int)L[i] : 0;
+        bool more = true;
+        for (int t = 1, x = i; t < c0 && more; t++) {  // the gaps decide: member i + t less member i, modulo Z
+            if (++x >= c0) x -= c0;
+            int e = 0x7fffffff;
+            if (active) {
+                e = (int)L[x] - ki;
+                if (e < 0) e += Z;
+            }
+            const int mn = __reduce_min_sync(0xffffffffu, e);
             active = active && e == mn;
-            if (__popc(__ballot_sync(0xffffffffu, active)) <= 1) break;
-            if (++cu.t == cu.c && cu.seg + 1 < nseg) cur_enter(cu, cu.seg + 1, L, segs, Z, s);
+            more = __popc(__ballot_sync(0xffffffffu, active)) > 1;
+        }
+        const int s = active ? (Z - (ki - (int)L[0] + k0)) : 0;  // shift, 1 .. Z
+        for (int sg = 1; sg < nseg && more; sg++) {
+            const int st = segs[sg], c = segs[sg + 1] - st;
+            const int jz = block(L[st]) * Z;
+            int x = active ? past(sg, Z - s) : st;
+            for (int t = 0; t < c && more; t++, x++) {
+                if (x >= st + c) x -= c;
+                int e = 0x7fffffff;
+                if (active) {
+                    e = (int)L[x] - jz + s;
+                    if (e >= Z) e -= Z;
+                }
+                const int mn = __reduce_min_sync(0xffffffffu, e);
+                active = active && e == mn;
+                more = __popc(__ballot_sync(0xffffffffu, active)) > 1;
+            }
         }
         const unsigned am = __ballot_sync(0xffffffffu, active);
-        best_s = __shfl_sync(0xffffffffu, s, __ffs(am) - 1);
+        best = __shfl_sync(0xffffffffu, i, __ffs(am) - 1);
     }
-    // write the key for best_s
+    // the key under best's shift
+    const int s = Z - ((int)L[best] - (int)L[0] + k0);  // 1 .. Z
+    for (int sg = lane; sg < nseg; sg += 32) segw[sg] = (uint16_t)past(sg, Z - s);
+    __syncwarp();
+    int sg = 0;
     for (int pos = lane; pos < a; pos += 32) {
-        int seg = 0;
-        while (seg + 1 < nseg && segs[seg + 1] <= pos) seg++;
-        Cursor cu;
-        cur_enter(cu, seg, L, segs, Z, best_s);
-        cu.t = pos - cu.st;
-        key[pos] = (uint16_t)cur_elem(cu, L, Z, best_s);
+        while (segs[sg + 1] <= pos) sg++;
+        const int st = segs[sg], en = segs[sg + 1];
+        int x = segw[sg] + (pos - st);
+        if (x >= en) x -= en - st;
+        const int jz = block(L[x]) * Z;
+        int k = (int)L[x] - jz + s;
+        if (k >= Z) k -= Z;
+        key[pos] = (uint16_t)(jz + k);
     }
     __syncwarp();
     return Z / stab;
@@ -1015,7 +1041,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) enum_kernel(DevCode g, DecodePa
 // the sieve kernel: one warp per failing candidate
 // ---------------------------------------------------------------------------
 template <bool QC>
-__global__ void __launch_bounds__(512) sieve_kernel(DevCode g, EnumBuffers b, SlotLayout lay, int is_float) {
+__global__ void __launch_bounds__(512, 2) sieve_kernel(DevCode g, EnumBuffers b, SlotLayout lay, int is_float) {
     extern __shared__ __align__(16) unsigned char smem[];
     const SGraph sg = load_tables(g, smem);
     __syncthreads();
@@ -1033,7 +1059,7 @@ __global__ void __launch_bounds__(512) sieve_kernel(DevCode g, EnumBuffers b, Sl
     int *deg = (int *)(slot + lay.r_off);
     uint16_t *key = (uint16_t *)(slot + lay.r_off);
     uint16_t *L = (uint16_t *)(slot + lay.p_off);
-    uint32_t *S = (uint32_t *)(slot + lay.xa_off);
+    uint32_t *S = (uint32_t *)(slot + lay.xa_off), *added = (uint32_t *)(slot + lay.xb_off);
     Sieve<QC> sv{g, sg, gp};
 
     const long long total = (long long)b.ctr->n_cand_total;
@@ -1052,7 +1078,7 @@ __global__ void __launch_bounds__(512) sieve_kernel(DevCode g, EnumBuffers b, Sl
         const int nI = (I4.x >= 0) + (I4.y >= 0) + (I4.z >= 0) + (I4.w >= 0);
         const uint32_t *xk = b.xstar + o * (long long)b.nw;
         int a = 0;
-        const int which = sv.run(S, xk, I, nI, deg, a);
+        const int which = sv.run(S, added, xk, I, nI, deg, a);
         int flags = which;
         long long tslot = -1;
         if (which == 0) {
@@ -1063,7 +1089,7 @@ __global__ void __launch_bounds__(512) sieve_kernel(DevCode g, EnumBuffers b, Sl
             sv.classify(deg, bb, elem);
             __syncwarp();
             list_bits(S, g.n, L, lane);
-            const int orbit = canon_key(g, L, a, S, key, misc->seg, lane);
+            const int orbit = canon_key(g, L, a, S, key, misc->seg, misc->segw, lane);
             const int thr_ord = is_float ? f2ord(b.c_thr_f[o]) : b.c_thr[o];
             tslot = ts_insert(b, key, a, bb, orbit, elem | (which << 1), lane);
             if (tslot >= 0 && lane == 0) {

@@ -21,7 +21,7 @@ namespace {
 
 struct ListLayout {
     int tables_bytes;
-    int r_off, p_off, s_off, xk_off, xp_off, deg_off, l_off, key_off, seen_off, misc_off;
+    int r_off, p_off, s_off, add_off, xk_off, xp_off, deg_off, l_off, key_off, seen_off, misc_off;
     int slot_bytes;
 };
 
@@ -34,6 +34,7 @@ ListLayout list_layout(const DevCode &g, int K) {
     L.r_off = x; x += al16(nmsg * 2);
     L.p_off = x; x += al16(g.n * 2);
     L.s_off = x; x += al16(nw * 4);
+    L.add_off = x; x += al16(nw * 4);
     L.xk_off = x; x += al16(nw * 4);
     L.xp_off = x; x += al16(nw * 4);
     L.deg_off = x; x += al16(g.m * 4);
@@ -51,7 +52,7 @@ constexpr int kSmemCta = 226 * 1024;
 constexpr int kListWarps = 20;
 
 template <int DCMAX, bool QC>
-__global__ void __launch_bounds__(32 * kListWarps) list_kernel(DevCode g, DecodeParams dp, EnumBuffers b, ListLayout lay, int G,
+__global__ void __launch_bounds__(32 * kListWarps, 1) list_kernel(DevCode g, DecodeParams dp, EnumBuffers b, ListLayout lay, int G,
                                                     int kstart_req) {
     extern __shared__ __align__(16) unsigned char smem[];
     const SGraph sg = load_tables(g, smem);
@@ -71,6 +72,7 @@ __global__ void __launch_bounds__(32 * kListWarps) list_kernel(DevCode g, Decode
     int16_t *P = (int16_t *)(slot + lay.p_off);
     int16_t *R = (int16_t *)(slot + lay.r_off);
     uint32_t *S = (uint32_t *)(slot + lay.s_off);
+    uint32_t *added = (uint32_t *)(slot + lay.add_off);
     uint32_t *Xk = (uint32_t *)(slot + lay.xk_off);
     uint32_t *Xp = (uint32_t *)(slot + lay.xp_off);
     int *deg = (int *)(slot + lay.deg_off);
@@ -134,12 +136,7 @@ __global__ void __launch_bounds__(32 * kListWarps) list_kernel(DevCode g, Decode
                     for (int part = 1; part <= 2; part++) {
                         // S1: Tree(X_k); S2: Tree(TS(X_k))
                         sv.load_x(S, Xk, I, nI, deg);
-                        if (part == 2) {
-                            sv.closure(S, deg);
-                            gp.sync();
-                            sv.count_deg(S, deg);
-                            gp.sync();
-                        }
+                        if (part == 2) sv.closure(S, added, deg);
                         sv.peel(S, deg);
                         const int a = sv.popcount(S);
                         if (a == 0) continue;
@@ -147,7 +144,7 @@ __global__ void __launch_bounds__(32 * kListWarps) list_kernel(DevCode g, Decode
                         sv.classify(deg, bb, elem);
                         if (gp.gw == 0) {
                             list_bits(S, g.n, L, lane);
-                            const int orbit = canon_key(g, L, a, S, key, misc->seg, lane);
+                            const int orbit = canon_key(g, L, a, S, key, misc->seg, misc->segw, lane);
                             const long long ts = ts_insert(b, key, a, bb, orbit, elem | (part << 1), lane);
                             if (lane == 0 && ts >= 0) {
                                 const int cnt = misc->ints[0];
