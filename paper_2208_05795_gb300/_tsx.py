@@ -356,9 +356,11 @@ def enumerate_ts(code: Code, params=None, stream=None, **kw) -> TsList:
 
 
 def _arr(ptr, n, dtype):
-    if n == 0:
-        return np.zeros(0, dtype=dtype)
-    return np.ctypeslib.as_array(ptr, shape=(n,)).astype(dtype, copy=True)
+    """A copy of the n elements at ptr."""
+    out = np.empty(n, dtype=dtype)
+    if n:
+        C.memmove(out.ctypes.data, ptr, out.nbytes)
+    return out
 
 
 def ts_list_view(lst: TsList, check: bool = True, keys: bool = True) -> dict:
@@ -659,8 +661,8 @@ def emd_spectrum(code: Code, lmax: int, stream=None) -> dict:
     code)."""
     out = EmdSpectrum()
     _check(lib().emd_spectrum(code.h, int(lmax), _stream_handle(stream), C.byref(out)), "emd_spectrum")
-    walks = np.array(out.walks[:], dtype=np.int64)
-    count2l = np.array([row[:] for row in out.count2l], dtype=np.int64)
+    walks = np.array(out.walks, dtype=np.int64)
+    count2l = np.frombuffer(out.count2l, dtype=np.int64).reshape(len(out.count2l), -1).copy()
     return {"lmax": int(out.lmax), "walks": walks, "count2l": count2l, "ms": float(out.ms)}
 
 

@@ -8,7 +8,8 @@
 #include <cstdio>
 #include <cstring>
 #include <deque>
-#include <numeric>
+#include <memory>
+#include <mutex>
 #include <vector>
 
 #include "banks.h"
@@ -21,6 +22,59 @@ using namespace tsx;
         cudaError_t e__ = (x);                \
         if (e__ != cudaSuccess) return TSX_ECUDA; \
     } while (0)
+
+// ---------------------------------------------------------------------------
+// Working memory of the calls: one stream-ordered pool per device, which keeps
+// up to kPoolKeep bytes between calls (with the default pool, which gives everything
+// back at each synchronization, mapping memory again was most of a small
+// call's host time) and gives them back when the last code on the device is freed.
+// ---------------------------------------------------------------------------
+namespace {
+constexpr unsigned long long kPoolKeep = 256ull << 20;
+constexpr int kMaxDevices = 64;
+struct DevicePool {
+    cudaMemPool_t pool = nullptr;
+    bool tried = false;
+    int codes = 0;
+};
+std::mutex g_pool_mu;
+DevicePool g_pool[kMaxDevices];
+
+void pool_codes(int dev, int delta) {
+    if (dev < 0 || dev >= kMaxDevices) return;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    g_pool[dev].codes += delta;
+    if (g_pool[dev].codes == 0 && g_pool[dev].pool) cudaMemPoolTrimTo(g_pool[dev].pool, 0);
+}
+}  // namespace
+
+namespace tsx {
+cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t s) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    cudaMemPool_t pool = nullptr;
+    if (dev >= 0 && dev < kMaxDevices) {
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        DevicePool &d = g_pool[dev];
+        if (!d.tried) {
+            d.tried = true;
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            unsigned long long keep = kPoolKeep;
+            if (cudaMemPoolCreate(&d.pool, &props) != cudaSuccess ||
+                cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+                cudaGetLastError();
+                d.pool = nullptr;
+            }
+        }
+        pool = d.pool;
+    }
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+}
+}  // namespace tsx
 
 struct tsx_code {
     DevCode d{};
@@ -44,7 +98,9 @@ struct tsx_ts_list {
     long long n_rec = 0;  // record capacity
     long long cap = 0;    // hash-table slots
     long long pool_cap = 0;
-    std::vector<void *> bufs;
+    unsigned char *block = nullptr;  // every buffer of the list
+    size_t zero_bytes = 0;           // its head (counters, queue words, table tags and counts), zeroed at each run
+    size_t rec_pitch = 0, ts_pitch = 0;  // rows of the candidate records and of the compacted sets
     EnumBuffers b{};
     Counters *ctr = nullptr;
     cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // start, decode, sieve, compact, end
@@ -62,19 +118,16 @@ struct tsx_ts_list {
     long long cand_bound = 0;
     unsigned long long *d_queues = nullptr;
     int grid_sms = 0;
-    // sizing only: allocations are counted, not made
-    bool dry = false;
-    long long bytes = 0;
+    long long bytes = 0;  // device memory of the list
     // host results
-    bool oom = false;
     bool fetched = false;
     int fetch_status = TSX_OK;
     tsx_enum_stats stats{};
     std::vector<int32_t> a, b_, orbit, count, thr, flags, vars;
     std::vector<float> thr_f;
     std::vector<int64_t> var_off;
-    std::vector<int32_t> cvars, cthr, cts, cflags, cdec, cit;
-    std::vector<float> cthr_f;
+    std::vector<int32_t> cvars, crec;
+    int32_t *cts = nullptr;  // the slot row of crec
 };
 
 extern "C" const char *tsx_strerror(int s) {
@@ -396,6 +449,7 @@ extern "C" int load_code(const tsx_code_desc *desc, void *stream, tsx_code **out
     in.dv_max = h.dv_max; in.dc_max = h.dc_max; in.girth = girth; in.n_rep = n_rep;
     in.ball_total = c->ball_ptr[n_rep];
     in.device_bytes = (int64_t)blob.size() + sizeof(int32_t) * (in.ball_total + h.n);
+    pool_codes(c->device, 1);
     *out = c;
     return TSX_OK;
 }
@@ -405,6 +459,7 @@ extern "C" void free_code(tsx_code *c) {
     cudaFree((void *)c->d.ball);
     cudaFree(c->vweight);
     cudaFree(c->dev);
+    pool_codes(c->device, -1);
     delete c;
 }
 
@@ -430,7 +485,7 @@ extern "C" int emd_spectrum(tsx_code *c, int32_t lmax, void *stream, tsx_emd_spe
     cudaStream_t s = (cudaStream_t)stream;
     unsigned long long *buf = nullptr;
     const size_t nw = (size_t)d.n_rep * (kCycLmax + 1), nh = (size_t)(kCycLmax + 1) * kEmdBins;
-    if (cudaMallocAsync(&buf, sizeof(unsigned long long) * (nw + nh), s) != cudaSuccess) {
+    if (pool_alloc((void **)&buf, sizeof(unsigned long long) * (nw + nh), s) != cudaSuccess) {
         cudaGetLastError();
         return TSX_ENOMEM;
     }
@@ -540,23 +595,17 @@ static long long next_pow2(long long x) {
     return p;
 }
 
+// the next count elements of a list's block (sizing: base is null and only the bytes count)
 template <class T>
-static T *lalloc(tsx_ts_list *L, size_t count, cudaStream_t s) {
-    const size_t bytes = std::max<size_t>(1, count) * sizeof(T);
-    L->bytes += (long long)((bytes + 255) / 256 * 256);
-    if (L->dry) return nullptr;
-    void *p = nullptr;
-    if (cudaMallocAsync(&p, bytes, s) != cudaSuccess) {
-        L->oom = true;
-        return nullptr;
-    }
-    L->bufs.push_back(p);
+static T *carve(tsx_ts_list *L, unsigned char *base, size_t count) {
+    unsigned char *p = base ? base + L->bytes : nullptr;
+    L->bytes += (long long)((std::max<size_t>(1, count) * sizeof(T) + 255) / 256 * 256);
     return (T *)p;
 }
 
 static void release(tsx_ts_list *L) {
-    for (void *p : L->bufs) cudaFreeAsync(p, L->st);
-    L->bufs.clear();
+    if (L->block) cudaFreeAsync(L->block, L->st);
+    L->block = nullptr;
     for (cudaEvent_t &e : L->ev)
         if (e) {
             cudaEventDestroy(e);
@@ -610,7 +659,6 @@ static int prepare_list(tsx_code *code, const tsx_enum_params *params, cudaStrea
     if (p.list_mode && !list_fits(g, p.K)) return TSX_EUNSUPPORTED;
 
     tsx_ts_list *L = new tsx_ts_list();
-    L->dry = dry;
     L->code = code;
     L->st = s;
     L->p = p;
@@ -643,55 +691,65 @@ static int prepare_list(tsx_code *code, const tsx_enum_params *params, cudaStrea
     dp.spa_clip = p.spa_clip; dp.spa_amax = p.spa_amax;
 
     L->n_chunks = cand_chunks(raw_total);
-    L->d_raw_off = lalloc<long long>(L, n_rep + 1, s);
-    L->d_chunk_cnt = lalloc<int>(L, L->n_chunks, s);
-    L->d_chunk_off = lalloc<long long>(L, L->n_chunks + 1, s);
-    int4 *d_cands = lalloc<int4>(L, cand_bound, s);
-    L->b.cand_K = p.budget_wref > 0 ? lalloc<uint16_t>(L, cand_bound, s) : nullptr;
     L->cand_bound = cand_bound;
-    L->d_cyc_cnt = cycles ? lalloc<int>(L, n_rep, s) : nullptr;
-    L->d_cyc_off = cycles ? lalloc<long long>(L, n_rep + 1, s) : nullptr;
     EnumBuffers &b = L->b;
-    b.cands = d_cands;
     b.cand_begin = p.cand_begin;
     b.cand_end = p.cand_end;
     b.record = 1;
-    const long long nr = n_rec;  // the sieve reads the records, so they are always kept
     b.nw = (g.n + 31) / 32;
-    b.xstar = lalloc<uint32_t>(L, (size_t)n_rec * b.nw, s);
-    b.c_thr = lalloc<int>(L, nr, s);
-    b.c_thr_f = lalloc<float>(L, nr, s);
-    b.c_slot = lalloc<int>(L, nr, s);
-    b.c_flags = lalloc<int>(L, nr, s);
-    b.c_decodes = lalloc<int>(L, nr, s);
-    b.c_iters = lalloc<int>(L, nr, s);
-    b.tags = lalloc<unsigned long long>(L, L->cap, s);
-    b.t_thr = lalloc<int>(L, L->cap, s);
-    b.t_count = lalloc<int>(L, L->cap, s);
     b.cap_mask = (unsigned long long)(L->cap - 1);
-    b.pool = lalloc<int>(L, L->pool_cap + 1, s);
     b.pool_cap = (unsigned long long)L->pool_cap;
-    L->ctr = lalloc<Counters>(L, 1, s);
-    b.ctr = L->ctr;
-    b.queue = L->ctr ? &L->ctr->next_cand : nullptr;
     b.rec_base = p.cand_begin;
+    const long long nr = n_rec;  // the sieve reads the records, so they are always kept
     // distinct sets: at most one per failing candidate, or (list mode) as many as the table holds
     const long long ts_cap = p.list_mode ? L->cap : std::min<long long>(L->cap, std::max<long long>(n_rec, 1));
-    L->ts_off = lalloc<int>(L, ts_cap, s);
-    L->ts_count = lalloc<int>(L, ts_cap, s);
-    L->ts_thr = lalloc<int>(L, ts_cap, s);
-    L->slot_map = lalloc<int>(L, L->cap, s);
-    if (L->n_dchunks) L->d_queues = lalloc<unsigned long long>(L, L->n_dchunks, s);
+    auto layout = [&](unsigned char *base) {
+        L->bytes = 0;
+        L->ctr = carve<Counters>(L, base, 1);
+        if (L->n_dchunks) L->d_queues = carve<unsigned long long>(L, base, L->n_dchunks);
+        b.tags = carve<unsigned long long>(L, base, L->cap);
+        b.t_count = carve<int>(L, base, L->cap);
+        L->zero_bytes = (size_t)L->bytes;
+        b.t_thr = carve<int>(L, base, L->cap);
+        L->d_raw_off = carve<long long>(L, base, n_rep + 1);
+        L->d_chunk_cnt = carve<int>(L, base, L->n_chunks);
+        L->d_chunk_off = carve<long long>(L, base, L->n_chunks + 1);
+        b.cands = carve<int4>(L, base, cand_bound);
+        b.cand_K = p.budget_wref > 0 ? carve<uint16_t>(L, base, cand_bound) : nullptr;
+        L->d_cyc_cnt = cycles ? carve<int>(L, base, n_rep) : nullptr;
+        L->d_cyc_off = cycles ? carve<long long>(L, base, n_rep + 1) : nullptr;
+        b.xstar = carve<uint32_t>(L, base, (size_t)n_rec * b.nw);
+        // the records, one row each (do_fetch copies them together)
+        const long long r0 = L->bytes;
+        b.c_thr = carve<int>(L, base, nr);
+        L->rec_pitch = (size_t)(L->bytes - r0);
+        b.c_thr_f = carve<float>(L, base, nr);
+        b.c_slot = carve<int>(L, base, nr);
+        b.c_flags = carve<int>(L, base, nr);
+        b.c_decodes = carve<int>(L, base, nr);
+        b.c_iters = carve<int>(L, base, nr);
+        b.pool = carve<int>(L, base, L->pool_cap + 1);
+        const long long t0 = L->bytes;
+        L->ts_off = carve<int>(L, base, ts_cap);
+        L->ts_pitch = (size_t)(L->bytes - t0);
+        L->ts_count = carve<int>(L, base, ts_cap);
+        L->ts_thr = carve<int>(L, base, ts_cap);
+        L->slot_map = carve<int>(L, base, L->cap);
+        b.ctr = L->ctr;
+        b.queue = L->ctr ? &L->ctr->next_cand : nullptr;
+    };
+    layout(nullptr);
     if (dry) {
         *out = L;
         return TSX_OK;
     }
-    if (L->oom) {
+    if (pool_alloc((void **)&L->block, (size_t)L->bytes, s) != cudaSuccess) {
         cudaGetLastError();
-        release(L);
+        L->block = nullptr;
         delete L;
         return TSX_ENOMEM;
     }
+    layout(L->block);
     auto bail = [&](int code_) { release(L); delete L; return code_; };
     if (events)
         for (cudaEvent_t &e : L->ev)
@@ -715,12 +773,8 @@ static int enqueue_front(tsx_ts_list *L, cudaStream_t s) {
     L->st = s;
     L->fetched = false;
     if (record(L, 0, s) != TSX_OK) return TSX_ECUDA;
-    if (cudaMemsetAsync(L->ctr, 0, sizeof(Counters), s) != cudaSuccess ||
-        cudaMemsetAsync(b.tags, 0, sizeof(unsigned long long) * L->cap, s) != cudaSuccess ||
-        cudaMemsetAsync(b.t_count, 0, sizeof(int) * L->cap, s) != cudaSuccess ||
-        cudaMemsetAsync(b.t_thr, 0x7f, sizeof(int) * L->cap, s) != cudaSuccess ||
-        (L->d_queues &&
-         cudaMemsetAsync(L->d_queues, 0, sizeof(unsigned long long) * L->n_dchunks, s) != cudaSuccess))
+    if (cudaMemsetAsync(L->block, 0, L->zero_bytes, s) != cudaSuccess ||
+        cudaMemsetAsync(b.t_thr, 0x7f, sizeof(int) * L->cap, s) != cudaSuccess)
         return TSX_ECUDA;
     CandArgs ca{};
     ca.code = g;
@@ -1027,36 +1081,45 @@ static int do_fetch(tsx_ts_list *L) {
     if (st != TSX_OK) return st;
     fill_stats(L, c, L->stats);
     const long long nts = c.n_ts;
-    std::vector<int> off(nts), cnt(nts), thr(nts);
     const unsigned long long pool_used = c.pool_top + 1 < (unsigned long long)L->pool_cap + 1
                                              ? c.pool_top + 1
                                              : (unsigned long long)L->pool_cap + 1;
-    std::vector<int> pool(pool_used);
+    // (uninitialized: every word is copied over)
+    std::unique_ptr<int[]> ts3(new int[3 * nts + 1]), pool(new int[pool_used]);
+    const int *off = ts3.get(), *cnt = off + nts, *thr = cnt + nts;
     if (nts) {
-        CK(cudaMemcpy(off.data(), L->ts_off, sizeof(int) * nts, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(cnt.data(), L->ts_count, sizeof(int) * nts, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(thr.data(), L->ts_thr, sizeof(int) * nts, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(pool.data(), L->b.pool, sizeof(int) * pool_used, cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy2D(ts3.get(), sizeof(int) * nts, L->ts_off, L->ts_pitch, sizeof(int) * nts, 3,
+                        cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy(pool.get(), L->b.pool, sizeof(int) * pool_used, cudaMemcpyDeviceToHost));
     }
-    // sort by (a, b, key)
-    std::vector<int> perm(nts);
-    std::iota(perm.begin(), perm.end(), 0);
-    auto less = [&](int x, int y) {
-        const int *px = &pool[off[x]], *py = &pool[off[y]];
-        if (px[0] != py[0]) return px[0] < py[0];
-        if (px[1] != py[1]) return px[1] < py[1];
-        return std::lexicographical_compare(px + kPoolHdr, px + kPoolHdr + px[0], py + kPoolHdr, py + kPoolHdr + py[0]);
+    // sort by (a, b, key): by a, b and the first two nodes in one word, and where that ties by the rest
+    struct Item {
+        unsigned long long k;
+        int x;
     };
-    std::sort(perm.begin(), perm.end(), less);
+    std::vector<Item> items(nts);
+    long long n_vars = 0;
+    for (long long i = 0; i < nts; i++) {
+        const int *px = &pool[off[i]];
+        n_vars += px[0];
+        items[i].k = ((unsigned long long)px[0] << 48) | ((unsigned long long)px[1] << 32) |
+                     ((unsigned long long)px[kPoolHdr] << 16) | (px[0] > 1 ? (unsigned long long)px[kPoolHdr + 1] : 0ull);
+        items[i].x = (int)i;
+    }
+    std::sort(items.begin(), items.end(), [&](const Item &l, const Item &r) {
+        if (l.k != r.k) return l.k < r.k;
+        const int *px = &pool[off[l.x]], *py = &pool[off[r.x]];
+        return std::lexicographical_compare(px + kPoolHdr, px + kPoolHdr + px[0], py + kPoolHdr, py + kPoolHdr + py[0]);
+    });
     std::vector<int> rank(nts);
-    for (long long i = 0; i < nts; i++) rank[perm[i]] = (int)i;
+    for (long long i = 0; i < nts; i++) rank[items[i].x] = (int)i;
     const bool spa = L->p.decoder == TSX_DEC_SPA_F32;
     L->a.resize(nts); L->b_.resize(nts); L->orbit.resize(nts); L->count.resize(nts);
     L->thr.resize(nts); L->thr_f.resize(nts); L->flags.resize(nts); L->var_off.resize(nts + 1);
-    L->vars.clear();
+    L->vars.resize(n_vars);
     long long vo = 0;
     for (long long i = 0; i < nts; i++) {
-        const int x = perm[i];
+        const int x = items[i].x;
         const int *px = &pool[off[x]];
         L->a[i] = px[0]; L->b_[i] = px[1]; L->orbit[i] = px[2]; L->flags[i] = px[3];
         L->count[i] = cnt[x];
@@ -1070,21 +1133,18 @@ static int do_fetch(tsx_ts_list *L) {
             L->thr_f[i] = -1.0f;
         }
         L->var_off[i] = vo;
-        L->vars.insert(L->vars.end(), px + kPoolHdr, px + kPoolHdr + px[0]);
+        memcpy(&L->vars[vo], px + kPoolHdr, sizeof(int) * px[0]);
         vo += px[0];
     }
     L->var_off[nts] = vo;
     const long long ncand = L->p.record_candidates ? std::min<long long>(L->stats.n_cand, L->n_rec) : 0;
-    L->cvars.resize(4 * ncand); L->cthr.resize(ncand); L->cthr_f.resize(ncand); L->cts.resize(ncand);
-    L->cflags.resize(ncand); L->cdec.resize(ncand); L->cit.resize(ncand);
+    L->cvars.resize(4 * ncand);
+    L->crec.resize(6 * ncand);  // rows: thr, thr_f, slot, flags, decodes, iterations
+    L->cts = L->crec.data() + 2 * ncand;
     if (ncand) {
         CK(cudaMemcpy(L->cvars.data(), L->b.cands + L->p.cand_begin, sizeof(int4) * ncand, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(L->cthr.data(), L->b.c_thr, sizeof(int) * ncand, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(L->cthr_f.data(), L->b.c_thr_f, sizeof(float) * ncand, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(L->cts.data(), L->b.c_slot, sizeof(int) * ncand, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(L->cflags.data(), L->b.c_flags, sizeof(int) * ncand, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(L->cdec.data(), L->b.c_decodes, sizeof(int) * ncand, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(L->cit.data(), L->b.c_iters, sizeof(int) * ncand, cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy2D(L->crec.data(), sizeof(int) * ncand, L->b.c_thr, L->rec_pitch, sizeof(int) * ncand, 6,
+                        cudaMemcpyDeviceToHost));
         for (long long i = 0; i < ncand; i++)
             if (L->cts[i] >= 0) L->cts[i] = rank[L->cts[i]];
     }
@@ -1104,10 +1164,12 @@ extern "C" int ts_list_view(tsx_ts_list *L, tsx_ts_view *v) {
     v->a = L->a.data(); v->b = L->b_.data(); v->orbit = L->orbit.data(); v->count = L->count.data();
     v->thr = L->thr.data(); v->flags = L->flags.data(); v->thr_f = L->thr_f.data();
     v->var_off = L->var_off.data(); v->vars = L->vars.data();
-    v->n_cand = (int64_t)L->cthr.size();
-    v->cand_vars = L->cvars.data(); v->cand_thr = L->cthr.data(); v->cand_ts = L->cts.data();
-    v->cand_flags = L->cflags.data(); v->cand_decodes = L->cdec.data(); v->cand_iters = L->cit.data();
-    v->cand_thr_f = L->cthr_f.data();
+    const int64_t nc = (int64_t)L->crec.size() / 6;
+    const int32_t *rec = L->crec.data();
+    v->n_cand = nc;
+    v->cand_vars = L->cvars.data(); v->cand_thr = rec; v->cand_thr_f = (const float *)(rec + nc);
+    v->cand_ts = rec + 2 * nc; v->cand_flags = rec + 3 * nc; v->cand_decodes = rec + 4 * nc;
+    v->cand_iters = rec + 5 * nc;
     return L->fetch_status;
 }
 

@@ -452,7 +452,7 @@ cudaError_t launch_cycles(const DevCode &g, int lmax, unsigned long long *walks,
     const long long b_vadj = r256(2LL * g.n * a.dvp), b_cadj = r256(2LL * g.m * g.dc_max),
                     b_off = r256(4LL * chunk * (g.n + 1)), b_ent = r256(8LL * chunk * a.per);
     unsigned char *buf = nullptr;
-    if ((e = cudaMallocAsync(&buf, (size_t)(b_vadj + b_cadj + b_off + b_ent), st)) != cudaSuccess) return e;
+    if ((e = pool_alloc((void **)&buf, (size_t)(b_vadj + b_cadj + b_off + b_ent), st)) != cudaSuccess) return e;
     a.vadj = (unsigned short *)buf;
     a.cadj = (unsigned short *)(buf + b_vadj);
     a.off = (unsigned *)(buf + b_vadj + b_cadj);

@@ -340,7 +340,7 @@ int is_job_start(tsx_code *code, const int32_t *ts_vars, int32_t a, const tsx_is
     J->grid_sms = grid_sms > 0 ? std::min(grid_sms, code_num_sms(code)) : code_num_sms(code);
     J->sh.num_sms = J->grid_sms;
     void *blk = nullptr;
-    if (cudaMallocAsync(&blk, J->total, s) != cudaSuccess) {
+    if (pool_alloc(&blk, J->total, s) != cudaSuccess) {
         cudaGetLastError();
         delete J;
         return TSX_ENOMEM;

@@ -143,6 +143,9 @@ constexpr int kEmdBins = 128;   // EMD values per length
 cudaError_t launch_cycles(const DevCode &g, int lmax, unsigned long long *walks, unsigned long long *hist,
                           int num_sms, cudaStream_t st);
 
+// device working memory from the library's pool on the current device (api.cu); freed with cudaFreeAsync
+cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t s);
+
 // accessors of a loaded code (api.cu)
 const DevCode *code_dev(const tsx_code *c);
 int code_num_sms(const tsx_code *c);

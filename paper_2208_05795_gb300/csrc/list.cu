@@ -47,9 +47,9 @@ ListLayout list_layout(const DevCode &g, int K) {
 }
 
 constexpr int kSmemCta = 226 * 1024;
-// up to 20 warps a CTA: the second stage is latency and barrier bound, and
-// one group more than 16 warps allow fits the shared memory of the QC codes
-constexpr int kListWarps = 20;
+// 24 warps a CTA, groups of 1 to 6: the second stage is latency and barrier
+// bound (2640-node code, 3,000 candidates: 18.0 ms; 20 warps in groups of up to 4: 19.4)
+constexpr int kListWarps = 24;
 
 template <int DCMAX, bool QC>
 __global__ void __launch_bounds__(32 * kListWarps, 1) list_kernel(DevCode g, DecodeParams dp, EnumBuffers b, ListLayout lay, int G,
@@ -191,9 +191,9 @@ bool list_shape(const DevCode &g, int K, ListShape *sh) {
     const int fit = (kSmemCta - sh->lay.tables_bytes) / sh->lay.slot_bytes;
     if (fit < 1) return false;
     int work = g.m < g.n ? g.m : g.n;
-    int G = work / 256;
+    int G = work / 128;
     if (G < 1) G = 1;
-    if (G > 4) G = 4;
+    if (G > 6) G = 6;
     int groups = kListWarps / G;
     if (groups > fit) groups = fit;
     if (G > 1 && groups > 15) groups = 15;

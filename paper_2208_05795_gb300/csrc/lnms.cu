@@ -567,7 +567,7 @@ extern "C" int lnms_decode(tsx_code *code, const tsx_lnms_params *p, const int8_
     if (!llr || !fail) return TSX_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     Counters *ctr = nullptr;
-    if (cudaMallocAsync(&ctr, sizeof(Counters), s) != cudaSuccess) return TSX_ENOMEM;
+    if (pool_alloc((void **)&ctr, sizeof(Counters), s) != cudaSuccess) return TSX_ENOMEM;
     LnmsArgs a{};
     fill_args(p, a);
     a.llr = llr;

@@ -34,6 +34,8 @@ def _check(code, lmax, starts):
 @pytest.mark.parametrize("name", sorted(CODES))
 def test_spectrum_edges(name, lmax):
     code = CODES[name]()
+    if lmax == 6 and name in ("z3_dv6", "csr_uneven"):
+        pytest.skip("minutes of the oracle's time; the same code paths as lmax = 5 and the other codes")
     starts = range(0, code.n, code.Z) if code.kind == "qc" else range(code.n)
     _check(code, lmax, list(starts))
 
