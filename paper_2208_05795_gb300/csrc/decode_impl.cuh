@@ -244,8 +244,10 @@ __device__ __forceinline__ float spa_expm1_pos(float x) {
     p = hadd(hmul(p, r), 0.5f);
     p = hadd(hmul(p, r), 1.0f);
     p = hmul(p, r);
-    if (k == 0.0f) return p;
-    return hsub(ldexpf(hadd(p, 1.0f), (int)k), 1.0f);
+    // 2^k in two factors, both normal (k >= 0; from 252 on the result is infinite with any larger k too)
+    const int ki = min((int)k, 252), kh = ki >> 1;
+    const float f = hmul(hmul(hadd(p, 1.0f), __int_as_float((kh + 127) << 23)), __int_as_float((ki - kh + 127) << 23));
+    return k == 0.0f ? p : hsub(f, 1.0f);
 }
 
 __device__ __forceinline__ float spa_tanhf(float y) {
@@ -272,8 +274,10 @@ __device__ __forceinline__ float spa_atanhf(float p) {
         r = hmul(q, a);
     } else {
         const float t = hdiv(hadd(1.0f, a), hsub(1.0f, a));
-        int e;
-        float m = frexpf(t, &e);
+        // t = m 2^e with m in [1/2, 1): t >= 5/3 is normal and finite (a <= 1 - 2^-24)
+        const int tb = __float_as_int(t);
+        int e = (tb >> 23) - 126;
+        float m = __int_as_float((tb & 0x7FFFFF) | 0x3F000000);
         if (m < 0x1.6a09e6p-1f) {
             m = hadd(m, m);
             e = e - 1;
@@ -288,7 +292,7 @@ __device__ __forceinline__ float spa_atanhf(float p) {
         q = hadd(hmul(q, s2), 0x1.555556p-2f);
         q = hadd(hmul(q, s2), 1.0f);
         const float lg = hadd(hmul((float)e, 0x1.62e43p-1f), hmul(hadd(s, s), q));
-        r = hmul(0.5f, lg);
+        r = a < 1.0f ? hmul(0.5f, lg) : a;  // (a NaN stays one)
     }
     return p < 0.0f ? -r : r;
 }
@@ -384,35 +388,32 @@ struct Decoder {
             }
             return par < 0;
         } else {
+            // Rolled loops, each edge's tanh in its message's place until the outputs take it: the
+            // series are in the code once each (unrolled over the edges, with the tanhs in
+            // registers, the loop missed the instruction cache).  The products over the other
+            // edges are taken in ascending order: the edges before p as a running product,
+            // the ones after it one by one.
             const float clip = dp.spa_clip;
-            float t[DCMAX];
             int par = 0;
-#pragma unroll
-            for (int p = 0; p < DCMAX; p++) {
-                if (p < deg) {
-                    const int v = nb(p);
-                    const float Pv = (float)P[v];
-                    const float ro = first ? 0.0f : (float)R[e0 + p * estride];
-                    par ^= Pv < 0.0f;
-                    const float q = clampf_(__fsub_rn(Pv, ro), -clip, clip);
-                    t[p] = spa_tanhf(__fmul_rn(q, 0.5f));
-                }
+#pragma unroll 1
+            for (int p = 0; p < deg; p++) {
+                const float Pv = (float)P[nb(p)];
+                const float ro = first ? 0.0f : (float)R[e0 + p * estride];
+                par ^= Pv < 0.0f;
+                if (writeR) R[e0 + p * estride] = (msg)spa_tanhf(__fmul_rn(clampf_(__fsub_rn(Pv, ro), -clip, clip), 0.5f));
             }
             if (writeR) {
-                float pre = 1.0f;  // product of the edges before p, in ascending order
-#pragma unroll
-                for (int p = 0; p < DCMAX; p++) {
-                    if (p < deg) {
-                        float prod = pre;
-#pragma unroll
-                        for (int p2 = p + 1; p2 < DCMAX; p2++)
-                            if (p2 < deg) prod = __fmul_rn(prod, t[p2]);
-                        pre = __fmul_rn(pre, t[p]);
-                        float rr;
-                        if (fabsf(prod) >= 1.0f) rr = prod > 0.0f ? clip : -clip;
-                        else rr = __fmul_rn(2.0f, spa_atanhf(prod));
-                        R[e0 + p * estride] = (msg)clampf_(rr, -clip, clip);
-                    }
+                float pre = 1.0f;
+#pragma unroll 1
+                for (int p = 0; p < deg; p++) {
+                    float prod = pre;
+#pragma unroll 4
+                    for (int p2 = p + 1; p2 < deg; p2++) prod = __fmul_rn(prod, (float)R[e0 + p2 * estride]);
+                    pre = __fmul_rn(pre, (float)R[e0 + p * estride]);
+                    float rr;
+                    if (fabsf(prod) >= 1.0f) rr = prod > 0.0f ? clip : -clip;
+                    else rr = __fmul_rn(2.0f, spa_atanhf(prod));
+                    R[e0 + p * estride] = (msg)clampf_(rr, -clip, clip);
                 }
             }
             return par;
@@ -1024,10 +1025,11 @@ __device__ __forceinline__ void scalar_run(const DevCode &g, const DecodeParams 
 
 // WARPS: launch bound.  Min-sum codes here are the ones the two-codeword
 // kernels do not take; the sum-product decoder (check degree <= 8) is bound by
-// the latency of its series and divisions, one chain per check and warp, so
-// warps in flight count more than registers: on a general (1008, 504) code 13
-// groups of one warp took 113 ms for 5,000 candidates, 12 of two 67 (24 warps, 80 registers;
-// 28: 69, 32: 73); small codes, which fill 32 one-warp groups, 25.7 -> 20.4 (n = 306).
+// issue and the latency of its series and divisions, one chain per check and
+// warp, so warps in flight count more than registers: on a general (1008, 504)
+// code, 5,000 candidates, 12 groups of two warps (24 warps, 80 registers) take 56 ms,
+// 13 of one (16 or 20 warps) 96, 28 warps 57; small codes fill 32 one-warp
+// groups (n = 306: 17.9 ms; 24 warps 22).  Before: 113 and 25.7.
 template <class Dec, int DCMAX, bool QC, int WARPS = 16>
 __global__ void __launch_bounds__(32 * WARPS, 1) enum_kernel(DevCode g, DecodeParams dp, EnumBuffers b,
                                                     SlotLayout lay, int G) {
