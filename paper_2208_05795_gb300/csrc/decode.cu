@@ -68,7 +68,7 @@ SlotLayout make_layout(const DevCode &g, int decoder, int kind, bool odd_rows) {
         L.xb_off = x; x += al16(nw * 4);  // what the closure adds
     }
     const bool pair = kind == kLayPair || kind == kLayPairVn;
-    L.misc_off = x; x += al16((int)(pair ? sizeof(PairMisc) : sizeof(Misc)));
+    L.misc_off = x; x += al16((int)(pair ? sizeof(PairMisc) : kind == kLayIs ? kIsMiscBytes : sizeof(Misc)));
     L.slot_bytes = x;
     return L;
 }

@@ -22,6 +22,15 @@
 namespace tsx {
 namespace {
 
+// the group's shared scratch: the noise on the trapping set's nodes of each half's sample, where
+// the set has at most kTsNoise nodes
+constexpr int kTsNoise = 64;
+struct IsMisc : Misc {
+    long long next[2][2];  // [half][turn]: the sample drawn ahead (two places: one is written while the other is read)
+    float noise[2][kTsNoise];
+};
+static_assert(sizeof(IsMisc) <= kIsMiscBytes, "room of the sampling kernel's scratch");
+
 struct IsArgs {
     unsigned long long job, s0;
     long long nsamp;
@@ -50,7 +59,7 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kern
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int grp = warp / G;
     unsigned char *slot = smem + lay.tables_bytes + grp * lay.slot_bytes;
-    Misc *misc = (Misc *)(slot + lay.misc_off);
+    IsMisc *misc = (IsMisc *)(slot + lay.misc_off);
     Grp gp;
     gp.G = G;
     gp.T = 32 * G;
@@ -77,15 +86,19 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kern
     int k[2], first[2];
     int pcur = 0;
 
+    // Sample hh's index was drawn ahead by thread 0, which draws the one after it here and stores it
+    // once the channel values are made: the queue's latency is not waited for.
+    unsigned long long next = 0;
+    int turn[2] = {0, 0};
     auto fetch = [&](int hh) {
-        if (gp.gt == 0) misc->bcast[0] = (long long)atomicAdd(ia.queue, 1ull);
-        gp.sync();
-        const long long i = misc->bcast[0];
-        gp.sync();
+        const long long i = misc->next[hh][turn[hh]];
+        turn[hh] ^= 1;
         sidx[hh] = i < ia.nsamp ? i : -1;
         k[hh] = 0;
         first[hh] = 1;
+        if (gp.gt == 0 && sidx[hh] >= 0) next = atomicAdd(ia.queue, 1ull);
     };
+    const bool keep_noise = ia.a <= kTsNoise;
     // channel values of sample sidx[hh] into half hh of L2 (accumulator
     // start) and of the current posteriors (P = L); an idle half gets L = 0
     auto generate = [&](int hh, unsigned *Pc) {
@@ -93,6 +106,7 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kern
         for (int q = gp.gt; 4 * q < g.n; q += gp.T) {
             float gq[4];
             if (sidx[hh] >= 0) normals4(ia.job, s, (uint32_t)q, gq);
+            const unsigned tm = (Tm[q >> 3] >> ((4 * q) & 31)) & 15u;  // the quad's nodes in the trapping set
 #pragma unroll
             for (int j = 0; j < 4; j++) {
                 const int v = 4 * q + j;
@@ -101,7 +115,12 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kern
                 if (sidx[hh] >= 0) {
                     const float n = hmul(ia.sigf, gq[j]);
                     float y = hadd(1.0f, n);
-                    if ((Tm[v >> 5] >> (v & 31)) & 1u) y = hsub(y, ia.muf);
+                    if ((tm >> j) & 1u) {
+                        y = hsub(y, ia.muf);
+                        if (keep_noise)
+                            for (int t = 0; t < ia.a; t++)
+                                if (ia.T[t] == v) misc->noise[hh][t] = n;
+                    }
                     const float lq = roundf(hmul(y, ia.cq));
                     L = lq > (float)dp.sat ? dp.sat : (lq < -(float)dp.sat ? -dp.sat : (int)lq);
                 }
@@ -109,18 +128,9 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kern
                 dec.set_half(Pc, v, hh, (unsigned)(L + (int)kBeta));
             }
         }
+        if (gp.gt == 0 && sidx[hh] >= 0) misc->next[hh][turn[hh]] = (long long)next;
     };
-
-    {
-        unsigned *Pc = Pbuf;
-        for (int hh = 0; hh < 2; hh++) {
-            fetch(hh);
-            generate(hh, Pc);
-        }
-        gp.sync();
-    }
-    while (sidx[0] >= 0 || sidx[1] >= 0) {
-        unsigned *Pc = Pbuf + pcur * g.n, *Pn = Pbuf + (pcur ^ 1) * g.n;
+    auto reset = [&](unsigned *Pn) {  // the accumulator: the channel values
         if ((g.n & 3) == 0) {  // 16-byte copies (Pbuf is 16-byte aligned, so are Pn and L2)
             const uint4 *src = (const uint4 *)L2;
             uint4 *dst = (uint4 *)Pn;
@@ -128,26 +138,50 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kern
         } else {
             for (int v = gp.gt; v < g.n; v += gp.T) Pn[v] = L2[v];
         }
-        gp.sync();
+    };
+
+    if (gp.gt == 0)
+        for (int hh = 0; hh < 2; hh++) misc->next[hh][0] = (long long)atomicAdd(ia.queue, 1ull);
+    gp.sync();
+#pragma unroll
+    for (int hh = 0; hh < 2; hh++) {
+        fetch(hh);
+        generate(hh, Pbuf);
+    }
+    gp.sync();
+    reset(Pbuf + g.n);
+    gp.sync();
+    while (sidx[0] >= 0 || sidx[1] >= 0) {
+        unsigned *Pc = Pbuf + pcur * g.n, *Pn = Pbuf + (pcur ^ 1) * g.n;
         const unsigned km = (first[0] ? 0xFFFF0000u : 0xFFFFFFFFu) & (first[1] ? 0x0000FFFFu : 0xFFFFFFFFu);
         const bool wr = (sidx[0] >= 0 && k[0] < dp.K) || (sidx[1] >= 0 && k[1] < dp.K);
         // (the common form -- no half starting, messages written -- compiled with writeR constant)
         const int us = wr && km == 0xFFFFFFFFu ? dec.template check_pass<false>(km, true, Pc, Pn)
                                                : dec.template check_pass<true>(km, wr, Pc, Pn);
-        int restart[2] = {0, 0};
+        bool any = false;
+#pragma unroll
         for (int hh = 0; hh < 2; hh++) {
             if (sidx[hh] < 0) continue;
             const int u = hh == 0 ? (us & 0xFFFF) : (us >> 16);
-            if (u != 0 && k[hh] != dp.K) continue;
+            if (u != 0 && k[hh] != dp.K) {
+                k[hh]++;
+                first[hh] = 0;
+                continue;
+            }
             const bool fail = u != 0 || dec.any_neg(Pc, hh) != 0;
             if (gp.gt == 0) {
                 const unsigned long long s = ia.s0 + (unsigned long long)sidx[hh];
                 double lw = 0.0;
                 for (int t = 0; t < ia.a; t++) {
-                    const int v = ia.T[t];
-                    float gq[4];
-                    normals4(ia.job, s, (uint32_t)(v >> 2), gq);
-                    const double n = (double)hmul(ia.sigf, gq[v & 3]);
+                    double n;
+                    if (keep_noise) {
+                        n = (double)misc->noise[hh][t];
+                    } else {
+                        const int v = ia.T[t];
+                        float gq[4];
+                        normals4(ia.job, s, (uint32_t)(v >> 2), gq);
+                        n = (double)hmul(ia.sigf, gq[v & 3]);
+                    }
                     lw = __dadd_rn(lw, __dsub_rn(__dmul_rn(n, ia.A), ia.Bc));
                 }
                 ia.wfail[sidx[hh]] = fail ? exp(lw) : 0.0;
@@ -157,18 +191,13 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kern
             }
             my_dec++;
             my_it += k[hh];
-            restart[hh] = 1;
+            gp.sync();  // (the noise is read, and the next index stored)
+            fetch(hh);
+            if (sidx[hh] >= 0) generate(hh, Pn);
+            any = true;
         }
-        gp.sync();
-        for (int hh = 0; hh < 2; hh++) {
-            if (restart[hh]) {
-                fetch(hh);
-                if (sidx[hh] >= 0) generate(hh, Pn);
-            } else if (sidx[hh] >= 0) {
-                k[hh]++;
-                first[hh] = 0;
-            }
-        }
+        if (any) gp.sync();
+        reset(Pc);
         gp.sync();
         pcur ^= 1;
     }

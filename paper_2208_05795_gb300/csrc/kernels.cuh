@@ -85,9 +85,11 @@ __host__ __device__ constexpr int pair_kernel_warps(int dc, bool exact) {
 __host__ __device__ constexpr int scalar_warps(bool is_float, int dc) { return is_float && dc <= 8 ? 24 : 16; }
 // the multi-code kernel (24: spills, no faster)
 constexpr int kBatchWarps = 20;
-// the importance-sampling kernel's large-degree form: 18 measured faster than 16, 20 or 24 on the
-// n = 8,832 code (1,152 checks, two a thread)
-constexpr int kIsWarps = 18;
+// the importance-sampling kernel's large-degree form, one sample pair to a CTA on the n = 8,832
+// code: 24 warps 43.2 ms for 200,000 samples, 20: 44.1, 18: 46.2, 16: 48.3
+constexpr int kIsWarps = 24;
+// room of its groups' shared scratch (isfer.cu)
+constexpr int kIsMiscBytes = 1536;
 struct BatchArgs {
     BatchItem it[kMaxBatch];
 };

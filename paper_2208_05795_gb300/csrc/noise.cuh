@@ -33,8 +33,10 @@ __device__ __forceinline__ void philox4x32_10(uint32_t &c0, uint32_t &c1, uint32
 __device__ __forceinline__ float uniform24(uint32_t x) { return hmul((float)(2u * (x >> 9) + 1u), 0x1p-24f); }
 
 __device__ __forceinline__ float series_logf(float u) {
-    int e;
-    float m = frexpf(u, &e);
+    // u = m 2^e with m in [1/2, 1): u >= 2^-24 is normal
+    const int ub = __float_as_int(u);
+    int e = (ub >> 23) - 126;
+    float m = __int_as_float((ub & 0x7FFFFF) | 0x3F000000);
     if (m < 0x1.6a09e6p-1f) {
         m = hadd(m, m);
         e = e - 1;
@@ -76,22 +78,16 @@ __device__ __forceinline__ void sincos2pi(float t, float &s, float &c) {
     const int k = (int)kf;
     const float f = hsub(t4, kf);
     const float HALF_PI = 0x1.921fb6p+0f;
-    float sa, ca;
-    if (f <= 0.5f) {
-        const float a = hmul(f, HALF_PI);
-        sa = sin_poly(a);
-        ca = cos_poly(a);
-    } else {
-        const float a = hmul(hsub(1.0f, f), HALF_PI);
-        sa = cos_poly(a);
-        ca = sin_poly(a);
-    }
-    switch (k & 3) {
-        case 0: s = sa; c = ca; break;
-        case 1: s = ca; c = -sa; break;
-        case 2: s = -sa; c = -ca; break;
-        default: s = -ca; c = sa; break;
-    }
+    // both series once, on f or 1 - f (lanes of a warp differ), exchanged above 1/2
+    const bool low = f <= 0.5f;
+    const float a = hmul(low ? f : hsub(1.0f, f), HALF_PI);
+    const float ps = sin_poly(a), qc = cos_poly(a);
+    const float sa = low ? ps : qc, ca = low ? qc : ps;
+    // quadrant k: (sa, ca), (ca, -sa), (-sa, -ca), (-ca, sa)
+    s = (k & 1) ? ca : sa;
+    c = (k & 1) ? sa : ca;
+    if (k & 2) s = -s;
+    if ((k + 1) & 2) c = -c;
 }
 
 __device__ __forceinline__ void normals4(unsigned long long job, unsigned long long s, uint32_t q, float g[4]) {
