@@ -60,6 +60,11 @@ struct TabOff {
 __host__ __device__ inline TabOff tab_offsets(const DevCode &g, bool pair = false) {
     TabOff o{};
     int x = 0;
+    if (pair && g.by_rows) {
+        o.c_vn = x; x += al16(g.E * 2);
+        o.total = x;
+        return o;
+    }
     if (g.kind == TSX_CODE_QC) {
         o.rdeg = x; x += al16(g.m_b * 2);
         o.reoff = x; x += al16(g.m_b * 4);
@@ -127,6 +132,15 @@ __device__ void copy_bytes(void *dst, const void *src, int bytes) {
 __device__ SGraph load_tables(const DevCode &g, unsigned char *sm, bool pair = false) {
     TabOff o = tab_offsets(g, pair);
     SGraph s{};
+    if (pair && g.by_rows) {
+        uint16_t *cv = (uint16_t *)(sm + o.c_vn);
+        for (int c = threadIdx.x; c < g.m; c += blockDim.x) {
+            const int i = c / g.Z, r = c - i * g.Z;
+            for (int p = 0; p < 6; p++) cv[c * 6 + p] = (uint16_t)(g.rjz[i * 6 + p] + wrapZ(r + g.rs[i * 6 + p], g.Z));
+        }
+        s.c_vn = cv;
+        return s;
+    }
     if (g.kind == TSX_CODE_QC) {
         copy_bytes(sm + o.rdeg, g.rdeg, g.m_b * 2);
         copy_bytes(sm + o.reoff, g.reoff, g.m_b * 4);

@@ -893,7 +893,7 @@ cudaError_t launch_pair(const DevCode &g, const DecodeParams &dp, const EnumBuff
     const bool qc = g.kind == TSX_CODE_QC;
     const bool reg6 = g.dc_min == 6 && g.dc_max == 6;
     if (reg6)
-        return qc ? launch_persistent(pair_kernel<true, 6, true, I8>, sh, st, g, dp, b, sh.lay, sh.G)
+        return qc && !g.by_rows ? launch_persistent(pair_kernel<true, 6, true, I8>, sh, st, g, dp, b, sh.lay, sh.G)
                   : launch_persistent(pair_kernel<false, 6, true, I8>, sh, st, g, dp, b, sh.lay, sh.G);
     if (g.dc_max <= 8)
         return qc ? launch_persistent(pair_kernel<true, 8, false, I8>, sh, st, g, dp, b, sh.lay, sh.G)

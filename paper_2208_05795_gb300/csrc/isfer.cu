@@ -304,7 +304,7 @@ static int is_plan(tsx_code *code, const int32_t *ts_vars, int32_t a, const tsx_
     J.dp.alpha_num = p->alpha_num;
     J.dp.alpha_shift = p->alpha_shift;
     J.dp.base_llr = 1;
-    if (!plan_is_shape(g, J.dp, &J.sh, code_num_sms(code))) return TSX_EUNSUPPORTED;
+    if (!plan_is_shape(J.g, J.dp, &J.sh, code_num_sms(code))) return TSX_EUNSUPPORTED;
     const long long N = p->n_samples;
     J.N = N;
     J.chunk = chunk > 0 && chunk < N ? chunk : N;
@@ -393,7 +393,7 @@ int is_job_start(tsx_code *code, const int32_t *ts_vars, int32_t a, const tsx_is
         cudaEventRecord(J->e0, s) != cudaSuccess)
         return bail(TSX_ECUDA);
     const DevCode &g = J->g;
-    const bool qc = g.kind == TSX_CODE_QC;
+    const bool qc = g.kind == TSX_CODE_QC && !g.by_rows;
     const bool reg6 = g.dc_min == 6 && g.dc_max == 6;
     for (long long k = 0; k < J->n_chunks; k++) {
         IsArgs ik = ia;

@@ -30,6 +30,7 @@ struct DevCode {
     int dv_max, dc_max;
     int dc_min;         // smallest check degree (dc_min == dc_max: check-regular)
     int dv_min;         // smallest variable degree (dv_min == dv_max: variable-regular)
+    int by_rows;        // launch only: the two-codeword tables are c_vn of a QC code of check degree 6
     int E_odd;          // QC: edges with every row filled up to an odd number
     int girth, wstart;  // wstart = max(1, girth/2)
     int n_rep;

@@ -87,3 +87,11 @@ def test_batch_of_mixed_degrees(names):
     tsx.batch_run(b)
     for i, c in enumerate(codes):
         _same(tsx.batch_view(b, i), tsx.ts_list_view(tsx.enumerate_ts(c, kernel=1, **p)))
+
+
+@pytest.mark.parametrize("Z", [1, 2, 31, 64, 700, 1600, 1850])
+def test_degree_six_tables(Z):
+    """Rows as node lists (few groups to many), and exponents where the lists do not fit beside one pair."""
+    code = tsx.load_code(_qc(3, 6, Z, 30 + Z))
+    p = dict(P, max_size=1 if Z == 1 else 2, cand_end=60)
+    _same(tsx.ts_list_view(tsx.enumerate_ts(code, kernel=2, **p)), tsx.ts_list_view(tsx.enumerate_ts(code, kernel=1, **p)))
