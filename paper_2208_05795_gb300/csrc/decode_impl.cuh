@@ -48,6 +48,9 @@ struct DecSpa {
 
 __host__ __device__ inline int al16(int x) { return (x + 15) & ~15; }
 
+// entries in a row of the two-codeword kernels' QC table: even, so that two of them are one 16-byte load
+__host__ __device__ inline int rt_row(const DevCode &g) { return (g.dc_max + 1) & ~1; }
+
 struct TabOff {
     int rdeg, reoff, rjz, rs, rt, roff, ct, cdeg, ceoff, cs, ciz;
     int c_ptr, c_vn, v_ptr, v_edge;
@@ -69,7 +72,7 @@ __host__ __device__ inline TabOff tab_offsets(const DevCode &g, bool pair = fals
         o.rdeg = x; x += al16(g.m_b * 2);
         o.reoff = x; x += al16(g.m_b * 4);
         if (pair) {
-            o.rt = x; x += al16(g.m_b * g.dc_max * 8);
+            o.rt = x; x += al16(g.m_b * rt_row(g) * 8);
             o.roff = x; x += al16(g.m_b * 4);
             o.ct = x; x += al16(g.n_b * g.dv_max * 16);
         } else {
@@ -96,7 +99,7 @@ struct SGraph {
     const int16_t *rdeg;
     const int32_t *reoff, *rjz;
     // two-codeword kernels
-    const int2 *rt;       // [m_b * dc_max] {4 rjz, 4 rs}
+    const int2 *rt;       // [m_b * rt_row] {4 rjz, 4 rs}
     const int32_t *roff;  // [m_b] first message of a row block, rows of an odd number of words
     const int4 *ct;       // [n_b * dv_max] {message offset, words a row, shift} of the t-th block of a column
     const int16_t *rs, *cdeg;
@@ -146,7 +149,11 @@ __device__ SGraph load_tables(const DevCode &g, unsigned char *sm, bool pair = f
         copy_bytes(sm + o.reoff, g.reoff, g.m_b * 4);
         if (pair) {
             int2 *rt = (int2 *)(sm + o.rt);
-            for (int i = threadIdx.x; i < g.m_b * g.dc_max; i += blockDim.x) rt[i] = make_int2(4 * g.rjz[i], 4 * (int)g.rs[i]);
+            const int row = rt_row(g);
+            for (int x = threadIdx.x; x < g.m_b * g.dc_max; x += blockDim.x) {
+                const int i = x / g.dc_max;
+                rt[i * row + x - i * g.dc_max] = make_int2(4 * g.rjz[x], 4 * (int)g.rs[x]);
+            }
             s.rt = rt;
             int *roff = (int *)(sm + o.roff);
             int4 *ct = (int4 *)(sm + o.ct);

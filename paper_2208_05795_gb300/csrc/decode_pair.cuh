@@ -98,6 +98,11 @@ __device__ __forceinline__ uint2 lds64(unsigned a) {
     asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
     return v;
 }
+__device__ __forceinline__ uint4 lds128(unsigned a) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
 __device__ __forceinline__ void sts32(unsigned a, unsigned v) {
     asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
@@ -339,17 +344,21 @@ struct PairDecoder {
     // words a check, so that lanes hit different banks and every offset is a constant.
     // Edges are taken four at a time, loads first: no load waits behind the
     // stores of the edges before it.
-    template <bool MASK, class PV, class Stride>
+    template <bool MASK, class PV, class PV2, class Stride>
     __device__ __forceinline__ int node_twopass(int deg, unsigned km, bool writeR, unsigned Pc, unsigned Pn,
-                                                PV pv, unsigned ra, Stride stride) const {
+                                                PV pv, PV2 pv2, unsigned ra, Stride stride) const {
         const unsigned rs = stride;
         unsigned sp = 0, sx = 0, M1 = pc.NS2, M2 = pc.NS2;
         auto first = [&](auto width, int p, unsigned a) {
             constexpr int W = decltype(width)::value;
             unsigned x[W], y[W], na[W];
+            if constexpr (W == 1) x[0] = pv(p);
+            else
+#pragma unroll
+                for (int e = 0; e < W; e += 2) pv2(p + e, x + e);
 #pragma unroll
             for (int e = 0; e < W; e++) {
-                x[e] = lds32(Pc + pv(p + e));
+                x[e] = lds32(Pc + x[e]);
                 y[e] = ldy<MASK>(a + e * rs, km);
             }
 #pragma unroll
@@ -371,7 +380,7 @@ struct PairDecoder {
         };
         int p = 0;
         unsigned a = ra;
-#pragma unroll 1
+#pragma unroll 2
         for (; p + 4 <= deg; p += 4, a += 4 * rs) first(Int<4>{}, p, a);
         if (deg & 2) {
             first(Int<2>{}, p, a);
@@ -384,9 +393,12 @@ struct PairDecoder {
             auto second = [&](auto width, int p, unsigned a) {
                 constexpr int W = decltype(width)::value;
                 unsigned po[W], d[W], na[W];
+                if constexpr (W == 1) po[0] = pv(p);
+                else
+#pragma unroll
+                    for (int e = 0; e < W; e += 2) pv2(p + e, po + e);
 #pragma unroll
                 for (int e = 0; e < W; e++) {
-                    po[e] = pv(p + e);
                     if constexpr (!I8) {
                         d[e] = ldR(a + e * rs);
                         na[e] = neg_abs(d[e]);
@@ -404,7 +416,7 @@ struct PairDecoder {
             };
             p = 0;
             a = ra;
-#pragma unroll 1
+#pragma unroll 2
             for (; p + 4 <= deg; p += 4, a += 4 * rs) second(Int<4>{}, p, a);
             if (deg & 2) {
                 second(Int<2>{}, p, a);
@@ -433,12 +445,20 @@ struct PairDecoder {
             for (int c = gp.gt; c < g.m; c += gp.T) {
                 const int i = Z > 1 ? (int)__umulhi((unsigned)c, zm) : c;
                 const int r = c - i * Z;
-                const unsigned rt = rt0 + 8u * (unsigned)(i * g.dc_max);
+                const unsigned rt = rt0 + 8u * (unsigned)(i * rt_row(g));
                 const unsigned r4 = 4u * (unsigned)r;
+                const auto at = [&](unsigned x, unsigned y) {  // 4 x column block start, 4 x shift
+                    const unsigned t = r4 + y;
+                    return x + __viaddmin_u32(t, 0u - Z4, t);  // min(t - Z4, t): t mod Z4
+                };
                 const auto pv = [&](int p) {
-                    const uint2 e = lds64(rt + 8u * (unsigned)p);  // 4 x column block start, 4 x shift
-                    const unsigned t = r4 + e.y;
-                    return e.x + __viaddmin_u32(t, 0u - Z4, t);  // min(t - Z4, t): t mod Z4
+                    const uint2 e = lds64(rt + 8u * (unsigned)p);
+                    return at(e.x, e.y);
+                };
+                const auto pv2 = [&](int p, unsigned *o) {  // positions p and p + 1, p even
+                    const uint4 e = lds128(rt + 8u * (unsigned)p);
+                    o[0] = at(e.x, e.y);
+                    o[1] = at(e.z, e.w);
                 };
                 if constexpr (EXACT && !I8 && DC % 2 == 0) {
                     u += node_cm<MASK>(Rb + (unsigned)c * (DC * RSZ), km, writeR, Pc, Pn, pv);
@@ -449,7 +469,7 @@ struct PairDecoder {
                         u += node<MASK, DC, EXACT>(deg, km, writeR, Pc, Pn, pv,
                                                    [&](int p) { return ra + (unsigned)p * rs; });
                     } else {
-                        u += node_twopass<MASK>(deg, km, writeR, Pc, Pn, pv,
+                        u += node_twopass<MASK>(deg, km, writeR, Pc, Pn, pv, pv2,
                                                 Rb + (unsigned)((sg.roff[i] + r * (deg | 1)) * RSZ), Int<RSZ>{});
                     }
                 }
@@ -461,6 +481,10 @@ struct PairDecoder {
                 const int e0 = EXACT ? c * DC : (int)sg.c_ptr[c];  // check-regular: rows of DC edges
                 const unsigned cva = cv + 2u * (unsigned)e0;
                 const auto pv = [&](int p) { return 4u * lds16(cva + 2u * (unsigned)p); };
+                const auto pv2 = [&](int p, unsigned *o) {
+                    o[0] = pv(p);
+                    o[1] = pv(p + 1);
+                };
                 if constexpr (EXACT && !I8 && DC % 2 == 0) {
                     // check-regular: messages check-major
                     u += node_cm<MASK>(Rb + (unsigned)(e0 * RSZ), km, writeR, Pc, Pn, pv);
@@ -470,7 +494,7 @@ struct PairDecoder {
                     if constexpr (DC <= 8)
                         u += node<MASK, DC, EXACT>(deg, km, writeR, Pc, Pn, pv,
                                                    [&](int p) { return ra + (unsigned)p * rs; });
-                    else u += node_twopass<MASK>(deg, km, writeR, Pc, Pn, pv, ra, rs);
+                    else u += node_twopass<MASK>(deg, km, writeR, Pc, Pn, pv, pv2, ra, rs);
                 }
             }
         }

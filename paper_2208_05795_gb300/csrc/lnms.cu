@@ -307,10 +307,18 @@ __global__ void __launch_bounds__(32 * kLnmsWarps, 1) lnms_pair_kernel(DevCode g
         my_fail += w != 0;
     };
     // byte offset of the p-th node of a row: column block start + (r + shift) mod Z
+    auto at = [&](unsigned x, unsigned y, unsigned r4) {
+        const unsigned t = r4 + y;
+        return Pa + x + __viaddmin_u32(t, 0u - Z4, t);
+    };
     auto pos = [&](unsigned rt, int p, unsigned r4) {
         const uint2 e = lds64(rt + 8u * (unsigned)p);
-        const unsigned t = r4 + e.y;
-        return Pa + e.x + __viaddmin_u32(t, 0u - Z4, t);
+        return at(e.x, e.y, r4);
+    };
+    auto pos2 = [&](unsigned rt, int p, unsigned r4, unsigned *o) {  // p even: two table entries in one load
+        const uint4 e = lds128(rt + 8u * (unsigned)p);
+        o[0] = at(e.x, e.y, r4);
+        o[1] = at(e.z, e.w, r4);
     };
 
     for (int e = gp.gt; e < g.E_odd; e += gp.T) R[e] = 0;
@@ -323,14 +331,17 @@ __global__ void __launch_bounds__(32 * kLnmsWarps, 1) lnms_pair_kernel(DevCode g
         int u = 0;
         for (int i = 0; i < g.m_b; i++) {
             const int deg = sg.rdeg[i];
-            const unsigned rt = rt0 + 8u * (unsigned)(i * g.dc_max);
+            const unsigned rt = rt0 + 8u * (unsigned)(i * rt_row(g));
             for (int r = gp.gt; r < Z; r += gp.T) {
                 unsigned sp = (deg & 1) ? 0x80008000u : 0u;
                 int p = 0;
 #pragma unroll 1
-                for (; p + 4 <= deg; p += 4)
-                    sp ^= lds32(pos(rt, p, 4u * r)) ^ lds32(pos(rt, p + 1, 4u * r)) ^ lds32(pos(rt, p + 2, 4u * r)) ^
-                          lds32(pos(rt, p + 3, 4u * r));
+                for (; p + 4 <= deg; p += 4) {
+                    unsigned o[4];
+                    pos2(rt, p, 4u * r, o);
+                    pos2(rt, p + 2, 4u * r, o + 2);
+                    sp ^= lds32(o[0]) ^ lds32(o[1]) ^ lds32(o[2]) ^ lds32(o[3]);
+                }
 #pragma unroll 1
                 for (; p < deg; p++) sp ^= lds32(pos(rt, p, 4u * r));
                 u += (int)((sp >> 15) & 0x00010001u);
@@ -353,7 +364,7 @@ __global__ void __launch_bounds__(32 * kLnmsWarps, 1) lnms_pair_kernel(DevCode g
         }
         for (int i = 0; i < g.m_b; i++) {
             const int deg = sg.rdeg[i];
-            const unsigned rt = rt0 + 8u * (unsigned)(i * g.dc_max);
+            const unsigned rt = rt0 + 8u * (unsigned)(i * rt_row(g));
             for (int r = gp.gt; r < Z; r += gp.T) {
                 const unsigned r4 = 4u * (unsigned)r;
                 const unsigned ra = Ra + 4u * (unsigned)(sg.roff[i] + r * (deg | 1));
@@ -362,8 +373,12 @@ __global__ void __launch_bounds__(32 * kLnmsWarps, 1) lnms_pair_kernel(DevCode g
                 auto first = [&](auto width, int p) {
                     constexpr int W = decltype(width)::value;
                     unsigned x[W], na[W];
+                    if constexpr (W == 1) x[0] = pos(rt, p, r4);
+                    else
 #pragma unroll
-                    for (int e = 0; e < W; e++) x[e] = lds32(pos(rt, p + e, r4)) - lds32(ra + 4u * (unsigned)(p + e));
+                        for (int e = 0; e < W; e += 2) pos2(rt, p + e, r4, x + e);
+#pragma unroll
+                    for (int e = 0; e < W; e++) x[e] = lds32(x[e]) - lds32(ra + 4u * (unsigned)(p + e));
 #pragma unroll
                     for (int e = 0; e < W; e++) {
                         x[e] = vmaxu2(vminu2(x[e], hi), lo);
@@ -394,11 +409,12 @@ __global__ void __launch_bounds__(32 * kLnmsWarps, 1) lnms_pair_kernel(DevCode g
                 auto second = [&](auto width, int p) {
                     constexpr int W = decltype(width)::value;
                     unsigned po[W], x[W];
+                    if constexpr (W == 1) po[0] = pos(rt, p, r4);
+                    else
 #pragma unroll
-                    for (int e = 0; e < W; e++) {
-                        po[e] = pos(rt, p + e, r4);
-                        x[e] = lds32(ra + 4u * (unsigned)(p + e));
-                    }
+                        for (int e = 0; e < W; e += 2) pos2(rt, p + e, r4, po + e);
+#pragma unroll
+                    for (int e = 0; e < W; e++) x[e] = lds32(ra + 4u * (unsigned)(p + e));
 #pragma unroll
                     for (int e = 0; e < W; e++) {
                         const unsigned na = vminu2(x[e], (~x[e]) + 0x00010001u);
