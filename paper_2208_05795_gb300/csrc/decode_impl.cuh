@@ -18,6 +18,7 @@
 // recomputed as clamp(P_v - r) when a check reads them.  Neighbour indices
 // of QC codes come from the exponent matrix: (r + a) mod Z.
 #pragma once
+#include "fdiv.cuh"
 #include "graph.cuh"
 #include "kernels.cuh"
 
@@ -250,7 +251,6 @@ struct Grp {
 __device__ __forceinline__ float hadd(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float hsub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float hmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float hdiv(float a, float b) { return __fdiv_rn(a, b); }
 
 __device__ __forceinline__ float spa_expm1_pos(float x) {
     const float k = rintf(hmul(x, 0x1.715476p+0f));
@@ -274,47 +274,47 @@ __device__ __forceinline__ float spa_expm1_pos(float x) {
 __device__ __forceinline__ float spa_tanhf(float y) {
     const float a = fabsf(y);
     const float e = spa_expm1_pos(hadd(a, a));
-    const float t = hdiv(e, hadd(e, 2.0f));
+    // e / (e + 2): e / 2 where e + 2 rounds to 2, and 1 where it rounds to e (a NaN for infinite e, as inf / inf)
+    float t = div_tanh(e);
+    t = e < 0x1p-24f ? hmul(e, 0.5f) : t;
+    t = e < 0x1p26f ? t : hadd(hsub(e, e), 1.0f);
     return y < 0.0f ? -t : t;
 }
 
+// (both series always and no branch: two edges' chains interleave)
 __device__ __forceinline__ float spa_atanhf(float p) {
     const float a = fabsf(p);
-    float r;
-    if (a < 0.25f) {
-        const float a2 = hmul(a, a);
-        float q = 0x1.e1e1e2p-5f;  // 1/17
-        q = hadd(hmul(q, a2), 0x1.111112p-4f);
-        q = hadd(hmul(q, a2), 0x1.3b13b2p-4f);
-        q = hadd(hmul(q, a2), 0x1.745d18p-4f);
-        q = hadd(hmul(q, a2), 0x1.c71c72p-4f);
-        q = hadd(hmul(q, a2), 0x1.24924ap-3f);
-        q = hadd(hmul(q, a2), 0x1.99999ap-3f);
-        q = hadd(hmul(q, a2), 0x1.555556p-2f);
-        q = hadd(hmul(q, a2), 1.0f);
-        r = hmul(q, a);
-    } else {
-        const float t = hdiv(hadd(1.0f, a), hsub(1.0f, a));
-        // t = m 2^e with m in [1/2, 1): t >= 5/3 is normal and finite (a <= 1 - 2^-24)
-        const int tb = __float_as_int(t);
-        int e = (tb >> 23) - 126;
-        float m = __int_as_float((tb & 0x7FFFFF) | 0x3F000000);
-        if (m < 0x1.6a09e6p-1f) {
-            m = hadd(m, m);
-            e = e - 1;
-        }
-        const float s = hdiv(hsub(m, 1.0f), hadd(m, 1.0f));
-        const float s2 = hmul(s, s);
-        float q = 0x1.3b13b2p-4f;  // 1/13
-        q = hadd(hmul(q, s2), 0x1.745d18p-4f);
-        q = hadd(hmul(q, s2), 0x1.c71c72p-4f);
-        q = hadd(hmul(q, s2), 0x1.24924ap-3f);
-        q = hadd(hmul(q, s2), 0x1.99999ap-3f);
-        q = hadd(hmul(q, s2), 0x1.555556p-2f);
-        q = hadd(hmul(q, s2), 1.0f);
-        const float lg = hadd(hmul((float)e, 0x1.62e43p-1f), hmul(hadd(s, s), q));
-        r = a < 1.0f ? hmul(0.5f, lg) : a;  // (a NaN stays one)
-    }
+    const float a2 = hmul(a, a);
+    float q = 0x1.e1e1e2p-5f;  // 1/17
+    q = hadd(hmul(q, a2), 0x1.111112p-4f);
+    q = hadd(hmul(q, a2), 0x1.3b13b2p-4f);
+    q = hadd(hmul(q, a2), 0x1.745d18p-4f);
+    q = hadd(hmul(q, a2), 0x1.c71c72p-4f);
+    q = hadd(hmul(q, a2), 0x1.24924ap-3f);
+    q = hadd(hmul(q, a2), 0x1.99999ap-3f);
+    q = hadd(hmul(q, a2), 0x1.555556p-2f);
+    q = hadd(hmul(q, a2), 1.0f);
+    const float small = hmul(q, a);
+    // t = m 2^e with m in [1/2, 1): for a in [1/4, 1), t >= 5/3 is normal and finite
+    const float t = div_atanh(a);
+    const int tb = __float_as_int(t);
+    int e = (tb >> 23) - 126;
+    float m = __int_as_float((tb & 0x7FFFFF) | 0x3F000000);
+    const bool up = m < 0x1.6a09e6p-1f;
+    m = up ? hadd(m, m) : m;
+    e = up ? e - 1 : e;
+    const float s = div_log(m);
+    const float s2 = hmul(s, s);
+    float z = 0x1.3b13b2p-4f;  // 1/13
+    z = hadd(hmul(z, s2), 0x1.745d18p-4f);
+    z = hadd(hmul(z, s2), 0x1.c71c72p-4f);
+    z = hadd(hmul(z, s2), 0x1.24924ap-3f);
+    z = hadd(hmul(z, s2), 0x1.99999ap-3f);
+    z = hadd(hmul(z, s2), 0x1.555556p-2f);
+    z = hadd(hmul(z, s2), 1.0f);
+    const float lg = hadd(hmul((float)e, 0x1.62e43p-1f), hmul(hadd(s, s), z));
+    float r = a < 0.25f ? small : hmul(0.5f, lg);
+    r = a < 1.0f ? r : a;  // (a NaN stays one)
     return p < 0.0f ? -r : r;
 }
 
@@ -416,7 +416,7 @@ struct Decoder {
             // the ones after it one by one.
             const float clip = dp.spa_clip;
             int par = 0;
-#pragma unroll 1
+#pragma unroll 2
             for (int p = 0; p < deg; p++) {
                 const float Pv = (float)P[nb(p)];
                 const float ro = first ? 0.0f : (float)R[e0 + p * estride];
@@ -424,18 +424,28 @@ struct Decoder {
                 if (writeR) R[e0 + p * estride] = (msg)spa_tanhf(__fmul_rn(clampf_(__fsub_rn(Pv, ro), -clip, clip), 0.5f));
             }
             if (writeR) {
+                auto out = [&](float prod) {
+                    float rr = __fmul_rn(2.0f, spa_atanhf(prod));
+                    rr = fabsf(prod) >= 1.0f ? (prod > 0.0f ? clip : -clip) : rr;
+                    return clampf_(rr, -clip, clip);
+                };
                 float pre = 1.0f;
+                int p = 0;
 #pragma unroll 1
-                for (int p = 0; p < deg; p++) {
-                    float prod = pre;
+                for (; p + 1 < deg; p += 2) {  // two edges at a time: the same later edges follow in both products
+                    const float t0 = (float)R[e0 + p * estride], t1 = (float)R[e0 + (p + 1) * estride];
+                    float A = __fmul_rn(pre, t1), B = __fmul_rn(pre, t0);
+                    pre = __fmul_rn(B, t1);
 #pragma unroll 4
-                    for (int p2 = p + 1; p2 < deg; p2++) prod = __fmul_rn(prod, (float)R[e0 + p2 * estride]);
-                    pre = __fmul_rn(pre, (float)R[e0 + p * estride]);
-                    float rr;
-                    if (fabsf(prod) >= 1.0f) rr = prod > 0.0f ? clip : -clip;
-                    else rr = __fmul_rn(2.0f, spa_atanhf(prod));
-                    R[e0 + p * estride] = (msg)clampf_(rr, -clip, clip);
+                    for (int p2 = p + 2; p2 < deg; p2++) {
+                        const float t = (float)R[e0 + p2 * estride];
+                        A = __fmul_rn(A, t);
+                        B = __fmul_rn(B, t);
+                    }
+                    R[e0 + p * estride] = (msg)out(A);
+                    R[e0 + (p + 1) * estride] = (msg)out(B);
                 }
+                if (p < deg) R[e0 + p * estride] = (msg)out(pre);
             }
             return par;
         }
@@ -1049,7 +1059,7 @@ __device__ __forceinline__ void scalar_run(const DevCode &g, const DecodeParams 
 // issue and the latency of its series and divisions, one chain per check and
 // warp, so warps in flight count more than registers: on a general (1008, 504)
 // code, 5,000 candidates, 12 groups of two warps (24 warps, 80 registers) take 56 ms,
-// 13 of one (16 or 20 warps) 96, 28 warps 57; small codes fill 32 one-warp
+// 13 of one (16 or 20 warps) 96, 28 warps 57 (with divisions by branch; 43 without); small codes fill 32 one-warp
 // groups (n = 306: 17.9 ms; 24 warps 22).  Before: 113 and 25.7.
 template <class Dec, int DCMAX, bool QC, int WARPS = 16>
 __global__ void __launch_bounds__(32 * WARPS, 1) enum_kernel(DevCode g, DecodeParams dp, EnumBuffers b,

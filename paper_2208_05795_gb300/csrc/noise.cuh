@@ -41,7 +41,7 @@ __device__ __forceinline__ float series_logf(float u) {
         m = hadd(m, m);
         e = e - 1;
     }
-    const float s = hdiv(hsub(m, 1.0f), hadd(m, 1.0f));
+    const float s = div_log(m);
     const float s2 = hmul(s, s);
     float q = 0x1.3b13b2p-4f;  // 1/13
     q = hadd(hmul(q, s2), 0x1.745d18p-4f);
