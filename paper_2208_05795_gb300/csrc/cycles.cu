@@ -156,13 +156,23 @@ constexpr unsigned short kNone = 0xFFFFu;
 
 // Adjacency of the code as rows of 16-bit ids (kNone: no such edge): vadj
 // [n][dvp], dvp = dv_max filled up to a multiple of 4, and cadj [m][dc_max].
-__global__ void adj_kernel(DevCode g, int dvp, unsigned short *vadj, unsigned short *cadj) {
+// by_block (QC, m_b <= dvp): a node's check of row block i is entry i, so that two
+// nodes' common checks are in the same entry of both rows.
+__global__ void adj_kernel(DevCode g, int dvp, int by_block, unsigned short *vadj, unsigned short *cadj) {
     const long long nv = (long long)g.n * dvp, nc = (long long)g.m * g.dc_max;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nv + nc;
          i += (long long)gridDim.x * blockDim.x) {
         if (i < nv) {
             const int v = (int)(i / dvp), t = (int)(i - (long long)v * dvp);
-            vadj[i] = t < vn_degree(g, v) ? (unsigned short)vn_check(g, v, t) : kNone;
+            int x = t < vn_degree(g, v) ? vn_check(g, v, t) : kNone;
+            if (by_block) {
+                x = kNone;
+                for (int q = 0; q < vn_degree(g, v); q++) {
+                    const int c = vn_check(g, v, q);
+                    if (c / g.Z == t) x = c;
+                }
+            }
+            vadj[i] = (unsigned short)x;
         } else {
             const int c = (int)((i - nv) / g.dc_max), p = (int)((i - nv) - (long long)c * g.dc_max);
             cadj[i - nv] = p < cn_degree(g, c) ? (unsigned short)cn_vn(g, c, p) : kNone;
@@ -250,8 +260,8 @@ __global__ void __launch_bounds__(512) pairs_kernel(Paths a) {
 }
 
 // checks meeting exactly one of the L distinct nodes vs[0..L-1], whose rows of
-// vadj are compared pair by pair
-template <int L, int DVP>
+// vadj are compared pair by pair (BLK: by_block rows, the same entries only)
+template <int L, int DVP, bool BLK>
 __device__ __forceinline__ int emd_distinct(const unsigned short *vadj, const int *vs) {
     unsigned short ch[L][DVP];
 #pragma unroll
@@ -268,7 +278,8 @@ __device__ __forceinline__ int emd_distinct(const unsigned short *vadj, const in
             for (int y = 0; y < L; y++)
                 if (y != x)
 #pragma unroll
-                    for (int q = 0; q < DVP; q++) other |= ch[y][q] == ch[x][t];
+                    for (int q = 0; q < DVP; q++)
+                        if (!BLK || q == t) other |= ch[y][q] == ch[x][t];
             emd += !other;
         }
     return emd;
@@ -278,7 +289,7 @@ __device__ __forceinline__ int emd_distinct(const unsigned short *vadj, const in
 // already enough threads); it counts the walks that close two steps after
 // its last node (and, PD = LMAX - 3, after each node one step further), and
 // those of the shorter prefixes whose deeper indices are 0.
-template <int LMAX, int PD, int DVP>
+template <int LMAX, int PD, int DVP, bool BLK>
 __global__ void __launch_bounds__(256) walk_kernel(Paths a, long long n_prefix, unsigned long long *walks,
                                                    unsigned long long *hist2) {
     // the CTA's histogram and walk counts, low words and carries
@@ -332,7 +343,7 @@ __global__ void __launch_bounds__(256) walk_kernel(Paths a, long long n_prefix, 
                 bool fast = false;
                 if constexpr (DVP <= 4) fast = distinct;
                 if (fast) {
-                    if constexpr (DVP <= 4) emd = emd_distinct<L, DVP>(a.vadj, vs);
+                    if constexpr (DVP <= 4) emd = emd_distinct<L, DVP, BLK>(a.vadj, vs);
                 } else {
                     emd = emd_of(a.g, vs, L);
                     if (!distinct) wt = 2 * L / walk_reps(vs, cs, L);
@@ -398,7 +409,7 @@ __global__ void __launch_bounds__(256) walk_kernel(Paths a, long long n_prefix, 
             if (hs[i] || hc[i]) atomicAdd(&hist2[i], ((unsigned long long)hc[i] << 32) + hs[i]);
 }
 
-template <int LMAX, int DVP>
+template <int LMAX, int DVP, bool BLK>
 cudaError_t launch_walk(const Paths &a, long long steps, unsigned long long *walks, unsigned long long *hist,
                         int num_sms, cudaStream_t st) {
     // prefixes of LMAX - 2 steps while they are few, else of one step less with the last step looped over
@@ -410,8 +421,8 @@ cudaError_t launch_walk(const Paths &a, long long steps, unsigned long long *wal
     const long long np = loop ? less : full;
     long long blocks = (np + 255) / 256;
     if (blocks > (long long)num_sms * 64) blocks = (long long)num_sms * 64;
-    if (loop) walk_kernel<LMAX, LMAX - 3, DVP><<<(int)blocks, 256, 0, st>>>(a, np, walks, hist);
-    else walk_kernel<LMAX, LMAX - 2, DVP><<<(int)blocks, 256, 0, st>>>(a, np, walks, hist);
+    if (loop) walk_kernel<LMAX, LMAX - 3, DVP, BLK><<<(int)blocks, 256, 0, st>>>(a, np, walks, hist);
+    else walk_kernel<LMAX, LMAX - 2, DVP, BLK><<<(int)blocks, 256, 0, st>>>(a, np, walks, hist);
     return cudaGetLastError();
 }
 
@@ -458,8 +469,9 @@ cudaError_t launch_cycles(const DevCode &g, int lmax, unsigned long long *walks,
     a.off = (unsigned *)(buf + b_vadj + b_cadj);
     a.ent = (uint2 *)(buf + b_vadj + b_cadj + b_off);
     const long long na = (long long)g.n * a.dvp + (long long)g.m * g.dc_max;
-    adj_kernel<<<(int)std::min<long long>((na + 255) / 256, 4096), 256, 0, st>>>(g, a.dvp, (unsigned short *)a.vadj,
-                                                                                (unsigned short *)a.cadj);
+    const bool blk = g.kind == TSX_CODE_QC && g.m_b <= a.dvp;
+    adj_kernel<<<(int)std::min<long long>((na + 255) / 256, 4096), 256, 0, st>>>(
+        g, a.dvp, blk ? 1 : 0, (unsigned short *)a.vadj, (unsigned short *)a.cadj);
     e = cudaGetLastError();
     const long long steps = (long long)a.dvp * g.dc_max;
     for (int r0 = 0; r0 < g.n_rep && e == cudaSuccess; r0 += (int)chunk) {
@@ -467,10 +479,13 @@ cudaError_t launch_cycles(const DevCode &g, int lmax, unsigned long long *walks,
         a.nrep = (int)std::min<long long>(chunk, g.n_rep - r0);
         pairs_kernel<<<a.nrep, 512, 0, st>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
-        const bool d4 = a.dvp == 4;
-        if (lmax == 4) e = d4 ? launch_walk<4, 4>(a, steps, walks, hist, num_sms, st) : launch_walk<4, 16>(a, steps, walks, hist, num_sms, st);
-        else if (lmax == 5) e = d4 ? launch_walk<5, 4>(a, steps, walks, hist, num_sms, st) : launch_walk<5, 16>(a, steps, walks, hist, num_sms, st);
-        else e = d4 ? launch_walk<6, 4>(a, steps, walks, hist, num_sms, st) : launch_walk<6, 16>(a, steps, walks, hist, num_sms, st);
+        auto go = [&](auto l) {
+            constexpr int LM = decltype(l)::value;
+            if (a.dvp > 4) return launch_walk<LM, 16, false>(a, steps, walks, hist, num_sms, st);
+            return blk ? launch_walk<LM, 4, true>(a, steps, walks, hist, num_sms, st)
+                       : launch_walk<LM, 4, false>(a, steps, walks, hist, num_sms, st);
+        };
+        e = lmax == 4 ? go(Depth<4>{}) : lmax == 5 ? go(Depth<5>{}) : go(Depth<6>{});
     }
     cudaFreeAsync(buf, st);
     return e;
