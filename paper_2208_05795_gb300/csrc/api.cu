@@ -371,6 +371,7 @@ extern "C" int load_code(const tsx_code_desc *desc, void *stream, tsx_code **out
         const int dc = h.kind == TSX_CODE_QC ? h.rdeg[c] : h.c_ptr[c + 1] - h.c_ptr[c];
         if (dc < d.dc_min) d.dc_min = dc;
     }
+    d.row_odd = 1;
     if (h.kind == TSX_CODE_QC)
         for (int i = 0; i < h.m_b; i++) d.E_odd += h.Z * (h.rdeg[i] | 1);
     d.wstart = std::max(1, girth / 2);

@@ -28,13 +28,14 @@ int msg_bytes(int decoder) { return decoder == TSX_DEC_NMS_I8 ? 1 : (decoder == 
 int post_bytes(int decoder) { return decoder == TSX_DEC_SPA_F32 ? 4 : 2; }
 
 // odd_rows: the two-codeword kernels' variant for check degrees above 8 (QC: each row an odd number of words)
-SlotLayout make_layout(const DevCode &g, int decoder, int kind, bool odd_rows) {
+// noise: the sampling kernel keeps the noise on the set's nodes
+SlotLayout make_layout(const DevCode &g, int decoder, int kind, bool odd_rows, bool noise) {
     SlotLayout L{};
-    L.tables_bytes = al16(tab_offsets(g, kind == kLayPair || kind == kLayIs || kind == kLayPairVn).total);
+    L.tables_bytes = al16(tab_offsets(g, kind == kLayPairVn ? 2 : kind == kLayPair || kind == kLayIs ? 1 : 0).total);
     const int nw = (g.n + 31) / 32;
     // message slots: QC edges, or the position-major m x dc_max grid of a CSR code
     const int nmsg = g.kind == TSX_CODE_QC ? g.E : g.m * g.dc_max;
-    const int nmsg2 = g.kind == TSX_CODE_QC && odd_rows ? g.E_odd : nmsg;
+    const int nmsg2 = g.kind == TSX_CODE_QC && odd_rows && g.row_odd ? g.E_odd : nmsg;
     int x = 0;
     if (kind == kLayScalar) {
         L.r_off = x; x += al16(nmsg * msg_bytes(decoder));
@@ -58,17 +59,19 @@ SlotLayout make_layout(const DevCode &g, int decoder, int kind, bool odd_rows) {
         L.r_off = x; x += al16(nmsg2 * 4);
         L.p_off = x; x += al16(3 * g.n * 4);  // two posterior buffers and the channel values
         L.xa_off = x; x += al16(nw * 4);      // bitmask of the trapping set
-        L.xb_off = L.xa_off;
+        L.xb_off = x; x += noise ? kIsNoiseBytes : 0;  // the noise on its nodes, or none
     } else {
         int rbytes = 4 * g.m;
         if (rbytes < 2 * g.n) rbytes = 2 * g.n;
         L.r_off = x; x += al16(rbytes);
         L.p_off = x; x += al16(2 * g.n);
-        L.xa_off = x; x += al16(nw * 4);  // the set
-        L.xb_off = x; x += al16(nw * 4);  // what the closure adds
+        L.xa_off = x; x += al16(nw * 4);
+        L.xb_off = L.xa_off;
     }
     const bool pair = kind == kLayPair || kind == kLayPairVn;
-    L.misc_off = x; x += al16((int)(pair ? sizeof(PairMisc) : kind == kLayIs ? kIsMiscBytes : sizeof(Misc)));
+    L.misc_off = x;
+    x += al16((int)(pair ? sizeof(PairMisc) : kind == kLayIs ? kIsMiscBytes : kind == kLaySieve ? sizeof(SieveMisc)
+                                                                                               : sizeof(Misc)));
     L.slot_bytes = x;
     return L;
 }
@@ -80,9 +83,10 @@ constexpr int kSmemCta = 226 * 1024;
 // units > 0: how many codeword groups the launch has work for (pairs of
 // candidates), where the host knows it.
 bool plan(const DevCode &g, int decoder, int kind, int G, int groups, int ctas_per_sm, int num_sms,
-          LaunchShape *out, int max_warps = 16, long long units = 0, bool odd_rows = false) {
+          LaunchShape *out, int max_warps = 16, long long units = 0, bool odd_rows = false,
+          bool noise = true) {
     LaunchShape sh{};
-    sh.lay = make_layout(g, decoder, kind, odd_rows || g.dc_max > 8);
+    sh.lay = make_layout(g, decoder, kind, odd_rows || g.dc_max > 8, noise);
     const int room = kSmemCta - sh.lay.tables_bytes;
     const int fit = room / sh.lay.slot_bytes;
     if (fit < 1) return false;
@@ -163,6 +167,11 @@ cudaError_t launch_decode(const DevCode &g0, const DecodeParams &dp, const EnumB
     if (try_pair) {
         g.by_rows = rows_table(g, dp.decoder, kLayPair, num_sms, pair_warps(g), units);
         pair = plan(g, dp.decoder, kLayPair, G, groups, ctas_per_sm, num_sms, &sh, pair_warps(g), units);
+        if (!pair) {  // without the filled-up rows
+            g.row_odd = 0;
+            pair = plan(g, dp.decoder, kLayPair, G, groups, ctas_per_sm, num_sms, &sh, pair_warps(g), units);
+            if (!pair) g.row_odd = 1;
+        }
     }
     // QC codes of large check degree whose two-buffer layout does not fit: the variable-node-pass form
     if (!pair && try_pair && g.kind == TSX_CODE_QC && dp.decoder == TSX_DEC_NMS_I16 &&
@@ -245,12 +254,18 @@ cudaError_t launch_batch(const BatchArgs &items, int n, int variant, const Launc
     return i8 ? launch_batch8(items, n, qc, dcmax, reg6, sh, st) : launch_batch16(items, n, qc, dcmax, reg6, sh, st);
 }
 
-bool plan_is_shape(DevCode &g, const DecodeParams &dp, LaunchShape *sh, int num_sms) {
+bool plan_is_shape(DevCode &g, const DecodeParams &dp, LaunchShape *sh, int num_sms, bool *noise) {
     if (!pair_ok(g, dp)) return false;
     g.by_rows = rows_table(g, TSX_DEC_NMS_I16, kLayIs, num_sms, 16, 0);
     // (the launch bounds of is_kernel)
-    return plan(g, TSX_DEC_NMS_I16, kLayIs, 0, 0, 0, num_sms, sh,
-                g.kind == TSX_CODE_QC && g.dc_max > 8 ? kIsWarps : 16);
+    const int warps = g.kind == TSX_CODE_QC && g.dc_max > 8 ? kIsWarps : 16;
+    // with the set's noise kept and rows filled up to odd lengths where there is room for them
+    for (int form = 0; form < 3; form++) {
+        *noise = form == 0;
+        g.row_odd = form < 2;
+        if (plan(g, TSX_DEC_NMS_I16, kLayIs, 0, 0, 0, num_sms, sh, warps, 0, false, *noise)) return true;
+    }
+    return false;
 }
 
 bool decode_fits(const DevCode &g, int decoder) {

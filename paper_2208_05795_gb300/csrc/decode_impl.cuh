@@ -61,7 +61,8 @@ struct TabOff {
 // pair = the tables of the two-codeword kernels: no per-variable edge lists
 // for general codes (they have no variable-node pass), and for QC codes the
 // column start and shift of each position as one 8-byte entry in byte units
-__host__ __device__ inline TabOff tab_offsets(const DevCode &g, bool pair = false) {
+// (pair = 2: and the column entries of the variable-node-pass form)
+__host__ __device__ inline TabOff tab_offsets(const DevCode &g, int pair = 0) {
     TabOff o{};
     int x = 0;
     if (pair && g.by_rows) {
@@ -75,7 +76,7 @@ __host__ __device__ inline TabOff tab_offsets(const DevCode &g, bool pair = fals
         if (pair) {
             o.rt = x; x += al16(g.m_b * rt_row(g) * 8);
             o.roff = x; x += al16(g.m_b * 4);
-            o.ct = x; x += al16(g.n_b * g.dv_max * 16);
+            if (pair == 2) { o.ct = x; x += al16(g.n_b * g.dv_max * 8); }
         } else {
             o.rjz = x; x += al16(g.m_b * g.dc_max * 4);
             o.rs = x; x += al16(g.m_b * g.dc_max * 2);
@@ -102,7 +103,8 @@ struct SGraph {
     // two-codeword kernels
     const int2 *rt;       // [m_b * rt_row] {4 rjz, 4 rs}
     const int32_t *roff;  // [m_b] first message of a row block, rows of an odd number of words
-    const int4 *ct;       // [n_b * dv_max] {message offset, words a row, shift} of the t-th block of a column
+    const int2 *ct;       // [n_b * dv_max] {message offset, words a row | shift << 8} of the t-th block of a column
+                          // (variable-node-pass form only)
     const int16_t *rs, *cdeg;
     const int32_t *ceoff;
     const int16_t *cs;
@@ -110,11 +112,11 @@ struct SGraph {
     const uint16_t *c_ptr, *c_vn, *v_ptr, *v_edge;
 };
 
-// First message of row block i where each row takes an odd number of words
-// (two-codeword kernels, check degree > 8); row_offset(g, m_b) is the total.
+// First message of row block i (two-codeword kernels, check degree > 8): each
+// row takes an odd number of words (row_odd), or its degree.
 __device__ __forceinline__ int row_offset(const DevCode &g, int i) {
     int x = 0;
-    for (int k = 0; k < i; k++) x += g.Z * (g.rdeg[k] | 1);
+    for (int k = 0; k < i; k++) x += g.Z * (g.rdeg[k] | g.row_odd);
     return x;
 }
 
@@ -133,7 +135,7 @@ __device__ void copy_bytes(void *dst, const void *src, int bytes) {
     }
 }
 
-__device__ SGraph load_tables(const DevCode &g, unsigned char *sm, bool pair = false) {
+__device__ SGraph load_tables(const DevCode &g, unsigned char *sm, int pair = 0) {
     TabOff o = tab_offsets(g, pair);
     SGraph s{};
     if (pair && g.by_rows) {
@@ -157,16 +159,18 @@ __device__ SGraph load_tables(const DevCode &g, unsigned char *sm, bool pair = f
             }
             s.rt = rt;
             int *roff = (int *)(sm + o.roff);
-            int4 *ct = (int4 *)(sm + o.ct);
             for (int i = threadIdx.x; i < g.m_b; i += blockDim.x) roff[i] = row_offset(g, i);
-            for (int x = threadIdx.x; x < g.n_b * g.dv_max; x += blockDim.x) {
-                const int j = x / g.dv_max;
-                if (x - j * g.dv_max >= g.cdeg[j]) continue;
-                const int i = g.ciz[x] / g.Z, p = (g.ceoff[x] - g.reoff[i]) / g.Z;
-                ct[x] = make_int4(row_offset(g, i) + p, g.rdeg[i] | 1, g.cs[x], 0);
+            if (pair == 2) {
+                int2 *ct = (int2 *)(sm + o.ct);
+                for (int x = threadIdx.x; x < g.n_b * g.dv_max; x += blockDim.x) {
+                    const int j = x / g.dv_max;
+                    if (x - j * g.dv_max >= g.cdeg[j]) continue;
+                    const int i = g.ciz[x] / g.Z, p = (g.ceoff[x] - g.reoff[i]) / g.Z;
+                    ct[x] = make_int2(row_offset(g, i) + p, (g.rdeg[i] | g.row_odd) | ((int)g.cs[x] << 8));
+                }
+                s.ct = ct;
             }
             s.roff = roff;
-            s.ct = ct;
         } else {
             copy_bytes(sm + o.rjz, g.rjz, g.m_b * g.dc_max * 4);
             copy_bytes(sm + o.rs, g.rs, g.m_b * g.dc_max * 2);
@@ -322,8 +326,10 @@ __device__ __forceinline__ float spa_atanhf(float p) {
 struct Misc {
     int red[64];
     long long bcast[2];
-    int ints[8];
     unsigned long long okd, okit;  // converged decodes of this group and their iterations
+};
+// the sieve kernel's (one warp a slot)
+struct SieveMisc {
     uint16_t seg[kMaxNb + 2], segw[kMaxNb + 2];
 };
 
@@ -1080,7 +1086,7 @@ __global__ void __launch_bounds__(512, 2) sieve_kernel(DevCode g, EnumBuffers b,
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned char *slot = smem + lay.tables_bytes + warp * lay.slot_bytes;
-    Misc *misc = (Misc *)(slot + lay.misc_off);
+    SieveMisc *misc = (SieveMisc *)(slot + lay.misc_off);
     Grp gp;
     gp.G = 1;
     gp.T = 32;
@@ -1088,11 +1094,12 @@ __global__ void __launch_bounds__(512, 2) sieve_kernel(DevCode g, EnumBuffers b,
     gp.gt = lane;
     gp.lane = lane;
     gp.bar = 1;
-    gp.red = misc->red;
+    gp.red = nullptr;  // (one warp reduces in registers)
     int *deg = (int *)(slot + lay.r_off);
     uint16_t *key = (uint16_t *)(slot + lay.r_off);
     uint16_t *L = (uint16_t *)(slot + lay.p_off);
-    uint32_t *S = (uint32_t *)(slot + lay.xa_off), *added = (uint32_t *)(slot + lay.xb_off);
+    uint32_t *S = (uint32_t *)(slot + lay.xa_off);
+    uint32_t *added = (uint32_t *)L;  // (what a closure adds: done with before the member list is written)
     Sieve<QC> sv{g, sg, gp};
 
     const long long total = (long long)b.ctr->n_cand_total;

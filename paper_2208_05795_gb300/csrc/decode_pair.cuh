@@ -470,7 +470,7 @@ struct PairDecoder {
                                                    [&](int p) { return ra + (unsigned)p * rs; });
                     } else {
                         u += node_twopass<MASK>(deg, km, writeR, Pc, Pn, pv, pv2,
-                                                Rb + (unsigned)((sg.roff[i] + r * (deg | 1)) * RSZ), Int<RSZ>{});
+                                                Rb + (unsigned)((sg.roff[i] + r * (deg | g.row_odd)) * RSZ), Int<RSZ>{});
                     }
                 }
             }
@@ -565,14 +565,14 @@ struct PairDecoder {
             const int j = Z > 1 ? (int)__umulhi((unsigned)v, zm) : v;
             const int k = v - j * Z;
             const int dv = sg.cdeg[j];
-            const int4 *ct = sg.ct + j * g.dv_max;  // message offset, stride and shift of the t-th block
+            const int2 *ct = sg.ct + j * g.dv_max;  // message offset, stride and shift of the t-th block
             const unsigned l = (unsigned)(Lb + (int)kBeta - dv * kB);
             unsigned acc = l | (l << 16);
             for (int t = 0; t < dv; t++) {
                 // block (i, j) with shift s joins row r to column (r + s) mod Z: r = (k - s) mod Z
-                const int4 e = ct[t];
-                const int r = wrapZneg(k - e.z, Z);
-                acc += ldR(Rb + (unsigned)((e.x + r * e.y) * RSZ));
+                const int2 e = ct[t];
+                const int r = wrapZneg(k - (e.y >> 8), Z);
+                acc += ldR(Rb + (unsigned)((e.x + r * (e.y & 0xFF)) * RSZ));
             }
             P[v] = acc;
         }
@@ -886,7 +886,7 @@ template <bool I8>
 __global__ void __launch_bounds__(32 * pair_kernel_warps(32, false), 1) pair_vn_kernel(DevCode g, DecodeParams dp, EnumBuffers b,
                                                                SlotLayout lay, int G) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const SGraph sg = load_tables(g, smem, true);
+    const SGraph sg = load_tables(g, smem, 2);
     __syncthreads();
     pair_run<true, 32, false, I8, true>(g, dp, b, lay, G, sg, smem, (threadIdx.x >> 5) / G);
 }

@@ -22,14 +22,13 @@
 namespace tsx {
 namespace {
 
-// the group's shared scratch: the noise on the trapping set's nodes of each half's sample, where
-// the set has at most kTsNoise nodes
+// The group's shared scratch.  The noise on the trapping set's nodes of each half's sample is kept
+// beside it ([half][kTsNoise] floats) where there is room and the set has at most kTsNoise nodes.
 constexpr int kTsNoise = 64;
 struct IsMisc : Misc {
     long long next[2][2];  // [half][turn]: the sample drawn ahead (two places: one is written while the other is read)
-    float noise[2][kTsNoise];
 };
-static_assert(sizeof(IsMisc) <= kIsMiscBytes, "room of the sampling kernel's scratch");
+static_assert(sizeof(IsMisc) <= kIsMiscBytes && 2 * kTsNoise * sizeof(float) <= kIsNoiseBytes, "the sampling kernel's room");
 
 struct IsArgs {
     unsigned long long job, s0;
@@ -38,6 +37,7 @@ struct IsArgs {
     double A, Bc;
     const int *T;
     int a;
+    int keep_noise;
     double *wfail;            // [nsamp] fail * w
     unsigned char *fail_out;  // [nsamp] or null
     double *logw_out;         // [nsamp] or null
@@ -98,7 +98,8 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kern
         first[hh] = 1;
         if (gp.gt == 0 && sidx[hh] >= 0) next = atomicAdd(ia.queue, 1ull);
     };
-    const bool keep_noise = ia.a <= kTsNoise;
+    float *noise = (float *)(slot + lay.xb_off);
+    const bool keep_noise = ia.keep_noise && ia.a <= kTsNoise;
     // channel values of sample sidx[hh] into half hh of L2 (accumulator
     // start) and of the current posteriors (P = L); an idle half gets L = 0
     auto generate = [&](int hh, unsigned *Pc) {
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kern
                         y = hsub(y, ia.muf);
                         if (keep_noise)
                             for (int t = 0; t < ia.a; t++)
-                                if (ia.T[t] == v) misc->noise[hh][t] = n;
+                                if (ia.T[t] == v) noise[hh * kTsNoise + t] = n;
                     }
                     const float lq = roundf(hmul(y, ia.cq));
                     L = lq > (float)dp.sat ? dp.sat : (lq < -(float)dp.sat ? -dp.sat : (int)lq);
@@ -175,7 +176,7 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kern
                 for (int t = 0; t < ia.a; t++) {
                     double n;
                     if (keep_noise) {
-                        n = (double)misc->noise[hh][t];
+                        n = (double)noise[hh * kTsNoise + t];
                     } else {
                         const int v = ia.T[t];
                         float gq[4];
@@ -304,7 +305,9 @@ static int is_plan(tsx_code *code, const int32_t *ts_vars, int32_t a, const tsx_
     J.dp.alpha_num = p->alpha_num;
     J.dp.alpha_shift = p->alpha_shift;
     J.dp.base_llr = 1;
-    if (!plan_is_shape(J.g, J.dp, &J.sh, code_num_sms(code))) return TSX_EUNSUPPORTED;
+    bool noise = false;
+    if (!plan_is_shape(J.g, J.dp, &J.sh, code_num_sms(code), &noise)) return TSX_EUNSUPPORTED;
+    J.ia.keep_noise = noise;
     const long long N = p->n_samples;
     J.N = N;
     J.chunk = chunk > 0 && chunk < N ? chunk : N;

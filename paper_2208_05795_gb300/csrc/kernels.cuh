@@ -88,8 +88,8 @@ constexpr int kBatchWarps = 20;
 // the importance-sampling kernel's large-degree form, one sample pair to a CTA on the n = 8,832
 // code: 24 warps 43.2 ms for 200,000 samples, 20: 44.1, 18: 46.2, 16: 48.3
 constexpr int kIsWarps = 24;
-// room of its groups' shared scratch (isfer.cu)
-constexpr int kIsMiscBytes = 1536;
+// its groups' shared scratch, and the room for the noise on the set's nodes (isfer.cu)
+constexpr int kIsMiscBytes = 320, kIsNoiseBytes = 512;
 struct BatchArgs {
     BatchItem it[kMaxBatch];
 };
@@ -119,9 +119,10 @@ cudaError_t launch_decode(const DevCode &g, const DecodeParams &dp, const EnumBu
 cudaError_t launch_sieve(const DevCode &g, const EnumBuffers &b, int decoder, int num_sms, cudaStream_t st);
 
 // Shape of the importance-sampling kernel (two samples per lane) and the form
-// of the code's tables (g.by_rows); false if the 16-bit bias bounds or the
+// of the code's tables and rows (g.by_rows, g.row_odd), and whether the noise on
+// the set's nodes is kept; false if the 16-bit bias bounds or the
 // shared memory do not allow it.
-bool plan_is_shape(DevCode &g, const DecodeParams &dp, LaunchShape *sh, int num_sms);
+bool plan_is_shape(DevCode &g, const DecodeParams &dp, LaunchShape *sh, int num_sms, bool *noise);
 
 // Whether one codeword of g fits the shared memory of a CTA.
 bool decode_fits(const DevCode &g, int decoder);

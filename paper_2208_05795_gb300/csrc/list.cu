@@ -19,9 +19,16 @@
 namespace tsx {
 namespace {
 
+struct ListMisc {
+    int red[8];  // (groups of at most 6 warps)
+    long long bcast;
+    int count;   // sets this candidate has counted
+    uint16_t seg[kMaxNb + 2], segw[kMaxNb + 2];
+};
+
 struct ListLayout {
     int tables_bytes;
-    int r_off, p_off, s_off, add_off, xk_off, xp_off, deg_off, l_off, key_off, seen_off, misc_off;
+    int r_off, p_off, s_off, xk_off, xp_off, deg_off, l_off, key_off, seen_off, misc_off;
     int slot_bytes;
 };
 
@@ -34,14 +41,13 @@ ListLayout list_layout(const DevCode &g, int K) {
     L.r_off = x; x += al16(nmsg * 2);
     L.p_off = x; x += al16(g.n * 2);
     L.s_off = x; x += al16(nw * 4);
-    L.add_off = x; x += al16(nw * 4);
     L.xk_off = x; x += al16(nw * 4);
     L.xp_off = x; x += al16(nw * 4);
     L.deg_off = x; x += al16(g.m * 4);
     L.l_off = x; x += al16(g.n * 2);
     L.key_off = x; x += al16(g.n * 2);
     L.seen_off = x; x += al16(2 * (K + 1) * 4);  // at most two sets per iteration
-    L.misc_off = x; x += al16((int)sizeof(Misc));
+    L.misc_off = x; x += al16((int)sizeof(ListMisc));
     L.slot_bytes = x;
     return L;
 }
@@ -60,7 +66,7 @@ __global__ void __launch_bounds__(32 * kListWarps, 1) list_kernel(DevCode g, Dec
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int grp = warp / G;
     unsigned char *slot = smem + lay.tables_bytes + grp * lay.slot_bytes;
-    Misc *misc = (Misc *)(slot + lay.misc_off);
+    ListMisc *misc = (ListMisc *)(slot + lay.misc_off);
     Grp gp;
     gp.G = G;
     gp.T = 32 * G;
@@ -72,11 +78,11 @@ __global__ void __launch_bounds__(32 * kListWarps, 1) list_kernel(DevCode g, Dec
     int16_t *P = (int16_t *)(slot + lay.p_off);
     int16_t *R = (int16_t *)(slot + lay.r_off);
     uint32_t *S = (uint32_t *)(slot + lay.s_off);
-    uint32_t *added = (uint32_t *)(slot + lay.add_off);
     uint32_t *Xk = (uint32_t *)(slot + lay.xk_off);
     uint32_t *Xp = (uint32_t *)(slot + lay.xp_off);
     int *deg = (int *)(slot + lay.deg_off);
     uint16_t *L = (uint16_t *)(slot + lay.l_off);
+    uint32_t *added = (uint32_t *)L;  // (what a closure adds: done with before the member list is written)
     uint16_t *key = (uint16_t *)(slot + lay.key_off);
     int *seen = (int *)(slot + lay.seen_off);
     Decoder<DecNms16, DCMAX, QC> dec{g, sg, gp, dp, P, R};
@@ -101,9 +107,9 @@ __global__ void __launch_bounds__(32 * kListWarps, 1) list_kernel(DevCode g, Dec
     long long my_pat = 0, my_it = 0;
 
     while (true) {
-        if (gp.gt == 0) misc->bcast[0] = (long long)atomicAdd(&b.ctr->next_sieve, 1ull);
+        if (gp.gt == 0) misc->bcast = (long long)atomicAdd(&b.ctr->next_sieve, 1ull);
         gp.sync();
-        const long long o = misc->bcast[0];
+        const long long o = misc->bcast;
         gp.sync();
         if (o >= n) break;
         const int thr = b.c_thr[o];
@@ -113,7 +119,7 @@ __global__ void __launch_bounds__(32 * kListWarps, 1) list_kernel(DevCode g, Dec
         const int nI = (I4.x >= 0) + (I4.y >= 0) + (I4.z >= 0) + (I4.w >= 0);
         const int Limp = clampi(dp.base_llr - thr, -dp.sat, dp.sat);
         const int Kc = cand_limit(dp, b, b.cand_begin + o);
-        if (gp.gt == 0) misc->ints[0] = 0;  // sets this candidate has counted
+        if (gp.gt == 0) misc->count = 0;  // sets this candidate has counted
         for (int v = gp.gt; v < g.n; v += gp.T) P[v] = (int16_t)Lbase;
         gp.sync();
         if (gp.gt < nI) P[I[gp.gt]] = (int16_t)Limp;
@@ -147,12 +153,12 @@ __global__ void __launch_bounds__(32 * kListWarps, 1) list_kernel(DevCode g, Dec
                             const int orbit = canon_key(g, L, a, S, key, misc->seg, misc->segw, lane);
                             const long long ts = ts_insert(b, key, a, bb, orbit, elem | (part << 1), lane);
                             if (lane == 0 && ts >= 0) {
-                                const int cnt = misc->ints[0];
+                                const int cnt = misc->count;
                                 bool dup = false;
                                 for (int i = 0; i < cnt && !dup; i++) dup = seen[i] == (int)ts;
                                 if (!dup) {
                                     seen[cnt] = (int)ts;
-                                    misc->ints[0] = cnt + 1;
+                                    misc->count = cnt + 1;
                                     atomicMin(&b.t_thr[ts], thr);
                                     atomicAdd(&b.t_count[ts], 1);
                                 }

@@ -95,3 +95,14 @@ def test_degree_six_tables(Z):
     code = tsx.load_code(_qc(3, 6, Z, 30 + Z))
     p = dict(P, max_size=1 if Z == 1 else 2, cand_end=60)
     _same(tsx.ts_list_view(tsx.enumerate_ts(code, kernel=2, **p)), tsx.ts_list_view(tsx.enumerate_ts(code, kernel=1, **p)))
+
+
+@pytest.mark.parametrize("mb,nb,Z", [(3, 8, 1188), (4, 10, 817), (4, 9, 868)])
+def test_sampling_near_the_shared_memory_limit(mb, nb, Z):
+    """Codes whose sampling layout has no room for the kept noise, or for rows of odd length: still taken, with the
+    log-weights of a shorter list of nodes (which do not depend on the code) and no failure without noise to speak of."""
+    code = tsx.load_code(_qc(mb, nb, Z, 40 + nb))
+    kw = dict(ebn0_db=12.0, n_samples=6, job_key=3, rate=0.5, K=4, record=True)
+    r = tsx.is_fer_estimate(code, [0, 5, 9], **kw)
+    small = tsx.is_fer_estimate(tsx.load_code(_qc(3, 6, 16, 1)), [0, 5, 9], **kw)
+    assert np.array_equal(r["logw"], small["logw"]) and r["decodes"] == 6
