@@ -209,14 +209,18 @@ __device__ SGraph load_tables(const DevCode &g, unsigned char *sm, int pair = 0)
 struct Grp {
     int G, T, gt, lane, gw, bar;
     int *red;  // reduction scratch (shared): [0, 32) for sum(), [32, 64) for sum_pass()
+    // Both forms are volatile asm statements with a memory clobber: the two-codeword kernels read
+    // shared memory by volatile asm without one, and what was written by ordinary stores has to be
+    // ordered before such reads (and ordinary stores after them) in the source already; __syncwarp() is
+    // not an asm statement and orders ordinary accesses only.
     __device__ __forceinline__ void sync() const {
-        if (G == 1) __syncwarp();
+        if (G == 1) asm volatile("bar.warp.sync 0xffffffff;" ::: "memory");
         else asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(T) : "memory");
     }
     __device__ __forceinline__ int sum(int x) const {
         x = __reduce_add_sync(0xffffffffu, x);
         if (G == 1) {
-            __syncwarp();
+            sync();
             return x;
         }
         if (lane == 0) red[gw] = x;
@@ -230,7 +234,7 @@ struct Grp {
     __device__ __forceinline__ int sum_pass(int x) const {
         x = __reduce_add_sync(0xffffffffu, x);
         if (G == 1) {
-            __syncwarp();
+            sync();
             return x;
         }
         if (lane == 0) red[32 + gw] = x;

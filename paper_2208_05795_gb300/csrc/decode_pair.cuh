@@ -80,8 +80,9 @@ __device__ __forceinline__ unsigned prmt(unsigned a, unsigned b, unsigned sel) {
 __device__ __forceinline__ unsigned spread15(unsigned x) { return prmt(x, x, 0xBB99u); }
 // Shared-memory accesses of the check pass by 32-bit address: with pointers
 // the compiler keeps 64-bit generic addresses, whose arithmetic doubled the
-// large-degree loop (60 warp instructions per edge pair).  Volatile, so that
-// none moves across a barrier.
+// large-degree loop (60 warp instructions per edge pair).  Volatile and
+// without a memory clobber: none moves across Grp::sync(), which is volatile asm too and has the
+// clobber, and the ordinary accesses between two barriers keep their freedom.
 __device__ __forceinline__ unsigned saddr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ unsigned lds32(unsigned a) {
     unsigned v;
