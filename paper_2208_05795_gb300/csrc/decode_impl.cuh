@@ -112,11 +112,11 @@ struct SGraph {
     const uint16_t *c_ptr, *c_vn, *v_ptr, *v_edge;
 };
 
-// First message of row block i (two-codeword kernels, check degree > 8): each
-// row takes an odd number of words (row_odd), or its degree.
+// First message of row block i where rows are filled up (two-codeword kernels,
+// check degree > 8): each row takes an odd number of words.
 __device__ __forceinline__ int row_offset(const DevCode &g, int i) {
     int x = 0;
-    for (int k = 0; k < i; k++) x += g.Z * (g.rdeg[k] | g.row_odd);
+    for (int k = 0; k < i; k++) x += g.Z * (g.rdeg[k] | 1);
     return x;
 }
 
@@ -166,7 +166,8 @@ __device__ SGraph load_tables(const DevCode &g, unsigned char *sm, int pair = 0)
                     const int j = x / g.dv_max;
                     if (x - j * g.dv_max >= g.cdeg[j]) continue;
                     const int i = g.ciz[x] / g.Z, p = (g.ceoff[x] - g.reoff[i]) / g.Z;
-                    ct[x] = make_int2(row_offset(g, i) + p, (g.rdeg[i] | g.row_odd) | ((int)g.cs[x] << 8));
+                    ct[x] = g.row_odd ? make_int2(row_offset(g, i) + p, (g.rdeg[i] | 1) | ((int)g.cs[x] << 8))
+                                      : make_int2(g.ceoff[x], 1 | ((int)g.cs[x] << 8));
                 }
                 s.ct = ct;
             }

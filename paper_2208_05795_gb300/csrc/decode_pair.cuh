@@ -179,7 +179,13 @@ struct PairMisc : Misc {
 // after each check pass from the stored messages, instead of the
 // accumulating second buffer -- 4 bytes per node less, for codes whose
 // two-buffer layout does not fit a CTA.
-template <bool QC, int DC, bool EXACT, bool I8, bool VN = false>
+// FILL: QC rows of large degree filled up to an odd number of words.  A code that
+// fits a CTA only without the filling keeps its messages by position (message p of row r of a block
+// Z words after message p - 1), lanes on consecutive words: a check's words together without the
+// filling meet the same banks 32 times at degree 32 and 4 times at 28 (two buffers, 3,000 candidates: degree 32,
+// Z = 291: 147 ms, by position 16.4; degree 28, Z = 332: 23.3 and 14.9.  Sampling, degree 32,
+// Z = 254, 6,000 samples: 24.3 and 3.0).
+template <bool QC, int DC, bool EXACT, bool I8, bool VN = false, bool FILL = true>
 struct PairDecoder {
     static constexpr int RSZ = I8 ? 2 : 4;  // bytes of one packed message pair
     static constexpr int kB = I8 ? 128 : 0;  // message bias
@@ -342,7 +348,7 @@ struct PairDecoder {
     // loop did not fit the instruction cache: 0.57x on a degree-16 code.)
     // ra: address of the check's first message, stride: bytes between its
     // messages.  QC codes keep a check's messages together, an odd number of
-    // words a check, so that lanes hit different banks and every offset is a constant.
+    // words a check, so that lanes hit different banks and every offset is a constant (FILL).
     // Edges are taken four at a time, loads first: no load waits behind the
     // stores of the edges before it.
     template <bool MASK, class PV, class PV2, class Stride>
@@ -469,9 +475,12 @@ struct PairDecoder {
                         const unsigned ra = Rb + (unsigned)((sg.reoff[i] + r) * RSZ), rs = (unsigned)(Z * RSZ);
                         u += node<MASK, DC, EXACT>(deg, km, writeR, Pc, Pn, pv,
                                                    [&](int p) { return ra + (unsigned)p * rs; });
-                    } else {
+                    } else if constexpr (FILL) {
                         u += node_twopass<MASK>(deg, km, writeR, Pc, Pn, pv, pv2,
-                                                Rb + (unsigned)((sg.roff[i] + r * (deg | g.row_odd)) * RSZ), Int<RSZ>{});
+                                                Rb + (unsigned)((sg.roff[i] + r * (deg | 1)) * RSZ), Int<RSZ>{});
+                    } else {
+                        u += node_twopass<MASK>(deg, km, writeR, Pc, Pn, pv, pv2, Rb + (unsigned)((sg.reoff[i] + r) * RSZ),
+                                                (unsigned)(Z * RSZ));
                     }
                 }
             }
@@ -604,7 +613,7 @@ struct PairDecoder {
 // thread keeps, per half, only what each iteration needs (whether it runs,
 // its iteration, its limit, the smallest u_k); the schedule itself is in
 // shared memory and is advanced by thread 0 where a decode ends.
-template <bool QC, int DC, bool EXACT, bool I8, bool VN = false>
+template <bool QC, int DC, bool EXACT, bool I8, bool VN = false, bool FILL = true>
 __device__ __forceinline__ void pair_run(const DevCode &g, const DecodeParams &dp, const EnumBuffers &b,
                                          const SlotLayout &lay, int G, const SGraph &sg, unsigned char *smem, int grp) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -625,7 +634,7 @@ __device__ __forceinline__ void pair_run(const DevCode &g, const DecodeParams &d
     const int xstride = (nw + 3) & ~3;
 
     const PairConst pc = pair_const(dp);
-    PairDecoder<QC, DC, EXACT, I8, VN> dec{g, sg, gp, pc, saddr(slot + lay.r_off)};
+    PairDecoder<QC, DC, EXACT, I8, VN, FILL> dec{g, sg, gp, pc, saddr(slot + lay.r_off)};
 
     const long long total = (long long)b.ctr->n_cand_total;
     const long long end = b.cand_end < 0 || b.cand_end > total ? total : b.cand_end;
@@ -894,23 +903,23 @@ __device__ __forceinline__ void pair_run(const DevCode &g, const DecodeParams &d
     }
 }
 
-template <bool QC, int DC, bool EXACT, bool I8>
+template <bool QC, int DC, bool EXACT, bool I8, bool FILL = true>
 __global__ void __launch_bounds__(32 * pair_kernel_warps(DC, EXACT), 1)
     pair_kernel(DevCode g, DecodeParams dp, EnumBuffers b, SlotLayout lay, int G) {
     extern __shared__ __align__(16) unsigned char smem[];
     const SGraph sg = load_tables(g, smem, true);
     __syncthreads();
-    pair_run<QC, DC, EXACT, I8>(g, dp, b, lay, G, sg, smem, (threadIdx.x >> 5) / G);
+    pair_run<QC, DC, EXACT, I8, false, FILL>(g, dp, b, lay, G, sg, smem, (threadIdx.x >> 5) / G);
 }
 
 // the VN form for QC codes of large check degree whose two-buffer layout does not fit
-template <bool I8>
+template <bool I8, bool FILL>
 __global__ void __launch_bounds__(32 * pair_kernel_warps(32, false), 1) pair_vn_kernel(DevCode g, DecodeParams dp, EnumBuffers b,
                                                                SlotLayout lay, int G) {
     extern __shared__ __align__(16) unsigned char smem[];
     const SGraph sg = load_tables(g, smem, 2);
     __syncthreads();
-    pair_run<true, 32, false, I8, true>(g, dp, b, lay, G, sg, smem, (threadIdx.x >> 5) / G);
+    pair_run<true, 32, false, I8, true, FILL>(g, dp, b, lay, G, sg, smem, (threadIdx.x >> 5) / G);
 }
 
 // One persistent launch over several codes: every CTA works through the
@@ -944,6 +953,7 @@ cudaError_t launch_pair(const DevCode &g, const DecodeParams &dp, const EnumBuff
     if (g.dc_max <= 8)
         return qc ? launch_persistent(pair_kernel<true, 8, false, I8>, sh, st, g, dp, b, sh.lay, sh.G)
                   : launch_persistent(pair_kernel<false, 8, false, I8>, sh, st, g, dp, b, sh.lay, sh.G);
+    if (qc && !g.row_odd) return launch_persistent(pair_kernel<true, 32, false, I8, false>, sh, st, g, dp, b, sh.lay, sh.G);
     return qc ? launch_persistent(pair_kernel<true, 32, false, I8>, sh, st, g, dp, b, sh.lay, sh.G)
               : launch_persistent(pair_kernel<false, 32, false, I8>, sh, st, g, dp, b, sh.lay, sh.G);
 }

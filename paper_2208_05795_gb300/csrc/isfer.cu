@@ -50,7 +50,7 @@ struct IsArgs {
 // ---------------------------------------------------------------------------
 // (the check pass runs over all row blocks at once, so one sample pair can
 // take more warps than Z / 32)
-template <bool QC, int DC, bool EXACT>
+template <bool QC, int DC, bool EXACT, bool FILL = true>
 __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kernel(DevCode g, DecodeParams dp, IsArgs ia,
                                                                                SlotLayout lay, int G) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kern
     const int nw = (g.n + 31) >> 5;
 
     const PairConst pc = pair_const(dp);
-    PairDecoder<QC, DC, EXACT, false> dec{g, sg, gp, pc, saddr(slot + lay.r_off)};
+    PairDecoder<QC, DC, EXACT, false, false, FILL> dec{g, sg, gp, pc, saddr(slot + lay.r_off)};
 
     for (int w = gp.gt; w < nw; w += gp.T) Tm[w] = 0u;
     gp.sync();
@@ -415,6 +415,8 @@ int is_job_start(tsx_code *code, const int32_t *ts_vars, int32_t a, const tsx_is
         else if (g.dc_max <= 8)
             e = qc ? launch_persistent(is_kernel<true, 8, false>, sh, s, g, J->dp, ik, sh.lay, sh.G)
                    : launch_persistent(is_kernel<false, 8, false>, sh, s, g, J->dp, ik, sh.lay, sh.G);
+        else if (qc && !g.row_odd)
+            e = launch_persistent(is_kernel<true, 32, false, false>, sh, s, g, J->dp, ik, sh.lay, sh.G);
         else
             e = qc ? launch_persistent(is_kernel<true, 32, false>, sh, s, g, J->dp, ik, sh.lay, sh.G)
                    : launch_persistent(is_kernel<false, 32, false>, sh, s, g, J->dp, ik, sh.lay, sh.G);

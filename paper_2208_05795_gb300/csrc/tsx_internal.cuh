@@ -32,7 +32,8 @@ struct DevCode {
     int dv_min;         // smallest variable degree (dv_min == dv_max: variable-regular)
     int by_rows;        // launch only: the two-codeword tables are c_vn of a QC code of check degree 6
     int E_odd;          // QC: edges with every row filled up to an odd number
-    int row_odd;        // 1: the two-codeword kernels' rows of large degree are so filled (0: a launch that has no room)
+    int row_odd;        // 1: the two-codeword kernels' rows of large degree are so filled (0: a launch that has no room;
+                        // messages by position then, as a general code's)
     int girth, wstart;  // wstart = max(1, girth/2)
     int n_rep;
     // QC tables

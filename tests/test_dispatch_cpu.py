@@ -1,0 +1,93 @@
+"""Which kernel a code is decoded by (csrc/decode.cu, host code), on the CPU:
+the dispatch is compiled as it stands, with launchers that only say what they
+were given.  The codes here are described by their sizes alone."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+NVCC = os.environ.get("NVCC") or ("/usr/local/cuda/bin/nvcc" if os.path.exists("/usr/local/cuda/bin/nvcc") else shutil.which("nvcc"))
+MAIN = r'''
+#include <cstdio>
+#include "decode.cu"
+namespace tsx {
+static cudaError_t say(const char *what, const DevCode &g, const LaunchShape &sh) {
+    printf("%s %d %d %d %d\n", what, g.row_odd, sh.G, sh.groups, sh.smem_bytes);
+    return cudaSuccess;
+}
+cudaError_t launch_nms16(const DevCode &g, const DecodeParams &, const EnumBuffers &, const LaunchShape &sh, bool pair,
+                         cudaStream_t) { return say(pair ? "pair" : "one", g, sh); }
+cudaError_t launch_nms16_vn(const DevCode &g, const DecodeParams &, const EnumBuffers &, const LaunchShape &sh,
+                            cudaStream_t) { return say("vn", g, sh); }
+cudaError_t launch_nms8(const DevCode &g, const DecodeParams &, const EnumBuffers &, const LaunchShape &sh, bool pair,
+                        cudaStream_t) { return say(pair ? "pair" : "one", g, sh); }
+cudaError_t launch_spa(const DevCode &g, const DecodeParams &, const EnumBuffers &, const LaunchShape &sh,
+                       cudaStream_t) { return say("one", g, sh); }
+cudaError_t launch_sieve_kernel(const DevCode &, const EnumBuffers &, const LaunchShape &, int, cudaStream_t) {
+    return cudaSuccess;
+}
+cudaError_t launch_batch16(const BatchArgs &, int, bool, int, bool, const LaunchShape &, cudaStream_t) {
+    return cudaSuccess;
+}
+cudaError_t launch_batch8(const BatchArgs &, int, bool, int, bool, const LaunchShape &, cudaStream_t) {
+    return cudaSuccess;
+}
+}
+using namespace tsx;
+// lines: decoder, rows and columns of the base, Z, least and largest row degree (rows alternate)
+int main() {
+    int dec, mb, nb, Z, dmin, dmax;
+    while (scanf("%d %d %d %d %d %d", &dec, &mb, &nb, &Z, &dmin, &dmax) == 6) {
+        DevCode g{};
+        g.kind = TSX_CODE_QC; g.n = nb * Z; g.m = mb * Z; g.Z = Z; g.n_b = nb; g.m_b = mb; g.row_odd = 1;
+        for (int i = 0; i < mb; i++) {
+            const int d = i & 1 ? dmin : dmax;
+            g.E += d * Z;
+            g.E_odd += (d | 1) * Z;
+        }
+        g.dv_max = mb; g.dv_min = 1; g.dc_max = dmax; g.dc_min = dmin;
+        DecodeParams dp{};
+        dp.decoder = dec; dp.K = 20; dp.base_llr = 16; dp.sat = dec == TSX_DEC_NMS_I8 ? 127 : 511;
+        dp.alpha_num = 3; dp.alpha_shift = 2; dp.amp_steps = 10;
+        if (dec == 100) {  // the sampling kernel
+            LaunchShape sh;
+            bool noise = false;
+            dp.decoder = TSX_DEC_NMS_I16;
+            if (plan_is_shape(g, dp, &sh, 152, &noise)) say(noise ? "noise" : "is", g, sh);
+            else printf("none 0 0 0 0\n");
+            continue;
+        }
+        const EnumBuffers b{};
+        if (launch_decode(g, dp, b, 0, 0, 0, 152, 0, 100000, nullptr) != cudaSuccess) printf("none 0 0 0 0\n");
+    }
+}
+'''
+NMS16, NMS8, SAMPLING = 0, 1, 100
+
+
+@pytest.fixture(scope="module")
+def dispatch(tmp_path_factory):
+    if not NVCC:
+        pytest.skip("no nvcc")
+    d = tmp_path_factory.mktemp("dispatch")
+    (d / "main.cu").write_text(MAIN)
+    exe = str(d / "main")
+    csrc = os.path.join(ROOT, "paper_2208_05795_gb300", "csrc")
+    subprocess.run([NVCC, "-gencode", "arch=compute_103a,code=sm_103a", "-O1", "-std=c++17", "--expt-relaxed-constexpr",
+                    "-I", os.path.join(ROOT, "include"), "-I", csrc, str(d / "main.cu"), "-o", exe], check=True, timeout=600)
+
+    def run(cases):
+        text = "".join("%d %d %d %d %d %d\n" % c for c in cases)
+        out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True, timeout=300).stdout
+        rows = [line.split() for line in out.splitlines()]
+        assert len(rows) == len(cases)
+        return [(r[0],) + tuple(int(x) for x in r[1:]) for r in rows]
+
+    return run
+
+
+@pytest.mark.parametrize("dec,mb,nb,Z", [(NMS16, 4, 28, 332), (NMS16, 4, 24, 385), (NMS16, 4, 30, 310), (NMS8, 4, 28, 494)])
+def test_codes_that_fit_two_buffers_only_with_rows_as_they_are(dispatch, dec, mb, nb, Z):
+    assert dispatch([(dec, mb, nb, Z, nb, nb)])[0][:2] == ("pair", 0)
