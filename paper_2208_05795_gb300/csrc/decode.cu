@@ -117,6 +117,18 @@ bool plan(const DevCode &g, int decoder, int kind, int G, int groups, int ctas_p
     return true;
 }
 
+// A two-codeword layout with rows filled up to an odd number of words, or as they are where only
+// that fits a CTA (4 bytes a check of even degree: full 4 x 30 bases in the variable-node-pass form
+// need it from Z = 363 to 372; the one-codeword kernel takes 58 ms for 3,000 candidates at Z = 368, this form
+// 20.3).  Sets g.row_odd.
+bool plan_rows(DevCode &g, int decoder, int kind, int G, int groups, int ctas_per_sm, int num_sms, LaunchShape *out,
+               int max_warps, long long units, bool odd_rows = false) {
+    for (g.row_odd = 1; g.row_odd >= 0; g.row_odd--)
+        if (plan(g, decoder, kind, G, groups, ctas_per_sm, num_sms, out, max_warps, units, odd_rows)) return true;
+    g.row_odd = 1;
+    return false;
+}
+
 // the launch bound of the two-codeword kernel variant launch_pair picks for g
 int pair_warps(const DevCode &g) {
     const bool reg6 = g.dc_min == 6 && g.dc_max == 6;
@@ -166,17 +178,14 @@ cudaError_t launch_decode(const DevCode &g0, const DecodeParams &dp, const EnumB
     bool pair = false;
     if (try_pair) {
         g.by_rows = rows_table(g, dp.decoder, kLayPair, num_sms, pair_warps(g), units);
-        pair = plan(g, dp.decoder, kLayPair, G, groups, ctas_per_sm, num_sms, &sh, pair_warps(g), units);
-        if (!pair) {  // without the filled-up rows
-            g.row_odd = 0;
-            pair = plan(g, dp.decoder, kLayPair, G, groups, ctas_per_sm, num_sms, &sh, pair_warps(g), units);
-            if (!pair) g.row_odd = 1;
-        }
+        const auto fits = [&](int kind) {
+            return plan_rows(g, dp.decoder, kind, G, groups, ctas_per_sm, num_sms, &sh, pair_warps(g), units);
+        };
+        pair = fits(kLayPair);
+        // QC codes of large check degree whose two-buffer layout does not fit: the variable-node-pass form
+        if (!pair && g.kind == TSX_CODE_QC && dp.decoder == TSX_DEC_NMS_I16 && g.dc_max > 8 && fits(kLayPairVn))
+            return launch_nms16_vn(g, dp, b, sh, st);
     }
-    // QC codes of large check degree whose two-buffer layout does not fit: the variable-node-pass form
-    if (!pair && try_pair && g.kind == TSX_CODE_QC && dp.decoder == TSX_DEC_NMS_I16 &&
-        g.dc_max > 8 && plan(g, dp.decoder, kLayPairVn, G, groups, ctas_per_sm, num_sms, &sh, pair_warps(g), units))
-        return launch_nms16_vn(g, dp, b, sh, st);
     const int sw = scalar_warps(dp.decoder == TSX_DEC_SPA_F32, g.dc_max);
     if (!pair && !plan(g, dp.decoder, kLayScalar, G, groups, ctas_per_sm, num_sms, &sh, sw, n_cand))
         return cudaErrorInvalidConfiguration;

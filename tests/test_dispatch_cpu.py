@@ -88,6 +88,13 @@ def dispatch(tmp_path_factory):
     return run
 
 
+@pytest.mark.parametrize("mb,nb,Z", [(4, 30, 363), (4, 30, 368), (4, 30, 371), (4, 28, 392), (4, 24, 455), (4, 22, 500),
+                                     (4, 20, 550), (4, 16, 680), (4, 10, 1080), (3, 20, 690), (3, 12, 1140), (5, 16, 560),
+                                     (6, 14, 560)])
+def test_codes_that_fit_the_variable_node_pass_form_only_with_rows_as_they_are(dispatch, mb, nb, Z):
+    assert dispatch([(NMS16, mb, nb, Z, nb, nb)])[0][:2] == ("vn", 0)
+
+
 @pytest.mark.parametrize("dec,mb,nb,Z", [(NMS16, 4, 28, 332), (NMS16, 4, 24, 385), (NMS16, 4, 30, 310), (NMS8, 4, 28, 494)])
 def test_codes_that_fit_two_buffers_only_with_rows_as_they_are(dispatch, dec, mb, nb, Z):
     assert dispatch([(dec, mb, nb, Z, nb, nb)])[0][:2] == ("pair", 0)

@@ -17,6 +17,12 @@ def _both(code, **more):
     return tsx.ts_list_view(tsx.enumerate_ts(code, kernel=2, **p)), tsx.ts_list_view(tsx.enumerate_ts(code, kernel=1, **p))
 
 
+@pytest.mark.parametrize("mb,nb,Z", [(4, 30, 363), (4, 30, 368), (4, 30, 371), (4, 28, 392), (4, 24, 455), (4, 16, 680),
+                                     (4, 10, 1080), (3, 12, 1140)])
+def test_variable_node_pass_form(mb, nb, Z):
+    _same(*_both(tsx.load_code(_qc(mb, nb, Z, 60 + nb))))
+
+
 @pytest.mark.parametrize("mb,nb,Z,decoder", [(4, 28, 332, "nms16"), (4, 24, 385, "nms16"), (4, 30, 310, "nms16"),
                                              (4, 28, 494, "nms8")])
 def test_two_buffer_form(mb, nb, Z, decoder):
