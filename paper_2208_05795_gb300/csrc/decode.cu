@@ -25,14 +25,17 @@ namespace {
 enum { kLayScalar = 0, kLayPair = 1, kLaySieve = 2, kLayIs = 3, kLayPairVn = 4 };
 
 int msg_bytes(int decoder) { return decoder == TSX_DEC_NMS_I8 ? 1 : (decoder == TSX_DEC_SPA_F32 ? 4 : 2); }
+constexpr int kPairMiscBytes = 464;  // the two-codeword kernels' scratch where there is room
+static_assert(sizeof(PairMisc) <= kPairMiscBytes, "the two-codeword kernels' scratch");
 int post_bytes(int decoder) { return decoder == TSX_DEC_SPA_F32 ? 4 : 2; }
 
 // odd_rows: the two-codeword kernels' variant for check degrees above 8 (QC: each row an odd number of words)
 // noise: the sampling kernel keeps the noise on the set's nodes
-SlotLayout make_layout(const DevCode &g, int decoder, int kind, bool odd_rows, bool noise) {
+// tight: nothing to spare, for a code that fits a CTA only so (plan)
+SlotLayout make_layout(const DevCode &g, int decoder, int kind, bool odd_rows, bool noise, bool tight) {
     SlotLayout L{};
     L.tables_bytes = al16(tab_offsets(g, kind == kLayPairVn ? 2 : kind == kLayPair || kind == kLayIs ? 1 : 0).total);
-    const int nw = (g.n + 31) / 32;
+    const int nw = (g.n + 31) / 32, nx = tight ? nw : (nw + 3) & ~3;
     // message slots: QC edges, or the position-major m x dc_max grid of a CSR code
     const int nmsg = g.kind == TSX_CODE_QC ? g.E : g.m * g.dc_max;
     const int nmsg2 = g.kind == TSX_CODE_QC && odd_rows && g.row_odd ? g.E_odd : nmsg;
@@ -44,16 +47,14 @@ SlotLayout make_layout(const DevCode &g, int decoder, int kind, bool odd_rows, b
         L.xb_off = x; x += al16(nw * 4);
     } else if (kind == kLayPair) {
         const int rsz = decoder == TSX_DEC_NMS_I8 ? 2 : 4;
-        const int xstride = (nw + 3) & ~3;
         L.r_off = x; x += al16(nmsg2 * rsz);
         L.p_off = x; x += al16(2 * g.n * 4);  // current and accumulating posteriors
-        L.xa_off = x; x += al16(4 * xstride * 4);
+        L.xa_off = x; x += al16(4 * nx * 4);
         L.xb_off = L.xa_off;
     } else if (kind == kLayPairVn) {
-        const int xstride = (nw + 3) & ~3;
         L.r_off = x; x += al16(nmsg2 * 4);
         L.p_off = x; x += al16(g.n * 4);  // one posterior buffer, rebuilt by the variable-node pass
-        L.xa_off = x; x += al16(4 * xstride * 4);
+        L.xa_off = x; x += al16(4 * nx * 4);
         L.xb_off = L.xa_off;
     } else if (kind == kLayIs) {
         L.r_off = x; x += al16(nmsg2 * 4);
@@ -69,8 +70,9 @@ SlotLayout make_layout(const DevCode &g, int decoder, int kind, bool odd_rows, b
         L.xb_off = L.xa_off;
     }
     const bool pair = kind == kLayPair || kind == kLayPairVn;
+    if (!tight && (pair || kind == kLayIs) && g.kind == TSX_CODE_QC && !g.by_rows) L.tables_bytes += al16(4 * g.m_b);
     L.misc_off = x;
-    x += al16((int)(pair ? sizeof(PairMisc) : kind == kLayIs ? kIsMiscBytes : kind == kLaySieve ? sizeof(SieveMisc)
+    x += al16((int)(pair ? (tight ? sizeof(PairMisc) : kPairMiscBytes) : kind == kLayIs ? kIsMiscBytes : kind == kLaySieve ? sizeof(SieveMisc)
                                                                                                : sizeof(Misc)));
     L.slot_bytes = x;
     return L;
@@ -86,9 +88,15 @@ bool plan(const DevCode &g, int decoder, int kind, int G, int groups, int ctas_p
           LaunchShape *out, int max_warps = 16, long long units = 0, bool odd_rows = false,
           bool noise = true) {
     LaunchShape sh{};
-    sh.lay = make_layout(g, decoder, kind, odd_rows || g.dc_max > 8, noise);
-    const int room = kSmemCta - sh.lay.tables_bytes;
-    const int fit = room / sh.lay.slot_bytes;
+    // With a little room to spare in each slot (up to 200 bytes), or without where only that fits.  The
+    // shapes below were measured with it; a group more from so few bytes can take half of the others' warps
+    // (sum-product, 12 groups of two warps: 43 ms, 13 of one: 62).
+    int fit = 0;
+    for (int tight = 0; tight < 2 && fit < 1; tight++) {
+        sh.lay = make_layout(g, decoder, kind, odd_rows || g.dc_max > 8, noise, tight);
+        const int room = kSmemCta - sh.lay.tables_bytes;
+        fit = room >= sh.lay.slot_bytes ? room / sh.lay.slot_bytes : 0;
+    }
     if (fit < 1) return false;
     if (kind == kLaySieve) G = 1;
     if (G <= 0) {
@@ -119,7 +127,7 @@ bool plan(const DevCode &g, int decoder, int kind, int G, int groups, int ctas_p
 
 // A two-codeword layout with rows filled up to an odd number of words, or as they are where only
 // that fits a CTA (4 bytes a check of even degree: full 4 x 30 bases in the variable-node-pass form
-// need it from Z = 363 to 372; the one-codeword kernel takes 58 ms for 3,000 candidates at Z = 368, this form
+// need it from Z = 364 to 372; the one-codeword kernel takes 58 ms for 3,000 candidates at Z = 368, this form
 // 20.3).  Sets g.row_odd.
 bool plan_rows(DevCode &g, int decoder, int kind, int G, int groups, int ctas_per_sm, int num_sms, LaunchShape *out,
                int max_warps, long long units, bool odd_rows = false) {

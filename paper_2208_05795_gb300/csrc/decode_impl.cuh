@@ -53,7 +53,7 @@ __host__ __device__ inline int al16(int x) { return (x + 15) & ~15; }
 __host__ __device__ inline int rt_row(const DevCode &g) { return (g.dc_max + 1) & ~1; }
 
 struct TabOff {
-    int rdeg, reoff, rjz, rs, rt, roff, ct, cdeg, ceoff, cs, ciz;
+    int rdeg, reoff, rjz, rs, rt, ct, cdeg, ceoff, cs, ciz;
     int c_ptr, c_vn, v_ptr, v_edge;
     int total;
 };
@@ -75,7 +75,6 @@ __host__ __device__ inline TabOff tab_offsets(const DevCode &g, int pair = 0) {
         o.reoff = x; x += al16(g.m_b * 4);
         if (pair) {
             o.rt = x; x += al16(g.m_b * rt_row(g) * 8);
-            o.roff = x; x += al16(g.m_b * 4);
             if (pair == 2) { o.ct = x; x += al16(g.n_b * g.dv_max * 8); }
         } else {
             o.rjz = x; x += al16(g.m_b * g.dc_max * 4);
@@ -99,10 +98,10 @@ __host__ __device__ inline TabOff tab_offsets(const DevCode &g, int pair = 0) {
 
 struct SGraph {
     const int16_t *rdeg;
-    const int32_t *reoff, *rjz;
+    const int32_t *reoff;  // [m_b] first message of a row block (filled-up rows: see load_tables)
+    const int32_t *rjz;
     // two-codeword kernels
     const int2 *rt;       // [m_b * rt_row] {4 rjz, 4 rs}
-    const int32_t *roff;  // [m_b] first message of a row block, rows of an odd number of words
     const int2 *ct;       // [n_b * dv_max] {message offset, words a row | shift << 8} of the t-th block of a column
                           // (variable-node-pass form only)
     const int16_t *rs, *cdeg;
@@ -135,7 +134,8 @@ __device__ void copy_bytes(void *dst, const void *src, int bytes) {
     }
 }
 
-__device__ SGraph load_tables(const DevCode &g, unsigned char *sm, int pair = 0) {
+// filled (QC, two-codeword kernels): the row blocks start where rows of an odd number of words put them
+__device__ SGraph load_tables(const DevCode &g, unsigned char *sm, int pair = 0, bool filled = false) {
     TabOff o = tab_offsets(g, pair);
     SGraph s{};
     if (pair && g.by_rows) {
@@ -149,7 +149,8 @@ __device__ SGraph load_tables(const DevCode &g, unsigned char *sm, int pair = 0)
     }
     if (g.kind == TSX_CODE_QC) {
         copy_bytes(sm + o.rdeg, g.rdeg, g.m_b * 2);
-        copy_bytes(sm + o.reoff, g.reoff, g.m_b * 4);
+        int *reoff = (int *)(sm + o.reoff);
+        for (int i = threadIdx.x; i < g.m_b; i += blockDim.x) reoff[i] = filled ? row_offset(g, i) : g.reoff[i];
         if (pair) {
             int2 *rt = (int2 *)(sm + o.rt);
             const int row = rt_row(g);
@@ -158,20 +159,17 @@ __device__ SGraph load_tables(const DevCode &g, unsigned char *sm, int pair = 0)
                 rt[i * row + x - i * g.dc_max] = make_int2(4 * g.rjz[x], 4 * (int)g.rs[x]);
             }
             s.rt = rt;
-            int *roff = (int *)(sm + o.roff);
-            for (int i = threadIdx.x; i < g.m_b; i += blockDim.x) roff[i] = row_offset(g, i);
             if (pair == 2) {
                 int2 *ct = (int2 *)(sm + o.ct);
                 for (int x = threadIdx.x; x < g.n_b * g.dv_max; x += blockDim.x) {
                     const int j = x / g.dv_max;
                     if (x - j * g.dv_max >= g.cdeg[j]) continue;
                     const int i = g.ciz[x] / g.Z, p = (g.ceoff[x] - g.reoff[i]) / g.Z;
-                    ct[x] = g.row_odd ? make_int2(row_offset(g, i) + p, (g.rdeg[i] | 1) | ((int)g.cs[x] << 8))
-                                      : make_int2(g.ceoff[x], 1 | ((int)g.cs[x] << 8));
+                    ct[x] = filled ? make_int2(row_offset(g, i) + p, (g.rdeg[i] | 1) | ((int)g.cs[x] << 8))
+                                   : make_int2(g.ceoff[x], 1 | ((int)g.cs[x] << 8));
                 }
                 s.ct = ct;
             }
-            s.roff = roff;
         } else {
             copy_bytes(sm + o.rjz, g.rjz, g.m_b * g.dc_max * 4);
             copy_bytes(sm + o.rs, g.rs, g.m_b * g.dc_max * 2);
@@ -186,7 +184,7 @@ __device__ SGraph load_tables(const DevCode &g, unsigned char *sm, int pair = 0)
         }
         copy_bytes(sm + o.cdeg, g.cdeg, g.n_b * 2);
         s.rdeg = (const int16_t *)(sm + o.rdeg);
-        s.reoff = (const int32_t *)(sm + o.reoff);
+        s.reoff = reoff;
         s.cdeg = (const int16_t *)(sm + o.cdeg);
     } else {
         copy_bytes(sm + o.c_ptr, g.c_ptr, (g.m + 1) * 2);
@@ -209,7 +207,7 @@ __device__ SGraph load_tables(const DevCode &g, unsigned char *sm, int pair = 0)
 // ---------------------------------------------------------------------------
 struct Grp {
     int G, T, gt, lane, gw, bar;
-    int *red;  // reduction scratch (shared): [0, 32) for sum(), [32, 64) for sum_pass()
+    int *red;  // reduction scratch (shared): G words for sum(), from kMaxGroupWarps on for sum_pass()
     // Both forms are volatile asm statements with a memory clobber: the two-codeword kernels read
     // shared memory by volatile asm without one, and what was written by ordinary stores has to be
     // ordered before such reads (and ordinary stores after them) in the source already; __syncwarp() is
@@ -238,9 +236,9 @@ struct Grp {
             sync();
             return x;
         }
-        if (lane == 0) red[32 + gw] = x;
+        if (lane == 0) red[kMaxGroupWarps + gw] = x;
         sync();
-        return __reduce_add_sync(0xffffffffu, lane < G ? red[32 + lane] : 0);
+        return __reduce_add_sync(0xffffffffu, lane < G ? red[kMaxGroupWarps + lane] : 0);
     }
 };
 

@@ -147,18 +147,20 @@ struct PairConst {
 // Schedule state of one half, in the group's shared memory: written by the
 // group's thread 0 where a decode ends, read by the others after a barrier.
 // (Held in every thread's registers it cost 30 of them, and every warp ran
-// the bookkeeping.)
+// the bookkeeping.)  Narrow types: what the slot takes beyond a code's words decides
+// whether codes at the shared-memory limit run two codewords a lane.
 struct HalfS {
     long long idx;       // candidate (absolute index), -1: idle
     long long copy_o;    // record of the finished candidate whose x* is to be copied out, -1: none
-    int I[4], nI;        // impulse nodes
-    int lo, hi, st, phase;  // bisection
-    int ndec, nit, failed;
-    int Limp;            // channel LLR of the impulse nodes in the current decode
+    int lo, hi;          // bisection
+    int nit;
     int K;               // iteration limit of the candidate
-    int keep;            // x buffer (0/1) of the last failing decode; the current decode writes the other
-    int copy;            // x buffer to copy out
-    int fail;            // the decode that ended failed
+    int16_t I[4];        // impulse nodes (n < 2^15)
+    int16_t Limp;        // channel LLR of the impulse nodes in the current decode (|Limp| <= sat < 2^13)
+    uint8_t nI, st, phase, ndec, failed;  // (at most 21 decodes a candidate)
+    uint8_t keep;        // x buffer (0/1) of the last failing decode; the current decode writes the other
+    uint8_t copy;        // x buffer to copy out
+    uint8_t fail;        // the decode that ended failed
 };
 
 __device__ __forceinline__ PairConst pair_const(const DecodeParams &dp) {
@@ -171,7 +173,9 @@ __device__ __forceinline__ PairConst pair_const(const DecodeParams &dp) {
     return pc;
 }
 
-struct PairMisc : Misc {
+struct PairMisc {
+    int red[2 * kMaxGroupWarps];
+    unsigned long long okd, okit;  // converged decodes of this group and their iterations
     HalfS h[2];
 };
 
@@ -477,7 +481,7 @@ struct PairDecoder {
                                                    [&](int p) { return ra + (unsigned)p * rs; });
                     } else if constexpr (FILL) {
                         u += node_twopass<MASK>(deg, km, writeR, Pc, Pn, pv, pv2,
-                                                Rb + (unsigned)((sg.roff[i] + r * (deg | 1)) * RSZ), Int<RSZ>{});
+                                                Rb + (unsigned)((sg.reoff[i] + r * (deg | 1)) * RSZ), Int<RSZ>{});
                     } else {
                         u += node_twopass<MASK>(deg, km, writeR, Pc, Pn, pv, pv2, Rb + (unsigned)((sg.reoff[i] + r) * RSZ),
                                                 (unsigned)(Z * RSZ));
@@ -631,7 +635,6 @@ __device__ __forceinline__ void pair_run(const DevCode &g, const DecodeParams &d
     unsigned *Pbuf = (unsigned *)(slot + lay.p_off);  // [2][n] ([n] in the VN form)
     const int nw = (g.n + 31) >> 5;
     uint32_t *xb = (uint32_t *)(slot + lay.xa_off);  // 4 buffers of nw words: [half][2]
-    const int xstride = (nw + 3) & ~3;
 
     const PairConst pc = pair_const(dp);
     PairDecoder<QC, DC, EXACT, I8, VN, FILL> dec{g, sg, gp, pc, saddr(slot + lay.r_off)};
@@ -653,11 +656,11 @@ __device__ __forceinline__ void pair_run(const DevCode &g, const DecodeParams &d
         }
         const int4 I4 = b.cands[idx];
         h.idx = idx;
-        h.I[0] = I4.x; h.I[1] = I4.y; h.I[2] = I4.z; h.I[3] = I4.w;
+        h.I[0] = (int16_t)I4.x; h.I[1] = (int16_t)I4.y; h.I[2] = (int16_t)I4.z; h.I[3] = (int16_t)I4.w;
         h.nI = (I4.x >= 0) + (I4.y >= 0) + (I4.z >= 0) + (I4.w >= 0);
         h.lo = 0; h.hi = amax; h.st = 0; h.phase = 0;
         h.ndec = 0; h.nit = 0; h.failed = 0;
-        h.Limp = clampi(dp.base_llr - amax, -dp.sat, dp.sat);
+        h.Limp = (int16_t)clampi(dp.base_llr - amax, -dp.sat, dp.sat);
         h.K = cand_limit(dp, b, idx);
     };
     // the candidate's records; its x* is copied out by the whole group afterwards
@@ -681,7 +684,7 @@ __device__ __forceinline__ void pair_run(const DevCode &g, const DecodeParams &d
     auto next_amp = [&](HalfS &h) {
         if (h.st < dp.amp_steps && h.hi - h.lo > 1) {
             h.st++;
-            h.Limp = clampi(dp.base_llr - ((h.lo + h.hi) >> 1), -dp.sat, dp.sat);
+            h.Limp = (int16_t)clampi(dp.base_llr - ((h.lo + h.hi) >> 1), -dp.sat, dp.sat);
         } else {
             finish(h);
         }
@@ -834,7 +837,7 @@ __device__ __forceinline__ void pair_run(const DevCode &g, const DecodeParams &d
             const bool end_now = u == 0 || k[hh] == K[hh];
             if ((k[hh] >= g.wstart && u < ub[hh]) || (end_now && k[hh] < g.wstart)) {
                 ub[hh] = u;
-                dec.save_x(Pc, hh, xb + (2 * hh + (hs[hh].keep ^ 1)) * xstride);
+                dec.save_x(Pc, hh, xb + (2 * hh + (hs[hh].keep ^ 1)) * nw);
                 read_pc = true;
             }
             if (end_now) {
@@ -862,7 +865,7 @@ __device__ __forceinline__ void pair_run(const DevCode &g, const DecodeParams &d
                 if (!ended[hh]) continue;
                 const long long o = hs[hh].copy_o;
                 if (o >= 0) {  // x* of the candidate that ended (its buffer is not written before the next barrier)
-                    const uint32_t *src = xb + (2 * hh + hs[hh].copy) * xstride;
+                    const uint32_t *src = xb + (2 * hh + hs[hh].copy) * nw;
                     uint32_t *dst = b.xstar + o * (long long)b.nw;
                     for (int w = gp.gt; w < nw; w += gp.T) dst[w] = src[w];
                 }
@@ -907,7 +910,7 @@ template <bool QC, int DC, bool EXACT, bool I8, bool FILL = true>
 __global__ void __launch_bounds__(32 * pair_kernel_warps(DC, EXACT), 1)
     pair_kernel(DevCode g, DecodeParams dp, EnumBuffers b, SlotLayout lay, int G) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const SGraph sg = load_tables(g, smem, true);
+    const SGraph sg = load_tables(g, smem, 1, DC > 8 && FILL);
     __syncthreads();
     pair_run<QC, DC, EXACT, I8, false, FILL>(g, dp, b, lay, G, sg, smem, (threadIdx.x >> 5) / G);
 }
@@ -917,7 +920,7 @@ template <bool I8, bool FILL>
 __global__ void __launch_bounds__(32 * pair_kernel_warps(32, false), 1) pair_vn_kernel(DevCode g, DecodeParams dp, EnumBuffers b,
                                                                SlotLayout lay, int G) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const SGraph sg = load_tables(g, smem, 2);
+    const SGraph sg = load_tables(g, smem, 2, FILL);
     __syncthreads();
     pair_run<true, 32, false, I8, true, FILL>(g, dp, b, lay, G, sg, smem, (threadIdx.x >> 5) / G);
 }
@@ -934,7 +937,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 1) batch_kernel(const __grid
     extern __shared__ __align__(16) unsigned char smem[];
     for (int c = 0; c < n_items; c++) {
         const BatchItem &it = args.it[c];
-        const SGraph sg = load_tables(it.g, smem, true);
+        const SGraph sg = load_tables(it.g, smem, 1, DC > 8);
         __syncthreads();
         const int grp = (threadIdx.x >> 5) / it.G;
         if (grp < it.groups) pair_run<QC, DC, EXACT, I8>(it.g, it.dp, it.b, it.lay, it.G, sg, smem, grp);

@@ -54,7 +54,7 @@ template <bool QC, int DC, bool EXACT, bool FILL = true>
 __global__ void __launch_bounds__(QC && DC > 8 ? 32 * kIsWarps : 512, 1) is_kernel(DevCode g, DecodeParams dp, IsArgs ia,
                                                                                SlotLayout lay, int G) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const SGraph sg = load_tables(g, smem, true);
+    const SGraph sg = load_tables(g, smem, 1, DC > 8 && FILL);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int grp = warp / G;

@@ -90,6 +90,11 @@ constexpr int kBatchWarps = 20;
 constexpr int kIsWarps = 24;
 // its groups' shared scratch, and the room for the noise on the set's nodes (isfer.cu)
 constexpr int kIsMiscBytes = 320, kIsNoiseBytes = 512;
+// warps in a group, at most (the 32-warp form of the sum-product kernel has groups of one)
+constexpr int kMaxGroupWarps = 24;
+static_assert(pair_kernel_warps(32, false) <= kMaxGroupWarps && pair_kernel_warps(6, true) <= kMaxGroupWarps &&
+              scalar_warps(true, 8) <= kMaxGroupWarps && kBatchWarps <= kMaxGroupWarps && kIsWarps <= kMaxGroupWarps,
+              "the groups' reduction scratch");
 struct BatchArgs {
     BatchItem it[kMaxBatch];
 };

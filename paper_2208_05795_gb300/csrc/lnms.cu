@@ -52,6 +52,7 @@ struct LnmsArgs {
 
 // warps per CTA of the two-frame kernel (its launch bound); 16, 20 and 28 measured within 7 %
 constexpr int kLnmsWarps = 24;
+static_assert(kLnmsWarps <= kMaxGroupWarps, "the groups' reduction scratch");
 
 struct LnmsLayout {
     int tables_bytes, p_off, r_off, misc_off, slot_bytes;
@@ -208,7 +209,7 @@ __global__ void __launch_bounds__(512, 1) lnms_kernel(DevCode g, LnmsArgs a, Lnm
 // per frame).
 __global__ void __launch_bounds__(32 * kLnmsWarps, 1) lnms_pair_kernel(DevCode g, LnmsArgs a, SlotLayout lay, int G) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const SGraph sg = load_tables(g, smem, true);
+    const SGraph sg = load_tables(g, smem, 1, true);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int grp = warp / G;
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(32 * kLnmsWarps, 1) lnms_pair_kernel(DevCode g
             const unsigned rt = rt0 + 8u * (unsigned)(i * rt_row(g));
             for (int r = gp.gt; r < Z; r += gp.T) {
                 const unsigned r4 = 4u * (unsigned)r;
-                const unsigned ra = Ra + 4u * (unsigned)(sg.roff[i] + r * (deg | 1));
+                const unsigned ra = Ra + 4u * (unsigned)(sg.reoff[i] + r * (deg | 1));
                 unsigned sx = 0, M1 = 0, M2 = 0;  // the two largest beta - |q|
                 // q = sat(P - r), left in the message's word
                 auto first = [&](auto width, int p) {
@@ -457,7 +458,7 @@ struct LnmsShape {
 bool lnms_pair_shape(const DevCode &g, const LnmsArgs &a, int num_sms, LaunchShape *sh) {
     if ((long long)a.an * a.lim_v2c > 0xFFFF) return false;
     SlotLayout L{};
-    L.tables_bytes = al16(tab_offsets(g, true).total);
+    L.tables_bytes = al16(tab_offsets(g, 1).total) + al16(4 * g.m_b);  // (the measured shapes' sizes: see plan())
     int x = 0;
     L.r_off = x; x += al16(4 * g.E_odd);
     L.p_off = x; x += al16(4 * g.n);

@@ -88,7 +88,7 @@ def dispatch(tmp_path_factory):
     return run
 
 
-@pytest.mark.parametrize("mb,nb,Z", [(4, 30, 363), (4, 30, 368), (4, 30, 371), (4, 28, 392), (4, 24, 455), (4, 22, 500),
+@pytest.mark.parametrize("mb,nb,Z", [(4, 30, 365), (4, 30, 368), (4, 30, 371), (4, 28, 392), (4, 24, 455), (4, 22, 500),
                                      (4, 20, 550), (4, 16, 680), (4, 10, 1080), (3, 20, 690), (3, 12, 1140), (5, 16, 560),
                                      (6, 14, 560)])
 def test_codes_that_fit_the_variable_node_pass_form_only_with_rows_as_they_are(dispatch, mb, nb, Z):
@@ -98,3 +98,27 @@ def test_codes_that_fit_the_variable_node_pass_form_only_with_rows_as_they_are(d
 @pytest.mark.parametrize("dec,mb,nb,Z", [(NMS16, 4, 28, 332), (NMS16, 4, 24, 385), (NMS16, 4, 30, 310), (NMS8, 4, 28, 494)])
 def test_codes_that_fit_two_buffers_only_with_rows_as_they_are(dispatch, dec, mb, nb, Z):
     assert dispatch([(dec, mb, nb, Z, nb, nb)])[0][:2] == ("pair", 0)
+
+
+def _two_codeword_bytes(mb, nb, Z, posteriors, msg):
+    """Shared memory that suffices for a pair of codewords of a full base: the messages, one or two posterior
+    buffers, four error patterns, 336 bytes of scratch, and the tables."""
+    def up(x):
+        return (x + 15) // 16 * 16
+
+    n, E = nb * Z, mb * nb * Z
+    tables = up(2 * mb) + up(4 * mb) + up(4 * mb * nb) + up(2 * mb * nb) + up(2 * nb)
+    tables += up(4 * nb * mb) + up(2 * nb * mb) + up(4 * nb * mb)
+    words = ((n + 31) // 32 + 3) // 4 * 4
+    return up(tables) + up(msg * E) + up(4 * posteriors * n) + 16 * words + 336
+
+
+@pytest.mark.parametrize("mb", range(2, 9))
+def test_every_code_with_room_for_two_codewords_has_them(dispatch, mb):
+    cases = []
+    for nb in range(mb + 1, 33):
+        for dec, posteriors, msg in ((NMS16, 1 if nb > 8 else 2, 4), (NMS8, 2, 2)):
+            Z = max(z for z in range(1, 32767 // nb + 1) if _two_codeword_bytes(mb, nb, z, posteriors, msg) <= 226 * 1024)
+            cases += [(dec, mb, nb, z, nb, nb) for z in range(Z - 3, Z + 1)]
+    for c, got in zip(cases, dispatch(cases)):
+        assert got[0] in ("pair", "vn"), (c, got)
