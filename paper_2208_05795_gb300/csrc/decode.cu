@@ -227,7 +227,8 @@ bool plan_batch(const DevCode *const *g, const DecodeParams *dp, const EnumBuffe
         LaunchShape sh;
         int G, groups;
         items[i].scalar = 0;
-        if (!plan(*g[i], dec, kLayPair, 1, 1, 0, num_sms, &sh, kBatchWarps, 0, odd)) {
+        DevCode gi = *g[i];
+        if (!plan_rows(gi, dec, kLayPair, 1, 1, 0, num_sms, &sh, kBatchWarps, 0, odd)) {
             items[i].scalar = 1;  // decoded by a launch of its own
             continue;
         }
@@ -235,16 +236,16 @@ bool plan_batch(const DevCode *const *g, const DecodeParams *dp, const EnumBuffe
         if (g[i]->dc_max > dcmax) dcmax = g[i]->dc_max;
         if (G_req && G_req[i] > 0) {
             // the requested (tuned) group width, as many groups as fit
-            if (!plan(*g[i], dec, kLayPair, G_req[i], 0, 0, num_sms, &sh, kBatchWarps, 0, odd)) return false;
+            if (!plan_rows(gi, dec, kLayPair, G_req[i], 0, 0, num_sms, &sh, kBatchWarps, 0, odd)) return false;
             G = sh.G;
             groups = sh.groups;
         } else {
             // the single-code launch's automatic shape
-            if (!plan(*g[i], dec, kLayPair, 0, 0, 0, num_sms, &sh, kBatchWarps, 0, odd)) return false;
+            if (!plan_rows(gi, dec, kLayPair, 0, 0, 0, num_sms, &sh, kBatchWarps, 0, odd)) return false;
             G = sh.G;
             groups = sh.groups;
         }
-        items[i].g = *g[i];
+        items[i].g = gi;
         items[i].dp = dp[i];
         items[i].b = b[i];
         items[i].lay = sh.lay;

@@ -937,10 +937,18 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 1) batch_kernel(const __grid
     extern __shared__ __align__(16) unsigned char smem[];
     for (int c = 0; c < n_items; c++) {
         const BatchItem &it = args.it[c];
-        const SGraph sg = load_tables(it.g, smem, 1, DC > 8);
+        const bool filled = DC > 8 && it.g.row_odd;
+        const SGraph sg = load_tables(it.g, smem, 1, filled);
         __syncthreads();
         const int grp = (threadIdx.x >> 5) / it.G;
-        if (grp < it.groups) pair_run<QC, DC, EXACT, I8>(it.g, it.dp, it.b, it.lay, it.G, sg, smem, grp);
+        if (grp < it.groups) {
+            if constexpr (QC && DC > 8) {
+                if (!filled) pair_run<QC, DC, EXACT, I8, false, false>(it.g, it.dp, it.b, it.lay, it.G, sg, smem, grp);
+                else pair_run<QC, DC, EXACT, I8>(it.g, it.dp, it.b, it.lay, it.G, sg, smem, grp);
+            } else {
+                pair_run<QC, DC, EXACT, I8>(it.g, it.dp, it.b, it.lay, it.G, sg, smem, grp);
+            }
+        }
         __syncthreads();
     }
 }

@@ -60,11 +60,25 @@ int main() {
             continue;
         }
         const EnumBuffers b{};
+        if (dec >= 200) {  // in a multi-code launch with itself
+            dp.decoder = dec - 200;
+            dp.sat = dp.decoder == TSX_DEC_NMS_I8 ? 127 : 511;
+            const DevCode *const gs[2] = {&g, &g};
+            const DecodeParams dps[2] = {dp, dp};
+            const EnumBuffers bs[2] = {};
+            static BatchItem it[2];
+            LaunchShape sh;
+            int variant = 0;
+            if (!plan_batch(gs, dps, bs, nullptr, 2, 152, it, &sh, &variant)) printf("none 0 0 0 0\n");
+            else if (it[1].scalar) printf("own 0 0 0 0\n");
+            else printf("batch %d %d %d %d\n", it[1].g.row_odd, it[1].G, it[1].groups, sh.smem_bytes);
+            continue;
+        }
         if (launch_decode(g, dp, b, 0, 0, 0, 152, 0, 100000, nullptr) != cudaSuccess) printf("none 0 0 0 0\n");
     }
 }
 '''
-NMS16, NMS8, SAMPLING = 0, 1, 100
+NMS16, NMS8, SAMPLING, BATCH = 0, 1, 100, 200
 
 
 @pytest.fixture(scope="module")
@@ -122,3 +136,14 @@ def test_every_code_with_room_for_two_codewords_has_them(dispatch, mb):
             cases += [(dec, mb, nb, z, nb, nb) for z in range(Z - 3, Z + 1)]
     for c, got in zip(cases, dispatch(cases)):
         assert got[0] in ("pair", "vn"), (c, got)
+
+
+@pytest.mark.parametrize("mb", range(2, 9))
+def test_a_code_decoded_with_two_buffers_is_in_the_multi_code_launch(dispatch, mb):
+    """Each of them, alone and in a batch (the batch has one launch bound more or less, so shapes may differ)."""
+    cases = [(dec, mb, nb, Z, nb, nb) for nb in range(mb + 1, 33) for dec in (NMS16, NMS8)
+             for Z in range(30, 32767 // nb + 1, 3 if nb > 8 else 40)]
+    alone = dispatch(cases)
+    batch = dispatch([(BATCH + c[0],) + c[1:] for c in cases])
+    assert [b[0] == "batch" for b in batch] == [a[0] == "pair" for a in alone]
+    assert [b[1] for b in batch if b[0] == "batch"] == [a[1] for a in alone if a[0] == "pair"]

@@ -39,3 +39,15 @@ def test_sampling_rate_beside_the_line(mb, nb, filled, unfilled):
         kw = dict(ebn0_db=3.5, n_samples=3000, job_key=3, K=20)
         rate.append(max(r["edge_updates"] / r["ms"] for r in (tsx.is_fer_estimate(code, [0, 5, 9], **kw) for _ in range(3))))
     assert rate[1] > 0.5 * rate[0]
+
+
+@pytest.mark.parametrize("decoder", ["nms16", "nms8"])
+def test_in_a_batch(decoder):
+    shapes = [(4, 28, 332), (4, 9, 50), (4, 24, 385)] if decoder == "nms16" else [(4, 28, 494), (4, 9, 50)]
+    codes = [tsx.load_code(_qc(*s, 90)) for s in shapes]
+    p = dict(P, cand_end=120, decoder=decoder, **({"sat": 127} if decoder == "nms8" else {}))
+    b = tsx.batch_create(codes, p)
+    assert b.decode_launches == 1
+    tsx.batch_run(b)
+    for i, c in enumerate(codes):
+        _same(tsx.batch_view(b, i), tsx.ts_list_view(tsx.enumerate_ts(c, kernel=1, **p)))
