@@ -14,6 +14,7 @@
 
 #include "banks.h"
 #include "kernels.cuh"
+#include "rows.h"
 
 using namespace tsx;
 
@@ -1076,6 +1077,16 @@ extern "C" int ts_list_stats(tsx_ts_list *L, tsx_enum_stats *stats) {
     return TSX_OK;
 }
 
+// rows of a list's buffers to the host
+static cudaError_t fetch_rows(int *dst, const void *src, size_t pitch, size_t width, size_t rows) {
+    return (cudaError_t)copy_rows(
+        dst, src, pitch, width, rows,
+        [](void *d, size_t dp, const void *s, size_t sp, size_t w, size_t n) {
+            return (int)cudaMemcpy2D(d, dp, s, sp, w, n, cudaMemcpyDeviceToHost);
+        },
+        [](void *d, const void *s, size_t n) { return (int)cudaMemcpy(d, s, n, cudaMemcpyDeviceToHost); });
+}
+
 static int do_fetch(tsx_ts_list *L) {
     Counters c;
     int st = fetch_counters(L, c);
@@ -1089,8 +1100,7 @@ static int do_fetch(tsx_ts_list *L) {
     std::unique_ptr<int[]> ts3(new int[3 * nts + 1]), pool(new int[pool_used]);
     const int *off = ts3.get(), *cnt = off + nts, *thr = cnt + nts;
     if (nts) {
-        CK(cudaMemcpy2D(ts3.get(), sizeof(int) * nts, L->ts_off, L->ts_pitch, sizeof(int) * nts, 3,
-                        cudaMemcpyDeviceToHost));
+        CK(fetch_rows(ts3.get(), L->ts_off, L->ts_pitch, sizeof(int) * nts, 3));
         CK(cudaMemcpy(pool.get(), L->b.pool, sizeof(int) * pool_used, cudaMemcpyDeviceToHost));
     }
     // sort by (a, b, key): by a, b and the first two nodes in one word, and where that ties by the rest
@@ -1144,8 +1154,7 @@ static int do_fetch(tsx_ts_list *L) {
     L->cts = L->crec.data() + 2 * ncand;
     if (ncand) {
         CK(cudaMemcpy(L->cvars.data(), L->b.cands + L->p.cand_begin, sizeof(int4) * ncand, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy2D(L->crec.data(), sizeof(int) * ncand, L->b.c_thr, L->rec_pitch, sizeof(int) * ncand, 6,
-                        cudaMemcpyDeviceToHost));
+        CK(fetch_rows(L->crec.data(), L->b.c_thr, L->rec_pitch, sizeof(int) * ncand, 6));
         for (long long i = 0; i < ncand; i++)
             if (L->cts[i] >= 0) L->cts[i] = rank[L->cts[i]];
     }
