@@ -8,8 +8,10 @@
 #include <cstdio>
 #include <cstring>
 #include <deque>
+#include <future>
 #include <memory>
 #include <mutex>
+#include <system_error>
 #include <vector>
 
 #include "banks.h"
@@ -248,9 +250,6 @@ int build_csr(const tsx_code_desc &d, HostTables &h) {
     if ((long long)h.dc_max * d.m > 65535) return TSX_EUNSUPPORTED;
     h.v_edge.resize(E);
     h.v_chk.resize(E);
-    bool reg6 = true;
-    for (int c = 0; c < d.m; c++) reg6 = reg6 && h.c_ptr[c + 1] - h.c_ptr[c] == 6;
-    if (reg6) h.c_vnb = bank_order(d.m, 6, h.c_vn);
     std::vector<int> fill(d.n, 0);
     for (int c = 0; c < d.m; c++)  // checks ascending -> edges of v ascending by check
         for (int e = h.c_ptr[c]; e < h.c_ptr[c + 1]; e++) {
@@ -330,6 +329,19 @@ extern "C" int load_code(const tsx_code_desc *desc, void *stream, tsx_code **out
                                           : TSX_EINVAL;
     if (st != TSX_OK) return st;
     if (h.E == 0) return TSX_EINVAL;
+    // The bank order of a general code of check degree 6 is made on a thread beside the rest of the call, and
+    // joined where the call waits for its last copy (in line, m = 504: 1.01 ms a call, so 0.62;
+    // m = 2000: 3.70 and 2.25).
+    bool reg6 = h.kind == TSX_CODE_CSR;
+    for (int i = 0; reg6 && i < h.m; i++) reg6 = h.c_ptr[i + 1] - h.c_ptr[i] == 6;
+    std::future<std::vector<uint16_t>> banks;
+    if (reg6) {
+        h.c_vnb.resize(h.E);
+        try {
+            banks = std::async(std::launch::async, [&h] { return bank_order(h.m, 6, h.c_vn); });
+        } catch (const std::system_error &) {  // (no thread to be had: made in line below)
+        }
+    }
     adjacency(h);
     const int girth = girth_of(h);
     h.vadj.clear(); h.cadj.clear();
@@ -439,7 +451,10 @@ extern "C" int load_code(const tsx_code_desc *desc, void *stream, tsx_code **out
             cudaFree(ball);
             return fail(TSX_ENOMEM);
         }
-        if (cudaMemcpyAsync(c->vweight, vw.data(), sizeof(int) * h.n, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        if (reg6) h.c_vnb = banks.valid() ? banks.get() : bank_order(h.m, 6, h.c_vn);
+        if ((reg6 && cudaMemcpyAsync(dev + o_cvnb, h.c_vnb.data(), sizeof(uint16_t) * h.E, cudaMemcpyHostToDevice, s) !=
+                         cudaSuccess) ||
+            cudaMemcpyAsync(c->vweight, vw.data(), sizeof(int) * h.n, cudaMemcpyHostToDevice, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess) {
             cudaFree(c->vweight);
             cudaFree(ball);

@@ -14,7 +14,8 @@
 //      paths) gives the positions, each a set of different banks.
 // (1008, 504) PEG-like code: 3.36 -> 1.55 wavefronts an access; the decode
 // kernel, 97 % of whose cycles moved shared-memory wavefronts, 126 -> 105 ms on
-// 150,000 candidates.  About 1 ms of host time at m = 504.
+// 150,000 candidates.  Host time 0.5 ms at m = 504, 1.5 at m = 2000, 5 at m = 10,900
+// (load_code() makes it on a thread beside its other work).
 // The edges by which a bank exceeds dc go to the last positions, as far as
 // exchanges within their checks allow.
 #pragma once
@@ -32,7 +33,9 @@ inline std::vector<uint16_t> bank_order(int m, int dc, const std::vector<uint16_
     std::vector<int> slot_of(m), chk(m);  // slot of a check, check of a slot
     std::vector<int> cnt((size_t)ng * W, 0), size(ng, 0);
     auto over = [&](int x) { return (x - dc) * (x - dc); };
-    auto bank = [&](int c, int p) { return col[(size_t)c * dc + p] & (W - 1); };
+    std::vector<uint8_t> bk_of((size_t)m * dc);  // bank of a check's p-th edge
+    for (size_t e = 0; e < bk_of.size(); e++) bk_of[e] = col[e] & (W - 1);
+    auto bank = [&](int c, int p) { return (int)bk_of[(size_t)c * dc + p]; };
     // greedy: each check into the group with room where its banks are met least
     // (a group's count of a bank weighs as its square)
     uint32_t rng = 12345u;
@@ -44,13 +47,13 @@ inline std::vector<uint16_t> bank_order(int m, int dc, const std::vector<uint16_
         int best = -1, best_cost = 0;
         const int tries = ng < 24 ? ng : 24;  // (large codes: a sample of the groups)
         const int g0 = ng <= 24 ? 0 : (int)rnd((uint32_t)ng);
-        for (int t = 0, seen = 0; t < ng && seen < tries; t++) {
-            const int g = (g0 + t) % ng;
+        for (int t = 0, seen = 0, g = g0; t < ng && seen < tries; t++, g = g + 1 < ng ? g + 1 : 0) {
             const int room = g == ng - 1 ? m - W * (ng - 1) : W;
             if (size[g] >= room) continue;
             seen++;
             int cost = 2 * size[g] * dc / W;  // (fill evenly)
-            for (int p = 0; p < dc; p++) cost += 2 * cnt[(size_t)g * W + bank(c, p)] + 1;
+            const int *cn = &cnt[(size_t)g * W];
+            for (int p = 0; p < dc; p++) cost += 2 * cn[bank(c, p)] + 1;
             if (best < 0 || cost < best_cost) {
                 best = g;
                 best_cost = cost;
@@ -70,10 +73,8 @@ inline std::vector<uint16_t> bank_order(int m, int dc, const std::vector<uint16_
         int *ca = &cnt[(size_t)ga * W], *cb = &cnt[(size_t)gb * W];
         // moving a check out of a group lowers the cost by 2 (count - dc) - 1 per edge, into it raises it
         int gain = 0;
-        for (int p = 0; p < dc; p++) {
-            const int x = bank(a, p), y = bank(b, p);
-            gain += ca[x] - cb[x] + cb[y] - ca[y];
-        }
+        const uint8_t *xa = &bk_of[(size_t)a * dc], *xb = &bk_of[(size_t)b * dc];
+        for (int p = 0; p < dc; p++) gain += ca[xa[p]] - cb[xa[p]] + cb[xb[p]] - ca[xb[p]];
         if (gain <= dc) continue;  // (at most 2 dc more than the exact change: edges of the two in one bank)
         auto add = [&](int *cn, int c, int s, int &d) {
             for (int p = 0; p < dc; p++) {
