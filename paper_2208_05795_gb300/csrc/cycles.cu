@@ -182,7 +182,7 @@ __global__ void adj_kernel(DevCode g, int dvp, int by_block, unsigned short *vad
 
 struct Paths {
     DevCode g;
-    int dvp;                      // row length of vadj
+    int dvp, td;                  // row length of vadj, and its entries that may hold a check
     int rep0, nrep;               // representatives of this launch
     const unsigned short *vadj, *cadj;
     unsigned *off;                // [nrep][n + 1]: paths of rep0 + r that start at node w: ent[off[w] .. off[w + 1])
@@ -194,20 +194,20 @@ struct Paths {
 // u != v0, c != c', w != u (w may be v0), sorted by w: counted, scanned and
 // placed by counters in off.
 __global__ void __launch_bounds__(512) pairs_kernel(Paths a) {
-    const int r = blockIdx.x, n = a.g.n, dvp = a.dvp, dc = a.g.dc_max;
+    const int r = blockIdx.x, n = a.g.n, dvp = a.dvp, td = a.td, dc = a.g.dc_max;
     const int v0 = rep_vn(a.g, a.rep0 + r);
     unsigned *off = a.off + (long long)r * (n + 1);
     uint2 *ent = a.ent + (long long)r * a.per;
     for (int w = threadIdx.x; w <= n; w += blockDim.x) off[w] = 0;
     __syncthreads();
-    const int total = dvp * dc * dvp * dc;
+    const int total = td * dc * td * dc;
     auto each = [&](auto f) {
         for (int i = threadIdx.x; i < total; i += blockDim.x) {
             int x = i;
             const int p2 = x % dc;
             x /= dc;
-            const int t2 = x % dvp;
-            x /= dvp;
+            const int t2 = x % td;
+            x /= td;
             const int p1 = x % dc, t1 = x / dc;
             const int c1 = a.vadj[(long long)v0 * dvp + t1];
             if (c1 == kNone) continue;
@@ -289,8 +289,9 @@ __device__ __forceinline__ int emd_distinct(const unsigned short *vadj, const in
 // already enough threads); it counts the walks that close two steps after
 // its last node (and, PD = LMAX - 3, after each node one step further), and
 // those of the shorter prefixes whose deeper indices are 0.
+// (four CTAs an SM: 64 registers; left to itself the compiler takes 80 in some forms, 7 % slower)
 template <int LMAX, int PD, int DVP, bool BLK>
-__global__ void __launch_bounds__(256) walk_kernel(Paths a, long long n_prefix, unsigned long long *walks,
+__global__ void __launch_bounds__(256, 4) walk_kernel(Paths a, long long n_prefix, unsigned long long *walks,
                                                    unsigned long long *hist2) {
     // the CTA's histogram and walk counts, low words and carries
     __shared__ unsigned hs[(kLmax + 1) * kEmdBins], hc[(kLmax + 1) * kEmdBins], ws[kLmax + 1], wc[kLmax + 1];
@@ -301,7 +302,7 @@ __global__ void __launch_bounds__(256) walk_kernel(Paths a, long long n_prefix, 
         const unsigned old = atomicAdd(lo, x);
         if (old + x < old) atomicAdd(hi, 1u);
     };
-    const int dvp = a.dvp, dc = a.g.dc_max, n = a.g.n;
+    const int dvp = a.dvp, td = a.td, dc = a.g.dc_max, n = a.g.n;
     for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < n_prefix;
          id += (long long)gridDim.x * blockDim.x) {
         long long x = id;
@@ -310,8 +311,8 @@ __global__ void __launch_bounds__(256) walk_kernel(Paths a, long long n_prefix, 
         for (int l = PD; l >= 1; l--) {
             pp[l] = (int)(x % dc);
             x /= dc;
-            tt[l] = (int)(x % dvp);
-            x /= dvp;
+            tt[l] = (int)(x % td);
+            x /= td;
         }
         const int r = (int)x;
         const unsigned *off = a.off + (long long)r * (n + 1);
@@ -382,7 +383,7 @@ __global__ void __launch_bounds__(256) walk_kernel(Paths a, long long n_prefix, 
             close(Depth<PD>{});
             if constexpr (PD < LMAX - 2) {
                 // one step further, node by node
-                for (int t = 0; t < dvp; t++) {
+                for (int t = 0; t < td; t++) {
                     const int c = a.vadj[(long long)vs[PD] * dvp + t];
                     if (c == kNone || c == cs[PD]) continue;
                     for (int p = 0; p < dc; p++) {
@@ -470,10 +471,11 @@ cudaError_t launch_cycles(const DevCode &g, int lmax, unsigned long long *walks,
     a.ent = (uint2 *)(buf + b_vadj + b_cadj + b_off);
     const long long na = (long long)g.n * a.dvp + (long long)g.m * g.dc_max;
     const bool blk = g.kind == TSX_CODE_QC && g.m_b <= a.dvp;
+    a.td = blk ? g.m_b : g.dv_max;
     adj_kernel<<<(int)std::min<long long>((na + 255) / 256, 4096), 256, 0, st>>>(
         g, a.dvp, blk ? 1 : 0, (unsigned short *)a.vadj, (unsigned short *)a.cadj);
     e = cudaGetLastError();
-    const long long steps = (long long)a.dvp * g.dc_max;
+    const long long steps = (long long)a.td * g.dc_max;
     for (int r0 = 0; r0 < g.n_rep && e == cudaSuccess; r0 += (int)chunk) {
         a.rep0 = r0;
         a.nrep = (int)std::min<long long>(chunk, g.n_rep - r0);
