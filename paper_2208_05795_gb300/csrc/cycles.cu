@@ -183,22 +183,25 @@ __global__ void adj_kernel(DevCode g, int dvp, int by_block, unsigned short *vad
 struct Paths {
     DevCode g;
     int dvp, td;                  // row length of vadj, and its entries that may hold a check
+    int alone;                    // the walk kernel has by_block rows: a bucket a node, w not stored
     int rep0, nrep;               // representatives of this launch
     const unsigned short *vadj, *cadj;
-    unsigned *off;                // [nrep][n + 1]: paths of rep0 + r that start at node w: ent[off[w] .. off[w + 1])
-    uint2 *ent;                   // [nrep][per]: {u | c' << 16, c} of a path w - c - u - c' - v0
+    // [nrep][nb + 1]: paths of rep0 + r that start at a node w of bucket k = w & mask: ent[off[k] .. off[k + 1])
+    unsigned *off;
+    int nb, mask;                 // buckets (see launch_cycles)
+    uint2 *ent;                   // [nrep][per]: {u | c' << 16, c | w << 16 (alone: c)} of a path w - c - u - c' - v0
     long long per;                // room per representative
 };
 
 // One block per representative: the two-step paths w - c - u - c' - v0 with
-// u != v0, c != c', w != u (w may be v0), sorted by w: counted, scanned and
-// placed by counters in off.
+// u != v0, c != c', w != u (w may be v0), sorted by w's bucket: counted, scanned
+// and placed by counters in off.
 __global__ void __launch_bounds__(512) pairs_kernel(Paths a) {
-    const int r = blockIdx.x, n = a.g.n, dvp = a.dvp, td = a.td, dc = a.g.dc_max;
+    const int r = blockIdx.x, nb = a.nb, dvp = a.dvp, td = a.td, dc = a.g.dc_max;
     const int v0 = rep_vn(a.g, a.rep0 + r);
-    unsigned *off = a.off + (long long)r * (n + 1);
+    unsigned *off = a.off + (long long)r * (nb + 1);
     uint2 *ent = a.ent + (long long)r * a.per;
-    for (int w = threadIdx.x; w <= n; w += blockDim.x) off[w] = 0;
+    for (int w = threadIdx.x; w <= nb; w += blockDim.x) off[w] = 0;
     __syncthreads();
     const int total = td * dc * td * dc;
     auto each = [&](auto f) {
@@ -220,17 +223,17 @@ __global__ void __launch_bounds__(512) pairs_kernel(Paths a) {
             f(w, u, c1, c);
         }
     };
-    each([&](int w, int, int, int) { atomicAdd(&off[w + 1], 1u); });
+    each([&](int w, int, int, int) { atomicAdd(&off[(w & a.mask) + 1], 1u); });
     __syncthreads();
-    // inclusive scan of off[1 .. n] in blocks of blockDim
+    // inclusive scan of off[1 .. nb] in blocks of blockDim
     __shared__ unsigned wsum[16];
     __shared__ unsigned carry;
     if (threadIdx.x == 0) carry = 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int base = 1; base <= n; base += blockDim.x) {
+    for (int base = 1; base <= nb; base += blockDim.x) {
         __syncthreads();
         const int i = base + threadIdx.x;
-        unsigned v = i <= n ? off[i] : 0u;
+        unsigned v = i <= nb ? off[i] : 0u;
         for (int o = 1; o < 32; o <<= 1) {
             const unsigned y = __shfl_up_sync(0xffffffffu, v, o);
             if (lane >= o) v += y;
@@ -240,21 +243,22 @@ __global__ void __launch_bounds__(512) pairs_kernel(Paths a) {
         unsigned add = carry;
         for (int k = 0; k < wid; k++) add += wsum[k];
         v += add;
-        if (i <= n) off[i] = v;
+        if (i <= nb) off[i] = v;
         __syncthreads();
         if (threadIdx.x == blockDim.x - 1) carry = v;
     }
     __syncthreads();
     // off[w] is the start of w; placing advances it to the end, which is the start of w + 1: shift back
     each([&](int w, int u, int c1, int c) {
-        ent[atomicAdd(&off[w], 1u)] = make_uint2((unsigned)u | ((unsigned)c1 << 16), (unsigned)c);
+        ent[atomicAdd(&off[w & a.mask], 1u)] =
+            make_uint2((unsigned)u | ((unsigned)c1 << 16), a.alone ? (unsigned)c : (unsigned)c | ((unsigned)w << 16));
     });
     __syncthreads();
-    for (int base = ((n + blockDim.x) / blockDim.x) * blockDim.x; base >= 0; base -= blockDim.x) {
+    for (int base = ((nb + blockDim.x) / blockDim.x) * blockDim.x; base >= 0; base -= blockDim.x) {
         const int w = base + threadIdx.x;
-        const unsigned x = w >= 1 && w <= n ? off[w - 1] : 0u;
+        const unsigned x = w >= 1 && w <= nb ? off[w - 1] : 0u;
         __syncthreads();
-        if (w <= n) off[w] = x;
+        if (w <= nb) off[w] = x;
         __syncthreads();
     }
 }
@@ -302,7 +306,7 @@ __global__ void __launch_bounds__(256, 4) walk_kernel(Paths a, long long n_prefi
         const unsigned old = atomicAdd(lo, x);
         if (old + x < old) atomicAdd(hi, 1u);
     };
-    const int dvp = a.dvp, td = a.td, dc = a.g.dc_max, n = a.g.n;
+    const int dvp = a.dvp, td = a.td, dc = a.g.dc_max;
     for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < n_prefix;
          id += (long long)gridDim.x * blockDim.x) {
         long long x = id;
@@ -315,7 +319,7 @@ __global__ void __launch_bounds__(256, 4) walk_kernel(Paths a, long long n_prefi
             x /= td;
         }
         const int r = (int)x;
-        const unsigned *off = a.off + (long long)r * (n + 1);
+        const unsigned *off = a.off + (long long)r * (a.nb + 1);
         const uint2 *ent = a.ent + (long long)r * a.per;
         int vs[kLmax], cs[kLmax + 1];
         vs[0] = rep_vn(a.g, a.rep0 + r);
@@ -323,10 +327,12 @@ __global__ void __launch_bounds__(256, 4) walk_kernel(Paths a, long long n_prefi
         // the walks of D + 2 nodes that continue v_D with a listed path
         auto close = [&](auto depth) {
             constexpr int D = decltype(depth)::value, L = D + 2;
-            const unsigned e1 = __ldg(off + vs[D] + 1);
-            for (unsigned e = __ldg(off + vs[D]); e < e1; e++) {
+            const int k = BLK ? vs[D] : vs[D] & a.mask;  // (by_block rows: QC, a bucket a node)
+            const unsigned e1 = __ldg(off + k + 1);
+            for (unsigned e = __ldg(off + k); e < e1; e++) {
                 const uint2 q = __ldg(ent + e);
-                const int u = (int)(q.x & 0xFFFFu), cl = (int)(q.x >> 16), c = (int)q.y;
+                if (!BLK && (int)(q.y >> 16) != vs[D]) continue;
+                const int u = (int)(q.x & 0xFFFFu), cl = (int)(q.x >> 16), c = BLK ? (int)q.y : (int)(q.y & 0xFFFFu);
                 if constexpr (D > 0)
                     if (c == cs[D] || cl == cs[1]) continue;
                 vs[D + 1] = u;
@@ -413,8 +419,8 @@ __global__ void __launch_bounds__(256, 4) walk_kernel(Paths a, long long n_prefi
 template <int LMAX, int DVP, bool BLK>
 cudaError_t launch_walk(const Paths &a, long long steps, unsigned long long *walks, unsigned long long *hist,
                         int num_sms, cudaStream_t st) {
-    // prefixes of LMAX - 2 steps while they are few, else of one step less with the last step looped over
-    // (no id is decoded, and no prefix walked, for each of a check's nodes)
+    // Prefixes of LMAX - 2 steps while they are few, else of one step less with the last step looped over
+    // (no id is decoded, and no prefix walked, for each of a check's nodes).
     long long full = a.nrep, less = a.nrep;
     for (int l = 0; l < LMAX - 2; l++) full *= steps;
     for (int l = 0; l < LMAX - 3; l++) less *= steps;
@@ -456,13 +462,26 @@ cudaError_t launch_cycles(const DevCode &g, int lmax, unsigned long long *walks,
     a.dvp = (g.dv_max + 3) / 4 * 4;
     a.per = (long long)g.dv_max * (g.dc_max - 1) * std::max(1, g.dv_max - 1) * (g.dc_max - 1);
     if (a.per < 1) a.per = 1;
-    const long long per_rep = 4LL * (g.n + 1) + 8 * a.per;
+    // Buckets: one a node (so that none holds two), or about three times as many as a representative has
+    // paths on average where that is less -- a general code has as many representatives as nodes, and
+    // zeroing, scanning and shifting n words for each was most of the call ((3,6) code of 20,000 nodes,
+    // walks of 4 nodes: 3.0 -> 0.47 ms; 32,000 nodes: 6.7 -> 0.55).
+    const double avg = (double)g.E / g.n * g.E / g.m * g.E / g.n * g.E / g.m;
+    a.nb = g.n;
+    a.mask = 0xFFFF;
+    for (int k = 64; g.kind == TSX_CODE_CSR && k < g.n; k *= 2)
+        if (k >= 3.0 * avg) {
+            a.nb = k;
+            a.mask = k - 1;
+            break;
+        }
+    const long long per_rep = 4LL * (a.nb + 1) + 8 * a.per;
     long long chunk = (64LL << 20) / per_rep;
     if (chunk < 1) chunk = 1;
     if (chunk > g.n_rep) chunk = g.n_rep;
     auto r256 = [](long long x) { return (x + 255) / 256 * 256; };
     const long long b_vadj = r256(2LL * g.n * a.dvp), b_cadj = r256(2LL * g.m * g.dc_max),
-                    b_off = r256(4LL * chunk * (g.n + 1)), b_ent = r256(8LL * chunk * a.per);
+                    b_off = r256(4LL * chunk * (a.nb + 1)), b_ent = r256(8LL * chunk * a.per);
     unsigned char *buf = nullptr;
     if ((e = pool_alloc((void **)&buf, (size_t)(b_vadj + b_cadj + b_off + b_ent), st)) != cudaSuccess) return e;
     a.vadj = (unsigned short *)buf;
@@ -472,6 +491,7 @@ cudaError_t launch_cycles(const DevCode &g, int lmax, unsigned long long *walks,
     const long long na = (long long)g.n * a.dvp + (long long)g.m * g.dc_max;
     const bool blk = g.kind == TSX_CODE_QC && g.m_b <= a.dvp;
     a.td = blk ? g.m_b : g.dv_max;
+    a.alone = blk && a.dvp <= 4;
     adj_kernel<<<(int)std::min<long long>((na + 255) / 256, 4096), 256, 0, st>>>(
         g, a.dvp, blk ? 1 : 0, (unsigned short *)a.vadj, (unsigned short *)a.cadj);
     e = cudaGetLastError();

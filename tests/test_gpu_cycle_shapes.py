@@ -1,5 +1,7 @@
 """GPU: the cycle search on general codes, where every node is a representative:
-small, large and uneven degrees, against the oracle."""
+small, large and uneven degrees, paths listed in fewer buckets than nodes.
+Against the oracle; and the cost of a representative does not grow with the
+code."""
 import numpy as np
 import pytest
 
@@ -23,6 +25,7 @@ def _rows(n, m, lo, hi, seed):
     return synth.csr_code(n, m, ptr, np.concatenate([np.sort(list(r)) for r in rows]).astype(np.int32))
 
 
+# (buckets: 64 to 256 of 700 nodes, one a node at 60)
 CODES = {
     "sparse": (lambda: _rows(900, 600, 2, 4, 1), (4, 5, 6)),
     "uneven": (lambda: _rows(700, 400, 2, 8, 2), (4, 5)),
@@ -65,3 +68,13 @@ def test_degree_two_prefixes():
     code = _degree_two(200, 150, 20, 8)
     _check(code, 5, range(code.n))
     assert _ms(code, 6)[0] < 8 * _ms(code, 4)[0]
+
+
+def test_cost_of_a_representative():
+    """Rows of six nodes, 2,500 and 30,000 nodes: twelve times the representatives, in less than twelve times as long;
+    with n words zeroed, scanned and shifted for each representative it grew with the square."""
+    ms = []
+    for n in (2500, 30000):
+        code = tsx.load_code(_rows(n, n // 3, 3, 6, 7))
+        ms.append(min(tsx.emd_spectrum(code, 4)["ms"] for _ in range(5)))
+    assert ms[1] < 12 * ms[0], ms
