@@ -292,10 +292,11 @@ __device__ __forceinline__ int emd_distinct(const unsigned short *vadj, const in
 // One thread per prefix of PD steps (PD = LMAX - 2, or LMAX - 3 where that is
 // already enough threads); it counts the walks that close two steps after
 // its last node (and, PD = LMAX - 3, after each node one step further), and
-// those of the shorter prefixes whose deeper indices are 0.
+// those of the shorter prefixes whose deeper indices are 0.  WARP: the lanes of
+// a warp share what follows each of their prefixes.
 // (four CTAs an SM: 64 registers; left to itself the compiler takes 80 in some forms, 7 % slower)
-template <int LMAX, int PD, int DVP, bool BLK>
-__global__ void __launch_bounds__(256, 4) walk_kernel(Paths a, long long n_prefix, unsigned long long *walks,
+template <int LMAX, int PD, int DVP, bool BLK, bool WARP>
+__global__ void __launch_bounds__(256, 4) walk_kernel(Paths a, long long n_prefix, int share, unsigned long long *walks,
                                                    unsigned long long *hist2) {
     // the CTA's histogram and walk counts, low words and carries
     __shared__ unsigned hs[(kLmax + 1) * kEmdBins], hc[(kLmax + 1) * kEmdBins], ws[kLmax + 1], wc[kLmax + 1];
@@ -307,9 +308,15 @@ __global__ void __launch_bounds__(256, 4) walk_kernel(Paths a, long long n_prefi
         if (old + x < old) atomicAdd(hi, 1u);
     };
     const int dvp = a.dvp, td = a.td, dc = a.g.dc_max;
-    for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < n_prefix;
-         id += (long long)gridDim.x * blockDim.x) {
-        long long x = id;
+    const int lane = threadIdx.x & 31;
+    // WARP: the first `share` lanes of a warp take a prefix each, far apart (next to each other they have
+    // the same representative, and the walks of a node of large degree would be one warp's)
+    const long long threads = (long long)gridDim.x * blockDim.x, warps = threads / 32;
+    const long long thread = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    for (long long base = WARP ? thread / 32 : thread; base < n_prefix; base += WARP ? share * warps : threads) {
+        const long long id = WARP ? base + lane * warps : base;
+        const bool mine = !WARP || (lane < share && id < n_prefix);
+        long long x = mine ? id : 0;
         int tt[PD + 1], pp[PD + 1];
 #pragma unroll
         for (int l = PD; l >= 1; l--) {
@@ -324,12 +331,12 @@ __global__ void __launch_bounds__(256, 4) walk_kernel(Paths a, long long n_prefi
         int vs[kLmax], cs[kLmax + 1];
         vs[0] = rep_vn(a.g, a.rep0 + r);
         unsigned cnt[LMAX + 1] = {};
-        // the walks of D + 2 nodes that continue v_D with a listed path
-        auto close = [&](auto depth) {
+        // the walks of D + 2 nodes that continue v_D with a listed path: every step-th from the first on
+        auto close = [&](auto depth, int first, int step) {
             constexpr int D = decltype(depth)::value, L = D + 2;
             const int k = BLK ? vs[D] : vs[D] & a.mask;  // (by_block rows: QC, a bucket a node)
             const unsigned e1 = __ldg(off + k + 1);
-            for (unsigned e = __ldg(off + k); e < e1; e++) {
+            for (unsigned e = __ldg(off + k) + first; e < e1; e += step) {
                 const uint2 q = __ldg(ent + e);
                 if (!BLK && (int)(q.y >> 16) != vs[D]) continue;
                 const int u = (int)(q.x & 0xFFFFu), cl = (int)(q.x >> 16), c = BLK ? (int)q.y : (int)(q.y & 0xFFFFu);
@@ -358,7 +365,7 @@ __global__ void __launch_bounds__(256, 4) walk_kernel(Paths a, long long n_prefi
                 add(&hs[L * kEmdBins + emd], &hc[L * kEmdBins + emd], (unsigned)wt);
             }
         };
-        bool ok = true;
+        bool ok = mine;
         // counted once: by the thread whose remaining indices are 0
         auto zero_from = [&](int l0) {
             bool z = true;
@@ -367,7 +374,7 @@ __global__ void __launch_bounds__(256, 4) walk_kernel(Paths a, long long n_prefi
                 if (l >= l0) z = z && tt[l] == 0 && pp[l] == 0;
             return z;
         };
-        if (zero_from(1)) close(Depth<0>{});
+        if (ok && zero_from(1)) close(Depth<0>{}, 0, 1);
 #pragma unroll
         for (int l = 1; l <= PD; l++) {
             if (!ok) break;
@@ -379,14 +386,45 @@ __global__ void __launch_bounds__(256, 4) walk_kernel(Paths a, long long n_prefi
             if (!ok) break;
             cs[l] = c;
             vs[l] = u;
-            if (l == 1 && PD > 1 && zero_from(2)) close(Depth<1>{});
+            if (l == 1 && PD > 1 && zero_from(2)) close(Depth<1>{}, 0, 1);
             if constexpr (PD > 2)
-                if (l == 2 && zero_from(3)) close(Depth<2>{});
+                if (l == 2 && zero_from(3)) close(Depth<2>{}, 0, 1);
             if constexpr (PD > 3)
-                if (l == 3 && zero_from(4)) close(Depth<3>{});
+                if (l == 3 && zero_from(4)) close(Depth<3>{}, 0, 1);
         }
-        if (ok) {
-            close(Depth<PD>{});
+        if constexpr (WARP) {
+            static_assert(PD == LMAX - 3, "one step further");
+            int mv[PD + 1], mc[PD + 1];
+#pragma unroll
+            for (int l = 0; l <= PD; l++) {
+                mv[l] = vs[l];
+                mc[l] = l ? cs[l] : 0;
+            }
+            for (unsigned todo = __ballot_sync(0xffffffffu, ok); todo; todo &= todo - 1) {
+                const int src = __ffs(todo) - 1;
+                const int rs = __shfl_sync(0xffffffffu, r, src);
+                off = a.off + (long long)rs * (a.nb + 1);
+                ent = a.ent + (long long)rs * a.per;
+#pragma unroll
+                for (int l = 0; l <= PD; l++) {
+                    vs[l] = __shfl_sync(0xffffffffu, mv[l], src);
+                    cs[l] = __shfl_sync(0xffffffffu, mc[l], src);
+                }
+                close(Depth<PD>{}, lane, 32);
+                for (int x = lane; x < td * dc; x += 32) {
+                    const int t = x / dc, p = x - t * dc;
+                    const int c = a.vadj[(long long)vs[PD] * dvp + t];
+                    if (c == kNone || c == cs[PD]) continue;
+                    const int u = a.cadj[(long long)c * dc + p];
+                    if (u == kNone || u == vs[PD]) continue;
+                    cs[PD + 1] = c;
+                    vs[PD + 1] = u;
+                    close(Depth<PD + 1>{}, 0, 1);
+                }
+                __syncwarp();
+            }
+        } else if (ok) {
+            close(Depth<PD>{}, 0, 1);
             if constexpr (PD < LMAX - 2) {
                 // one step further, node by node
                 for (int t = 0; t < td; t++) {
@@ -397,7 +435,7 @@ __global__ void __launch_bounds__(256, 4) walk_kernel(Paths a, long long n_prefi
                         if (u == kNone || u == vs[PD]) continue;
                         cs[PD + 1] = c;
                         vs[PD + 1] = u;
-                        close(Depth<PD + 1>{});
+                        close(Depth<PD + 1>{}, 0, 1);
                     }
                 }
             }
@@ -420,16 +458,26 @@ template <int LMAX, int DVP, bool BLK>
 cudaError_t launch_walk(const Paths &a, long long steps, unsigned long long *walks, unsigned long long *hist,
                         int num_sms, cudaStream_t st) {
     // Prefixes of LMAX - 2 steps while they are few, else of one step less with the last step looped over
-    // (no id is decoded, and no prefix walked, for each of a check's nodes).
+    // (no id is decoded, and no prefix walked, for each of a check's nodes).  Variable degrees above 4: often
+    // uneven, so that a few prefixes have most of the walks, and the EMD of a walk takes long: a warp shares
+    // what follows its prefixes then (general code of 1,500 nodes, rows of 2 to 12, walks of 4 nodes:
+    // 14.4 -> 2.6 ms; 300 nodes: 86 -> 8.7; 5 x 12 blocks, Z = 60, walks of 5 nodes: 17.4 -> 4.8).
     long long full = a.nrep, less = a.nrep;
     for (int l = 0; l < LMAX - 2; l++) full *= steps;
     for (int l = 0; l < LMAX - 3; l++) less *= steps;
     const bool loop = less >= 32LL * 1024;
-    const long long np = loop ? less : full;
-    long long blocks = (np + 255) / 256;
-    if (blocks > (long long)num_sms * 64) blocks = (long long)num_sms * 64;
-    if (loop) walk_kernel<LMAX, LMAX - 3, DVP, BLK><<<(int)blocks, 256, 0, st>>>(a, np, walks, hist);
-    else walk_kernel<LMAX, LMAX - 2, DVP, BLK><<<(int)blocks, 256, 0, st>>>(a, np, walks, hist);
+    constexpr bool kWarp = DVP > 4;
+    const long long np = loop ? less : full, most = (long long)num_sms * 64;
+    if (loop) {
+        // as many prefixes to a warp as leave every SM enough warps
+        const int share = !kWarp ? 1 : (int)std::min<long long>(32, (np + 8 * most - 1) / (8 * most));
+        const long long threads = kWarp ? (np + share - 1) / share * 32 : np;
+        walk_kernel<LMAX, LMAX - 3, DVP, BLK, kWarp>
+            <<<(int)std::min((threads + 255) / 256, most), 256, 0, st>>>(a, np, share, walks, hist);
+    } else {
+        walk_kernel<LMAX, LMAX - 2, DVP, BLK, false>
+            <<<(int)std::min((np + 255) / 256, most), 256, 0, st>>>(a, np, 1, walks, hist);
+    }
     return cudaGetLastError();
 }
 

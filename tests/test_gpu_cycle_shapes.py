@@ -1,13 +1,14 @@
 """GPU: the cycle search on general codes, where every node is a representative:
-small, large and uneven degrees, paths listed in fewer buckets than nodes.
-Against the oracle; and the cost of a representative does not grow with the
-code."""
+paths listed in fewer buckets than nodes, and prefixes of nodes of large and
+uneven degree shared by a warp.  Against the oracle; and the cost of a
+representative does not grow with the code, nor much that of a walk with uneven degrees."""
 import numpy as np
 import pytest
 
 import paper_2208_05795_gb300 as tsx
 import synth
 from test_gpu_cycle_edges import _check
+from test_gpu_pair_shapes import _qc
 
 pytestmark = pytest.mark.gpu
 
@@ -25,7 +26,7 @@ def _rows(n, m, lo, hi, seed):
     return synth.csr_code(n, m, ptr, np.concatenate([np.sort(list(r)) for r in rows]).astype(np.int32))
 
 
-# (buckets: 64 to 256 of 700 nodes, one a node at 60)
+# (buckets: 64 to 256 of 700 nodes, one a node at 60; a warp shares its prefixes from 32 K of one step less on)
 CODES = {
     "sparse": (lambda: _rows(900, 600, 2, 4, 1), (4, 5, 6)),
     "uneven": (lambda: _rows(700, 400, 2, 8, 2), (4, 5)),
@@ -39,6 +40,12 @@ CODES = {
 def test_general_codes(name, lmax):
     code = CODES[name][0]()
     _check(code, lmax, range(code.n))
+
+
+@pytest.mark.parametrize("mb,nb,Z,lmax", [(6, 10, 9, 5), (5, 8, 64, 5), (7, 9, 5, 5)])
+def test_qc_codes_of_large_degree(mb, nb, Z, lmax):
+    code = _qc(mb, nb, Z, 6, 0.3)
+    _check(code, lmax, range(0, code.n, code.Z))
 
 
 def _degree_two(n, m, most, seed):
@@ -78,3 +85,13 @@ def test_cost_of_a_representative():
         code = tsx.load_code(_rows(n, n // 3, 3, 6, 7))
         ms.append(min(tsx.emd_spectrum(code, 4)["ms"] for _ in range(5)))
     assert ms[1] < 12 * ms[0], ms
+
+
+def test_time_of_a_walk_in_an_uneven_code():
+    """Walks of nodes of large degree are shared out: a walk of a code with rows of 2 to 12 takes at most five times
+    as long as one of a code with even rows (13 times where a thread had all that follow its prefix)."""
+    t = []
+    for lo, hi in ((8, 8), (2, 12)):
+        ms, walks = _ms(_rows(300, 200, lo, hi, 9), 4)
+        t.append(ms / walks)
+    assert t[1] < 5 * t[0], t
