@@ -147,3 +147,11 @@ def test_a_code_decoded_with_two_buffers_is_in_the_multi_code_launch(dispatch, m
     batch = dispatch([(BATCH + c[0],) + c[1:] for c in cases])
     assert [b[0] == "batch" for b in batch] == [a[0] == "pair" for a in alone]
     assert [b[1] for b in batch if b[0] == "batch"] == [a[1] for a in alone if a[0] == "pair"]
+
+
+@pytest.mark.parametrize("mb,nb,Z,form", [(4, 16, 493, ("noise", 1)), (4, 16, 494, ("is", 1)), (4, 16, 505, ("is", 0)),
+                                          (4, 10, 817, ("is", 0)), (4, 30, 267, ("is", 1)), (4, 30, 270, ("is", 0)),
+                                          (4, 32, 254, ("is", 0)), (3, 8, 1188, ("noise", 1))])
+def test_sampling_forms(dispatch, mb, nb, Z, form):
+    """The set's noise kept ("noise") or not, rows filled up (1) or as they are."""
+    assert dispatch([(SAMPLING, mb, nb, Z, nb, nb)])[0][:2] == form
