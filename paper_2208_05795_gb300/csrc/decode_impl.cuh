@@ -688,8 +688,9 @@ struct Sieve {
 
     // b = checks of odd degree in T, elementary = every check degree <= 2
     __device__ void classify(const int *deg, int &b, int &elem) const {
-        int x = 0;  // odd degrees, and degrees above 2 from bit 16 up (m < 2^16; a group's sum stays below 2^31
-                    // because only their presence is counted there, once a thread)
+        // odd degrees in bits 0-19 (m < 2^16), and one flag a thread with degrees above 2 at bit 20: a group of
+        // T threads sums to less than T 2^20 + 2^16
+        int x = 0;
         for (int c = gp.gt; c < g.m; c += gp.T) {
             const int d = deg[c];
             x += d & 1;
