@@ -216,6 +216,8 @@ struct Grp {
         if (G == 1) asm volatile("bar.warp.sync 0xffffffff;" ::: "memory");
         else asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(T) : "memory");
     }
+    // LOOP: the warps' parts added one after the other (see enum_kernel)
+    template <bool LOOP = false>
     __device__ __forceinline__ int sum(int x) const {
         x = __reduce_add_sync(0xffffffffu, x);
         if (G == 1) {
@@ -224,7 +226,11 @@ struct Grp {
         }
         if (lane == 0) red[gw] = x;
         sync();
-        const int s = __reduce_add_sync(0xffffffffu, lane < G ? red[lane] : 0);
+        int s = 0;
+        if constexpr (LOOP)
+            for (int w = 0; w < G; w++) s += red[w];
+        else
+            s = __reduce_add_sync(0xffffffffu, lane < G ? red[lane] : 0);
         sync();
         return s;
     }
@@ -339,7 +345,7 @@ struct SieveMisc {
 // ---------------------------------------------------------------------------
 // one decode
 // ---------------------------------------------------------------------------
-template <class Dec, int DCMAX, bool QC>
+template <class Dec, int DCMAX, bool QC, bool LOOP = false>
 struct Decoder {
     using msg = typename Dec::msg;
     using post = typename Dec::post;
@@ -378,7 +384,7 @@ struct Decoder {
                 unsat += check_node(first, writeR, deg, c, g.m, [&](int p) { return (int)sg.c_vn[e0 + p]; });
             }
         }
-        return gp.sum(unsat);
+        return gp.template sum<LOOP>(unsat);
     }
 
     template <class NB>
@@ -932,7 +938,7 @@ __device__ long long ts_insert(const EnumBuffers &b, const uint16_t *key, int a,
 // ---------------------------------------------------------------------------
 // the kernel
 // ---------------------------------------------------------------------------
-template <class Dec, int DCMAX, bool QC>
+template <class Dec, int DCMAX, bool QC, bool LOOP>
 __device__ __forceinline__ void scalar_run(const DevCode &g, const DecodeParams &dp, const EnumBuffers &b,
                                            const SlotLayout &lay, int G, const SGraph &sg, unsigned char *smem,
                                            int grp) {
@@ -955,7 +961,7 @@ __device__ __forceinline__ void scalar_run(const DevCode &g, const DecodeParams 
     uint32_t *xa = (uint32_t *)(slot + lay.xa_off);
     uint32_t *xb = (uint32_t *)(slot + lay.xb_off);
 
-    Decoder<Dec, DCMAX, QC> dec{g, sg, gp, dp, P, R};
+    Decoder<Dec, DCMAX, QC, LOOP> dec{g, sg, gp, dp, P, R};
 
     const long long total = (long long)b.ctr->n_cand_total;
     const long long end = b.cand_end < 0 || b.cand_end > total ? total : b.cand_end;
@@ -1071,13 +1077,17 @@ __device__ __forceinline__ void scalar_run(const DevCode &g, const DecodeParams 
 // code, 5,000 candidates, 12 groups of two warps (24 warps, 80 registers) take 56 ms,
 // 13 of one (16 or 20 warps) 96, 28 warps 57 (with divisions by branch; 43 without); small codes fill 32 one-warp
 // groups (n = 306: 17.9 ms; 24 warps 22).  Before: 113 and 25.7.
-template <class Dec, int DCMAX, bool QC, int WARPS = 16>
+// LOOP: the form for groups of one warp of the min-sum QC codes of check degree above 8.  The check pass unrolled
+// over 32 edges fills the registers, and the sum over warps by one reduction, which such groups do not even
+// reach, moved its spills into the pass: 4 x 18 blocks, Z = 128, 8,000 candidates, 95 ms, with the loop 89; wider
+// groups take the reduction (Z = 300, degree 30: 29.4 against 30.5).
+template <class Dec, int DCMAX, bool QC, int WARPS = 16, bool LOOP = false>
 __global__ void __launch_bounds__(32 * WARPS, 1) enum_kernel(DevCode g, DecodeParams dp, EnumBuffers b,
                                                     SlotLayout lay, int G) {
     extern __shared__ __align__(16) unsigned char smem[];
     const SGraph sg = load_tables(g, smem);
     __syncthreads();
-    scalar_run<Dec, DCMAX, QC>(g, dp, b, lay, G, sg, smem, (threadIdx.x >> 5) / G);
+    scalar_run<Dec, DCMAX, QC, LOOP>(g, dp, b, lay, G, sg, smem, (threadIdx.x >> 5) / G);
 }
 
 // ---------------------------------------------------------------------------
@@ -1180,6 +1190,10 @@ cudaError_t launch_scalar(const DevCode &g, const DecodeParams &dp, const EnumBu
     if (g.dc_max <= 8)
         return qc ? launch_persistent(enum_kernel<Dec, 8, true, scalar_warps(Dec::kFloat, 8)>, sh, st, g, dp, b, sh.lay, sh.G)
                   : launch_persistent(enum_kernel<Dec, 8, false, scalar_warps(Dec::kFloat, 8)>, sh, st, g, dp, b, sh.lay, sh.G);
+    if constexpr (!Dec::kFloat) {
+        if (qc && sh.G == 1)
+            return launch_persistent(enum_kernel<Dec, 32, true, 16, true>, sh, st, g, dp, b, sh.lay, sh.G);
+    }
     return qc ? launch_persistent(enum_kernel<Dec, 32, true>, sh, st, g, dp, b, sh.lay, sh.G)
               : launch_persistent(enum_kernel<Dec, 32, false>, sh, st, g, dp, b, sh.lay, sh.G);
 }
