@@ -1078,9 +1078,9 @@ __device__ __forceinline__ void scalar_run(const DevCode &g, const DecodeParams 
 // 13 of one (16 or 20 warps) 96, 28 warps 57 (with divisions by branch; 43 without); small codes fill 32 one-warp
 // groups (n = 306: 17.9 ms; 24 warps 22).  Before: 113 and 25.7.
 // LOOP: the form for groups of one warp of the min-sum QC codes of check degree above 8.  The check pass unrolled
-// over 32 edges fills the registers, and the sum over warps by one reduction, which such groups do not even
-// reach, moved its spills into the pass: 4 x 18 blocks, Z = 128, 8,000 candidates, 95 ms, with the loop 89; wider
-// groups take the reduction (Z = 300, degree 30: 29.4 against 30.5).
+// over 32 edges fills the registers (about 200 bytes spilled), and the sum over warps by one reduction, which such
+// groups do not even reach, changes what is spilled: 4 x 18 blocks, Z = 128, 8,000 candidates, 95 ms, with the
+// loop 89; wider groups take the reduction (Z = 300, degree 30: 29.4 against 30.5).
 template <class Dec, int DCMAX, bool QC, int WARPS = 16, bool LOOP = false>
 __global__ void __launch_bounds__(32 * WARPS, 1) enum_kernel(DevCode g, DecodeParams dp, EnumBuffers b,
                                                     SlotLayout lay, int G) {
